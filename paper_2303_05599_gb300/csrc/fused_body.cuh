@@ -32,13 +32,6 @@
 
 namespace gl {
 
-template <typename R>
-struct ExpN;
-template <>
-struct ExpN<double> { static constexpr int n = 20; };
-template <>
-struct ExpN<float> { static constexpr int n = 6; };
-
 template <typename R, int TX, int TY>
 struct Tile {
     using V = typename Prec<R>::V;
@@ -406,10 +399,10 @@ __device__ __forceinline__ void fused_tile(const Fields<R>& in, const Fields<R>&
         store_alg_cs(out.e + (size_t)AP * Vn, g, Vn, my_ey);
         store_alg_cs(out.pi, g, Vn, p_new);
         store_alg_cs(out.phi, g, Vn, ph_new);
-        M3<R> nx = mul(exp_i_alg<R, ExpN<R>::n>(my_ex, a.dt_over_th), lk(0, ls));
+        M3<R> nx = mul(exp_i_alg<R>(my_ex, a.dt_over_th), lk(0, ls));
         if (a.reunit) reunit(nx);
         store_link_cs(out.U, 0, g, Vn, nx);
-        M3<R> ny = mul(exp_i_alg<R, ExpN<R>::n>(my_ey, a.dt_over_th), lk(1, ls));
+        M3<R> ny = mul(exp_i_alg<R>(my_ey, a.dt_over_th), lk(1, ls));
         if (a.reunit) reunit(ny);
         store_link_cs(out.U, 1, g, Vn, ny);
     }

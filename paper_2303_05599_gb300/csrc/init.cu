@@ -129,7 +129,7 @@ __global__ void wilson_accum_kernel(double2* Vd, const double2* rho, int64_t Vn)
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < Vn; s += (int64_t)gridDim.x * blockDim.x) {
         A8<double> al;
         for (int a = 0; a < 8; a++) al.v[a] = -rho[(size_t)a * Vn + s].x;
-        const M3<double> e = exp_i_alg<double, 20>(al, 1.0);
+        const M3<double> e = exp_i_alg<double>(al, 1.0);
         const M3<double> v = load_link(Vd, 0, s, Vn);
         store_link(Vd, 0, s, Vn, mul(v, e));
     }
@@ -207,7 +207,7 @@ __device__ int solve_link(const M3<double>& UA, const M3<double>& UB, M3<double>
         for (int k = 0; k < 30; k++) {
             A8<double> st;
             for (int a = 0; a < 8; a++) st.v[a] = lam * dx[a];
-            const M3<double> Un = mul(exp_i_alg<double, 20>(st, 1.0), U);
+            const M3<double> Un = mul(exp_i_alg<double>(st, 1.0), U);
             double Fn[8];
             const double rn = match_residual(W, Un, Fn);
             if (rn < r || k == 29) {

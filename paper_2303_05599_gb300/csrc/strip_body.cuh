@@ -134,11 +134,34 @@ __device__ __forceinline__ A8<float> alg_of(const float4 a, const float4 b) {
     return x;
 }
 
-// Products of SU(3) matrices with rows 0 and 1 multiplied out and row 2 the
-// conjugate cross product of the two, as for a stored link: c = a b and
-// c = a b^+.
-__device__ __forceinline__ M3<float> mul_su3(const M3<float>& a, const M3<float>& b) {
-    M3<float> c;
+// Components of i[P]_ah of the plaquette P = Ux UyR UxN^+ Uy^+.  A product of
+// SU(3) matrices needs its rows 0 and 1 only, which take rows 0 and 1 of its
+// left factor: the two inner products and P itself are formed as two rows
+// (Ux needs no third row here either), and row 2 of P, of which three entries
+// enter the result, is the conjugate cross product of its rows 0 and 1, as for
+// a stored link.  Rebuilding the third rows of the inner products and forming
+// all entries of the last one took 46 operations a site more.
+__device__ __forceinline__ A8<float> plaquette(const M3<float>& Ux, const M3<float>& UyR, const M3<float>& UxN,
+                                               const M3<float>& Uy) {
+    float ar[2][3], ai[2][3], br[2][3], bi[2][3];
+    auto times_dag = [](const float (*pr)[3], const float (*pi)[3], const M3<float>& m, float (*qr)[3],
+                        float (*qi)[3]) {
+#pragma unroll
+        for (int i = 0; i < 2; i++)
+#pragma unroll
+            for (int j = 0; j < 3; j++) {
+                float sr = 0.f, si = 0.f;
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    sr = fmaf(pr[i][k], m.re[j][k], sr);
+                    sr = fmaf(pi[i][k], m.im[j][k], sr);
+                    si = fmaf(pi[i][k], m.re[j][k], si);
+                    si = fmaf(-pr[i][k], m.im[j][k], si);
+                }
+                qr[i][j] = sr;
+                qi[i][j] = si;
+            }
+    };
 #pragma unroll
     for (int i = 0; i < 2; i++)
 #pragma unroll
@@ -146,36 +169,32 @@ __device__ __forceinline__ M3<float> mul_su3(const M3<float>& a, const M3<float>
             float sr = 0.f, si = 0.f;
 #pragma unroll
             for (int k = 0; k < 3; k++) {
-                sr = fmaf(a.re[i][k], b.re[k][j], sr);
-                sr = fmaf(-a.im[i][k], b.im[k][j], sr);
-                si = fmaf(a.re[i][k], b.im[k][j], si);
-                si = fmaf(a.im[i][k], b.re[k][j], si);
+                sr = fmaf(Ux.re[i][k], UyR.re[k][j], sr);
+                sr = fmaf(-Ux.im[i][k], UyR.im[k][j], sr);
+                si = fmaf(Ux.re[i][k], UyR.im[k][j], si);
+                si = fmaf(Ux.im[i][k], UyR.re[k][j], si);
             }
-            c.re[i][j] = sr;
-            c.im[i][j] = si;
+            ar[i][j] = sr;
+            ai[i][j] = si;
         }
-    rebuild_row2(c);
-    return c;
-}
-__device__ __forceinline__ M3<float> mul_nd_su3(const M3<float>& a, const M3<float>& b) {
-    M3<float> c;
-#pragma unroll
-    for (int i = 0; i < 2; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            float sr = 0.f, si = 0.f;
-#pragma unroll
-            for (int k = 0; k < 3; k++) {
-                sr = fmaf(a.re[i][k], b.re[j][k], sr);
-                sr = fmaf(a.im[i][k], b.im[j][k], sr);
-                si = fmaf(a.im[i][k], b.re[j][k], si);
-                si = fmaf(-a.re[i][k], b.im[j][k], si);
-            }
-            c.re[i][j] = sr;
-            c.im[i][j] = si;
-        }
-    rebuild_row2(c);
-    return c;
+    times_dag(ar, ai, UxN, br, bi);
+    times_dag(br, bi, Uy, ar, ai);
+    // row 2 of P: conj(P0 x P1); only Re, Im of its first two entries and Im of the third
+    const float r20 = ar[0][1] * ar[1][2] - ai[0][1] * ai[1][2] - (ar[0][2] * ar[1][1] - ai[0][2] * ai[1][1]);
+    const float i20 = ar[0][2] * ai[1][1] + ai[0][2] * ar[1][1] - (ar[0][1] * ai[1][2] + ai[0][1] * ar[1][2]);
+    const float r21 = ar[0][2] * ar[1][0] - ai[0][2] * ai[1][0] - (ar[0][0] * ar[1][2] - ai[0][0] * ai[1][2]);
+    const float i21 = ar[0][0] * ai[1][2] + ai[0][0] * ar[1][2] - (ar[0][2] * ai[1][0] + ai[0][2] * ar[1][0]);
+    const float i22 = ar[0][1] * ai[1][0] + ai[0][1] * ar[1][0] - (ar[0][0] * ai[1][1] + ai[0][0] * ar[1][1]);
+    A8<float> x;
+    x.v[0] = -(ai[0][1] + ai[1][0]);
+    x.v[1] = ar[1][0] - ar[0][1];
+    x.v[2] = ai[1][1] - ai[0][0];
+    x.v[3] = -(ai[0][2] + i20);
+    x.v[4] = r20 - ar[0][2];
+    x.v[5] = -(ai[1][2] + i21);
+    x.v[6] = r21 - ar[1][2];
+    x.v[7] = (2.f * i22 - ai[0][0] - ai[1][1]) * inv_sqrt3<float>();
+    return x;
 }
 
 // Component-wise updates of algebra elements on packed pairs of FP32
@@ -306,7 +325,7 @@ __device__ __forceinline__ void strip_halo(StripWarpSmem& S, const Fields<float>
     // Ux of the row above: the next lane's link, the last lane loads it
     M3<float> UxU = shfl_down_m3(Ux);
     if (L.lane == 31 && L.lane <= nb) UxU = load_link(in.U, 0, (int64_t)yu * N + L.xl, Vn);
-    const A8<float> A = iah_of_mul_nd(mul_nd_su3(mul_su3(Ux, UyR), UxU), Uy);
+    const A8<float> A = plaquette(Ux, UyR, UxU, Uy);
     const A8<float> Dn = shfl_up_a8(conj_dn_t(Uy, A));
     const A8<float> tx = conj_up_t(Ux, phR);
     const A8<float> cx = icomm(tx, ph);
@@ -402,7 +421,7 @@ __device__ __forceinline__ void strip_segment(StripWarpSmem& S, const Fields<flo
         // Each value is used as soon as it is known and the outputs stored as
         // they are formed, so that few values live at once.  The dry row forms
         // only what the carries need (A, Lf, the e_y update).
-        const A8<float> A = iah_of_mul_nd(mul_nd_su3(mul_su3(Ux, UyR), UxN), Uy);   // plaquette at (x, y)
+        const A8<float> A = plaquette(Ux, UyR, UxN, Uy);   // plaquette at (x, y)
         // ring slot k (Ux, Uy, phi and the right neighbour's Uy, phi of row r)
         // has been read into registers above: row r + 2 goes there
         if (r + 2 <= ye) strip_issue_row(S, k, in, Vn, N, L, r + 2);
@@ -442,7 +461,7 @@ __device__ __forceinline__ void strip_segment(StripWarpSmem& S, const Fields<flo
             if (st) {
                 store_alg(site, g, Vn, Ex);
                 store_alg_cs(out.e, g, Vn, exn);
-                M3<float> nx = mul(exp_i_alg<float, ExpN<float>::n>(exn, c_link), Ux);
+                M3<float> nx = mul(exp_i_alg<float>(exn, c_link), Ux);
                 if (ru == 0) reunit_rows(nx);
                 store_link_cs(out.U, 0, g, Vn, nx);
             }
@@ -478,7 +497,7 @@ __device__ __forceinline__ void strip_segment(StripWarpSmem& S, const Fields<flo
         if (r + 1 < ye) strip_issue_mom(S, in, Vn, N, L, r + 1);
         else cp_async_commit();
         if (st) {
-            M3<float> ny = mul(exp_i_alg<float, ExpN<float>::n>(eyn, c_link), Uy);
+            M3<float> ny = mul(exp_i_alg<float>(eyn, c_link), Uy);
             if (ru == 0) reunit_rows(ny);
             store_link_cs(out.U, 1, g, Vn, ny);
         }

@@ -443,11 +443,83 @@ __device__ __forceinline__ R casimir3(const A8<R>& q) {
     return r;
 }
 
-// exp(i s X) for Hermitian traceless X = x^a T^a.  Cayley-Hamilton gives
-// X^3 = c1 X + c0 with c1 = tr(X^2)/2 and c0 = det X, so every power of iX
-// is a combination of 1, X, X^2; the exponential series is summed on those
-// three scalar coefficients (scaling and squaring when |sX| > 1).
-template <typename R, int TERMS>
+// The coefficients of exp(iX) = f0 + f1 X + f2 X^2 for Hermitian traceless X
+// with X^3 = c1 X + c0 (Cayley-Hamilton: c1 = tr(X^2)/2, c0 = det X).
+template <typename R>
+struct ExpScale {
+    int nsq;    // squarings: the series is summed for scl X, scl = 2^-nsq
+    R scl;
+    int terms;  // FP64: its last power
+};
+
+// FP32: the series to X^6 for |X| <= 0.2 (truncation error below 1e-8),
+// reduced by X^3 = c1 X + c0 to one polynomial in (c0, c1) for each real
+// coefficient: 11 operations, where the recurrence of the reduced powers takes
+// about 48.  Two exponentials a site are 2 % of the field step's issue slots.
+__device__ __forceinline__ void exp_coeffs(float c0, float c1, const ExpScale<float>&, float* fr, float* fi) {
+    fr[0] = fmaf(-1.0f / 720, c0 * c0, 1.0f);
+    fi[0] = c0 * fmaf(1.0f / 120, c1, -1.0f / 6);
+    fr[1] = c0 * fmaf(-1.0f / 360, c1, 1.0f / 24);
+    fi[1] = fmaf(c1, fmaf(1.0f / 120, c1, -1.0f / 6), 1.0f);
+    fr[2] = fmaf(c1, fmaf(-1.0f / 720, c1, 1.0f / 24), -0.5f);
+    fi[2] = c0 * (1.0f / 120);
+}
+
+// FP64: Horner's rule on the reduced series.  With P = p0 + p1 X + p2 X^2,
+// 1/k! + iX P has the coefficients 1/k! + i c0 p2, i (p0 + c1 p2), i p1: four
+// operations a term.  FP64 operations take 64 cycles of a scheduler per warp
+// on GB300, so the number of terms follows the norm: 6 for |X| <= 0.01 (a
+// field step late in the run, a Newton step), 12 for 0.25, 18 for 1, 24 for 2
+// (one sheet of an MV nucleus), each with a truncation error below 3e-18.
+__device__ __forceinline__ void exp_coeffs(double c0, double c1, const ExpScale<double>& s, double* fr, double* fi) {
+    constexpr double F[25] = {1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040, 1.0 / 40320,
+                              1.0 / 362880, 1.0 / 3628800, 1.0 / 39916800, 1.0 / 479001600, 1.0 / 6227020800.0,
+                              1.0 / 87178291200.0, 1.0 / 1307674368000.0, 1.0 / 20922789888000.0,
+                              1.0 / 355687428096000.0, 1.0 / 6402373705728000.0, 1.0 / 121645100408832000.0,
+                              1.0 / 2432902008176640000.0, 1.0 / 51090942171709440000.0,
+                              1.0 / 1124000727777607680000.0, 1.0 / 25852016738884976640000.0,
+                              1.0 / 620448401733239439360000.0};
+    double r0 = s.terms == 24 ? F[24] : s.terms == 18 ? F[18] : s.terms == 12 ? F[12] : F[6];
+    double i0 = 0, r1 = 0, i1 = 0, r2 = 0, i2 = 0;
+#define GL_HORNER(k)                                         \
+    {                                                        \
+        const double n0r = fma(-c0, i2, F[k]), n0i = c0 * r2; \
+        const double n1r = -fma(c1, i2, i0), n1i = fma(c1, r2, r0); \
+        r2 = -i1;                                            \
+        i2 = r1;                                             \
+        r0 = n0r;                                            \
+        i0 = n0i;                                            \
+        r1 = n1r;                                            \
+        i1 = n1i;                                            \
+    }
+#define GL_HORNER6(k) \
+    GL_HORNER(k) GL_HORNER((k) - 1) GL_HORNER((k) - 2) GL_HORNER((k) - 3) GL_HORNER((k) - 4) GL_HORNER((k) - 5)
+    if (s.terms > 18) { GL_HORNER6(23) }
+    if (s.terms > 12) { GL_HORNER6(17) }
+    if (s.terms > 6) { GL_HORNER6(11) }
+    GL_HORNER6(5)
+#undef GL_HORNER6
+#undef GL_HORNER
+    fr[0] = r0; fi[0] = i0;
+    fr[1] = r1; fi[1] = i1;
+    fr[2] = r2; fi[2] = i2;
+}
+
+__device__ __forceinline__ ExpScale<float> exp_scale(float nrm2) {
+    ExpScale<float> s = {0, 1.0f, 6};
+    while (nrm2 > 0.04f && s.nsq < 30) { nrm2 *= 0.25f; s.scl *= 0.5f; s.nsq++; }
+    return s;
+}
+__device__ __forceinline__ ExpScale<double> exp_scale(double nrm2) {
+    ExpScale<double> s = {0, 1.0, 24};
+    while (nrm2 > 4.0 && s.nsq < 30) { nrm2 *= 0.25; s.scl *= 0.5; s.nsq++; }
+    if (nrm2 <= 1.0) s.terms = nrm2 <= 1e-4 ? 6 : nrm2 <= 0.0625 ? 12 : 18;
+    return s;
+}
+
+// exp(i s X) for Hermitian traceless X = x^a T^a (scaling and squaring beyond
+// the series' range)
+template <typename R>
 __device__ __forceinline__ M3<R> exp_i_alg(const A8<R>& x, R s) {
     // s X: 2 X from the components, times s / 2 (exact: a power of 2), one
     // product per distinct entry
@@ -466,15 +538,9 @@ __device__ __forceinline__ M3<R> exp_i_alg(const A8<R>& x, R s) {
     }
     M3<R> X2 = sq_herm(X);
     R c1 = R(0.5) * (X2.re[0][0] + X2.re[1][1] + X2.re[2][2]);
-    int nsq = 0;
-    R scl = R(1);
-    // Frobenius norm^2 of X is 2 c1; scale until the truncated series is
-    // accurate: |X| <= 1 with 12 or more terms, |X| <= 0.5 with 8 to 11,
-    // |X| <= 0.2 with fewer (truncation error below 1e-8 in each case)
-    const R lim = TERMS >= 12 ? R(1) : (TERMS >= 8 ? R(0.25) : R(0.04));
-    R nrm2 = R(2) * c1;
-    while (nrm2 > lim && nsq < 30) { nrm2 *= R(0.25); scl *= R(0.5); nsq++; }
-    if (nsq) {
+    const ExpScale<R> sc = exp_scale(R(2) * c1);  // the squared Frobenius norm of X is 2 c1
+    if (sc.nsq) {
+        const R scl = sc.scl;
 #pragma unroll
         for (int i = 0; i < 3; i++)
 #pragma unroll
@@ -484,32 +550,19 @@ __device__ __forceinline__ M3<R> exp_i_alg(const A8<R>& x, R s) {
             }
         c1 *= scl * scl;
     }
-    // det X of Hermitian X (real diagonal, X_ji = conj X_ij): x00 x11 x22
-    // + 2 Re(x01 x12 conj x02) - x00 |x12|^2 - x11 |x02|^2 - x22 |x01|^2
-    const R pr = X.re[0][1] * X.re[1][2] - X.im[0][1] * X.im[1][2];
-    const R pi_ = X.re[0][1] * X.im[1][2] + X.im[0][1] * X.re[1][2];
-    const R n01 = X.re[0][1] * X.re[0][1] + X.im[0][1] * X.im[0][1];
-    const R n02 = X.re[0][2] * X.re[0][2] + X.im[0][2] * X.im[0][2];
-    const R n12 = X.re[1][2] * X.re[1][2] + X.im[1][2] * X.im[1][2];
-    const R c0 = X.re[0][0] * (X.re[1][1] * X.re[2][2] - n12) - X.re[1][1] * n02 - X.re[2][2] * n01 +
-                 R(2) * (pr * X.re[0][2] + pi_ * X.im[0][2]);
-    // (iX)^k / k! = i^k (a_k + b_k X + g_k X^2) with real a, b, g: from
-    // X^3 = c1 X + c0, a_{k+1} = c0 g_k / (k+1), b_{k+1} = (a_k + c1 g_k) /
-    // (k+1), g_{k+1} = b_k / (k+1).  The factor i^k only decides, at compile
-    // time, which part of the complex sums f0, f1, f2 a term enters, and with
-    // which sign.
-    R a = R(1), b = R(0), g = R(0);
-    R f0r = R(1), f0i = R(0), f1r = R(0), f1i = R(0), f2r = R(0), f2i = R(0);
-#pragma unroll
-    for (int k = 1; k <= TERMS; k++) {
-        const R inv = R(1) / R(k);
-        const R na = c0 * g * inv, nb = (a + c1 * g) * inv, ng = b * inv;
-        a = na; b = nb; g = ng;
-        if ((k & 3) == 1) { f0i += a; f1i += b; f2i += g; }
-        else if ((k & 3) == 2) { f0r -= a; f1r -= b; f2r -= g; }
-        else if ((k & 3) == 3) { f0i -= a; f1i -= b; f2i -= g; }
-        else { f0r += a; f1r += b; f2r += g; }
-    }
+    // det X = tr(X^3) / 3 of the traceless X, from X and X^2 (both Hermitian)
+    R c0 = X.re[0][1] * X2.re[0][1];
+    c0 = fma(X.im[0][1], X2.im[0][1], c0);
+    c0 = fma(X.re[0][2], X2.re[0][2], c0);
+    c0 = fma(X.im[0][2], X2.im[0][2], c0);
+    c0 = fma(X.re[1][2], X2.re[1][2], c0);
+    c0 = fma(X.im[1][2], X2.im[1][2], c0);
+    c0 = fma(R(0.5) * X.re[0][0], X2.re[0][0], c0);
+    c0 = fma(R(0.5) * X.re[1][1], X2.re[1][1], c0);
+    c0 = fma(R(0.5) * X.re[2][2], X2.re[2][2], c0);
+    c0 *= R(2.0 / 3.0);
+    R fr[3], fi[3];
+    exp_coeffs(c0, c1, sc, fr, fi);
     M3<R> U;
 #pragma unroll
     for (int i = 0; i < 3; i++)
@@ -517,10 +570,10 @@ __device__ __forceinline__ M3<R> exp_i_alg(const A8<R>& x, R s) {
         for (int j = 0; j < 3; j++) {
             const R d = (i == j) ? R(1) : R(0);
             // (f0 + f1 X + f2 X2)_ij, complex coefficients
-            U.re[i][j] = f0r * d + f1r * X.re[i][j] - f1i * X.im[i][j] + f2r * X2.re[i][j] - f2i * X2.im[i][j];
-            U.im[i][j] = f0i * d + f1r * X.im[i][j] + f1i * X.re[i][j] + f2r * X2.im[i][j] + f2i * X2.re[i][j];
+            U.re[i][j] = fr[0] * d + fr[1] * X.re[i][j] - fi[1] * X.im[i][j] + fr[2] * X2.re[i][j] - fi[2] * X2.im[i][j];
+            U.im[i][j] = fi[0] * d + fr[1] * X.im[i][j] + fi[1] * X.re[i][j] + fr[2] * X2.im[i][j] + fi[2] * X2.re[i][j];
         }
-    for (int k = 0; k < nsq; k++) U = mul(U, U);
+    for (int k = 0; k < sc.nsq; k++) U = mul(U, U);
     return U;
 }
 
