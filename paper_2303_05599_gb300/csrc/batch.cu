@@ -518,6 +518,7 @@ struct gl_batch {
     PartsCheckEv* p_pchk;  // pinned [ne]: the index-check descriptors (allocated with h_bad)
     PartsCheckEv* d_pchk;  // [ne] the same on the device, and
     int* d_bad;            // [ne] the index-check flags
+    InitEv* d_init;        // [ne] the initial conditions' descriptors
     // observables requests: two slots, each with a pinned copy of h_obs for
     // its upload, pinned [ne][OBS_W] for the gathered rows, and an event
     // after its copy back (allocated on first use); obs_count requests are
@@ -603,7 +604,8 @@ size_t gl_batch_workspace_bytes(const gl_config* cfgs, const gl_species* species
     if (!cfgs || n_events < 1 || n_events > MAX_EVENTS) return 0;
     size_t o = a256b(sizeof(EvDesc) * n_events) + 256 + a256b(sizeof(BObs) * n_events) +
                a256b(sizeof(double) * OBS_W * n_events) + a256b(sizeof(SortEv) * n_events) +
-               a256b(sizeof(PartsCheckEv) * n_events) + a256b(sizeof(int) * n_events);
+               a256b(sizeof(PartsCheckEv) * n_events) + a256b(sizeof(int) * n_events) +
+               a256b(sizeof(InitEv) * n_events);
     for (int e = 0; e < n_events; e++) {
         const size_t w = ctx_workspace_bytes(&cfgs[e], species ? species + (size_t)e * n_species : nullptr, n_species);
         if (!w) return 0;
@@ -666,6 +668,8 @@ gl_status gl_batch_create(const gl_config* cfgs, const gl_species* species, int3
     o += a256b(sizeof(PartsCheckEv) * n_events);
     b->d_bad = (int*)(ws + o);
     o += a256b(sizeof(int) * n_events);
+    b->d_init = (InitEv*)(ws + o);
+    o += a256b(sizeof(InitEv) * n_events);
     for (int e = 0; e < n_events; e++) {
         const gl_species* sp = species ? species + (size_t)e * n_species : nullptr;
         const size_t w = ctx_workspace_bytes(&cfgs[e], sp, n_species);
@@ -733,16 +737,50 @@ gl_status gl_batch_init(gl_batch* b) {
     gl::ApiRange range_("gl_batch_init");
     if (!b) return GL_ERR_ARG;
     b->desc_valid = 0;
+    // the fields of all events in the same launches: a single event's leave
+    // most of the chip idle (its transforms and Newton solves are short)
+    InitEv* h = new (std::nothrow) InitEv[b->ne];
+    int* bad = new (std::nothrow) int[b->ne];
+    if (!h || !bad) {
+        delete[] h;
+        delete[] bad;
+        return bfail(b, GL_ERR_ARG, "out of host memory");
+    }
+    gl_status st = GL_OK;
     for (int e = 0; e < b->ne; e++) {
-        gl_status s = glasma_init(b->ev[e]);
-        if (s == GL_OK) s = wong_init(b->ev[e]);
-        if (s != GL_OK) {
-            char m[300];
-            snprintf(m, sizeof m, "event %d: %s", e, gl_error_string(b->ev[e]));
-            return bfail(b, s, m);
+        h[e] = ctx_init_event(b->ev[e], b->d_bad + e);
+        if (st == GL_OK && !init_supported(h[e].N)) {
+            char m[128];
+            snprintf(m, sizeof m, "event %d: glasma_init: N is beyond the transforms' shared memory", e);
+            st = bfail(b, GL_ERR_CUDA, m);
         }
     }
-    return GL_OK;
+    if (st == GL_OK) {
+        init_block_table(h, b->ne);
+        cudaMemcpyAsync(b->d_init, h, sizeof(InitEv) * b->ne, cudaMemcpyHostToDevice, b->stream);
+        launch_mv_init(h, b->d_init, b->ne, b->stream);
+        for (int e = 0; e < b->ne; e++) ctx_init_done(b->ev[e]);
+        for (int e = 0; e < b->ne && st == GL_OK; e++) {
+            st = wong_init(b->ev[e]);
+            if (st != GL_OK) {
+                char m[300];
+                snprintf(m, sizeof m, "event %d: %s", e, gl_error_string(b->ev[e]));
+                bfail(b, st, m);
+            }
+        }
+        cudaMemcpyAsync(bad, b->d_bad, sizeof(int) * b->ne, cudaMemcpyDeviceToHost, b->stream);
+        if (cudaStreamSynchronize(b->stream) != cudaSuccess || cudaGetLastError() != cudaSuccess)
+            st = bfail(b, GL_ERR_CUDA, "batch initial conditions failed");
+    }
+    for (int e = 0; e < b->ne && st == GL_OK; e++)
+        if (bad[e]) {
+            char m[160];
+            snprintf(m, sizeof m, "event %d: link matching did not converge on %d links", e, bad[e]);
+            st = bfail(b, GL_ERR_NUMERIC, m);
+        }
+    delete[] h;
+    delete[] bad;
+    return st;
 }
 
 // refresh the device descriptors from the contexts; all events must be at the

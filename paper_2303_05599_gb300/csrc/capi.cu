@@ -11,7 +11,6 @@
 #include "internal.h"
 
 namespace gl {
-size_t init_scratch_bytes(int64_t Vn);
 void launch_parts_convert(int prec, void* parts, int64_t np, double* stg, int to_device, cudaStream_t st);
 }  // namespace gl
 
@@ -142,7 +141,7 @@ static Carve carve(const gl_config* cfg, int64_t np, int ns) {
     const size_t nj = cfg->n_jets > 0 ? (size_t)cfg->n_jets : 0;
     c.jets = o; o += nj ? a256(nj * JET_LEN * (prec == 0 ? 8 : 4)) : 0;
     c.jet_partials = o; o += nj ? a256((1024 * 3 + 3) * sizeof(double)) : 0;
-    size_t sc = init_scratch_bytes(Vn);
+    size_t sc = init_scratch_bytes(cfg->N, cfg->Ns);
     size_t stg = (size_t)Vn * 6 * 8 * sizeof(double);
     if (stg > sc) sc = stg;
     if ((size_t)np * 16 * sizeof(double) > sc) sc = (size_t)np * 16 * sizeof(double);
@@ -248,6 +247,15 @@ PartsCheckEv ctx_parts_check_event(const gl_ctx* c) {
     e.block_begin = 0;
     e.nblocks = parts_check_blocks(c->np);
     return e;
+}
+InitEv ctx_init_event(const gl_ctx* c, int* bad) {
+    return init_event(c->prec, c->field[c->cur], c->scratch, c->N, c->cfg.Ns, c->g2mu_a, c->m_a, c->Lambda_a,
+                      c->cfg.seed, bad);
+}
+void ctx_init_done(gl_ctx* c) {
+    for (int k = 0; k < 2; k++) cudaMemsetAsync(c->site_buf[k], 0, site_bytes(c->prec, c->Vn), c->stream);
+    c->step = c->pstep = 0;
+    site_forget(c);
 }
 void ctx_obs_fill(const gl_ctx* c, uint32_t what, const double* host, gl_obs* o) {
     ::observables_fill(c, what, host, o);
@@ -383,15 +391,14 @@ static uint32_t active_mask(const gl_ctx* c, int64_t n) {
 gl_status glasma_init(gl_ctx* c) {
     gl::ApiRange range_("glasma_init");
     if (!c) return GL_ERR_ARG;
-    launch_mv_init(c->prec, c->field[c->cur], c->scratch, c->N, c->cfg.Ns, c->g2mu_a, c->m_a, c->Lambda_a,
-                   c->cfg.seed, c->d_bad, c->stream);
-    for (int k = 0; k < 2; k++) cudaMemsetAsync(c->site_buf[k], 0, site_bytes(c->prec, c->Vn), c->stream);
+    if (!init_supported(c->N)) return fail(c, GL_ERR_CUDA, "glasma_init: N is beyond the transforms' shared memory");
+    const InitEv ev = ctx_init_event(c, c->d_bad);
+    launch_mv_init(&ev, nullptr, 1, c->stream);
+    ctx_init_done(c);
     if (gl_status s = check_cuda(c, "glasma_init")) return s;
     int bad = 0;
     cudaMemcpyAsync(&bad, c->d_bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return check_cuda(c, "glasma_init sync");
-    c->step = c->pstep = 0;
-    site_forget(c);
     if (bad) {
         char m[128];
         snprintf(m, sizeof m, "link matching did not converge on %d links", bad);

@@ -2,7 +2,7 @@
 // arXiv:2303.05599), all in FP64:
 //   rho^a_n(x) ~ N(0, (g^2 mu a)^2 / Ns) per sheet n, colour a, site x
 //   alpha_n = rho_n / (k^2 + m^2) in Fourier space (lattice k^2, zero mode
-//             removed, modes with k > Lambda removed), radix-2 FFTs in shared memory
+//             removed, modes with k > Lambda removed)
 //   V^+(x) = prod_n exp(-i alpha_n(x)), sheet 1 leftmost
 //   U^{A,B}_i(x) = V(x) V^+(x+i)
 //   Glasma link U_i: tr T^a [(U^A + U^B)(1 + U^+) - h.c.] = 0, Newton iteration
@@ -12,155 +12,570 @@
 // The paper states only that the continuum conditions are discretised; the
 // matching condition is the standard one of the boost-invariant Glasma
 // literature it builds on.
+#include <math.h>
+#include <string.h>
+
 #include "internal.h"
 #include "layout.cuh"
 #include "philox.cuh"
 
 namespace gl {
 
-// scratch layout (bytes): [rho | U64] overlapped, then VdA, VdB
-//   rho: 8 planes of Vn double2;  U64: 2 dirs x 9 planes of Vn double2
-//   VdA, VdB: 9 planes of Vn double2 each
-static size_t init_region0(int64_t Vn) { return (size_t)18 * Vn * sizeof(double2); }
+// Work per nucleus and sheet: four complex planes, each two real colour planes
+// of rho (the Green function is real and even, so the two parts of a plane
+// stay apart through both transforms), and three launches over all events:
+//   rows      rho of a few lattice rows into shared memory, their forward
+//             transforms, out to `work`
+//   columns   a tile of columns in: forward transform, Green function, inverse
+//             transform, out
+//   sheets    rows in: inverse transform, then per site exp(-i alpha) and the
+//             product with the Wilson line
+// The transforms work in place: the forward ones (decimation in frequency)
+// leave each line in digit-reversed order, the Green table is stored in that
+// order, and the inverse ones (decimation in time) start from it, so nothing
+// is permuted.  Powers of two take radix 4 (and one radix 2), other sizes one
+// direct pass per prime factor; the twiddles come from one table per event.
+//
+// What bounds it: FP64 arithmetic (GB300 issues one FP64 warp instruction per
+// 19 cycles of an SM), so the passes are arranged to do less of it.  Radix-2
+// transforms of eight complex planes with a sincospi per butterfly, a
+// 20-term exponential series and whole matrices took 105.7 ms for a 256^2
+// event of 50 sheets, 223 us a transform pass.
+//
+// A sheet's planes wait in `work`, as many sheets a round as the scratch holds.
+// Small lattices (all sheets in one round) split each nucleus's product over
+// groups of consecutive sheets, whose partial products are multiplied at the
+// end: 1024 sites alone would leave most of the chip idle.  Rounds and groups
+// depend on N and Ns only, so an event's fields are bitwise the same alone and
+// in a batch.
 
-size_t init_scratch_bytes(int64_t Vn) { return init_region0(Vn) + (size_t)18 * Vn * sizeof(double2); }
+static constexpr int INIT_T = 256;                  // threads of the line kernels
+static constexpr int INIT_MAX_N = 3072;             // longest line
+static constexpr int INIT_GEN_OUT = 12;             // outputs a thread of a prime pass: 256 x 12 = 3072 points
+static constexpr size_t INIT_ROUND_BYTES = (size_t)32 << 20;  // scratch small events may use for more sheets a round
 
-__global__ void set_identity_kernel(double2* Vd, int64_t Vn) {
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < Vn; s += (int64_t)gridDim.x * blockDim.x)
-        for (int k = 0; k < 9; k++) Vd[(size_t)k * Vn + s] = make_double2(k % 4 == 0 ? 1.0 : 0.0, 0.0);
-}
+struct InitPlan {
+    int S, groups, per_group;  // sheets a round, groups of sheets, sheets a group
+    size_t v, tw, work, total; // byte offsets
+};
 
-__global__ void rho_kernel(double2* rho, int64_t Vn, int Ns, int nucleus, int sheet, double sigma, uint32_t k0,
-                           uint32_t k1) {
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < Vn; s += (int64_t)gridDim.x * blockDim.x) {
-        double z[8];
-        for (int j = 0; j < 2; j++) {
-            U4 w = philox4x32_10(U4{(uint32_t)s, (uint32_t)((nucleus * Ns + sheet) * 2 + j), 1u, 0u}, k0, k1);
-            box_muller(u01(w.x), u01(w.y), z[4 * j], z[4 * j + 1]);
-            box_muller(u01(w.z), u01(w.w), z[4 * j + 2], z[4 * j + 3]);
-        }
-        for (int a = 0; a < 8; a++) rho[(size_t)a * Vn + s] = make_double2(sigma * z[a], 0.0);
+static InitPlan init_plan(int N, int Ns) {
+    const size_t V = (size_t)N * N;
+    InitPlan p;
+    const size_t tw = ((size_t)N * 16 + 255) & ~(size_t)255;
+    // per site: 128 B a sheet (both nuclei), 8 B Green function, 192 B a group
+    // (two nuclei's lines as two rows); later 192 B links and 128 B commutators
+    // in the place of work and Green function
+    int g = (int)(16384 / V);
+    g = g < 1 ? 1 : (g > Ns ? Ns : g);
+    p.per_group = (Ns + g - 1) / g;
+    p.groups = (Ns + p.per_group - 1) / p.per_group;
+    p.S = Ns;
+    const size_t base = 576 * V;
+    const size_t room = base > INIT_ROUND_BYTES ? base : INIT_ROUND_BYTES;
+    if ((size_t)Ns * 128 * V + 8 * V + (size_t)p.groups * 192 * V + tw > room) {
+        p.groups = 1;
+        p.per_group = Ns;
+        p.S = (int)((room - 200 * V - tw) / (128 * V));
+        if (p.S < 2) p.S = 2;
+        if (p.S > Ns) p.S = Ns;
     }
+    size_t w = (size_t)p.S * 128 * V + 8 * V;
+    if (w < 320 * V) w = 320 * V;
+    p.v = 0;
+    p.tw = (size_t)p.groups * 192 * V;
+    p.work = p.tw + tw;
+    p.total = p.work + w;
+    return p;
 }
 
-// one line (row or column) of one plane per block, radix 2 in shared memory
-__global__ void fft_pow2_kernel(double2* data, int N, int log2N, int sign, int rows, int64_t Vn) {
-    extern __shared__ double2 sh[];
-    double2* base = data + (size_t)blockIdx.y * Vn;
-    const int line = blockIdx.x;
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        const int64_t idx = rows ? (int64_t)line * N + k : (int64_t)k * N + line;
-        const int rev = (int)(__brev((unsigned)k) >> (32 - log2N));
-        sh[rev] = base[idx];
+size_t init_scratch_bytes(int N, int Ns) { return init_plan(N, Ns).total; }
+
+// blocks of the kernels of one event
+static inline int rows_lines(int N) { return N >= 1024 ? 1 : 1024 / N; }          // lines a block of `rows`
+static inline int cols_tile(int N, bool pow2) {                                    // columns a block of `columns`
+    int c = pow2 ? (N > 1024 ? 2 : (N >= 256 ? 4 : 1024 / N)) : (N <= 256 ? 1024 / N : INIT_MAX_N / N);
+    return c < 1 ? 1 : (c > N ? N : c);
+}
+static inline int sheet_rows(int N) { return N >= 256 ? 1 : 256 / N; }             // rows a block of `sheets`
+
+InitEv init_event(int prec, void* fields, void* scratch, int N, int Ns, double g2mu_a, double m_a, double Lambda_a,
+                  uint64_t seed, int* bad) {
+    InitEv e;
+    memset(&e, 0, sizeof e);
+    const InitPlan p = init_plan(N, Ns);
+    const int64_t V = (int64_t)N * N;
+    e.N = N;
+    e.Ns = Ns;
+    e.S = p.S;
+    e.groups = p.groups;
+    e.per_group = p.per_group;
+    e.pow2 = (N & (N - 1)) == 0;
+    if (e.pow2) {
+        int l = 0;
+        while ((1 << l) < N) l++;
+        e.log2N = l;
+        for (; l >= 2; l -= 2) e.rad[e.nrad++] = 4;
+        if (l) e.rad[e.nrad++] = 2;
+    } else {
+        int r = N;
+        for (int q = 2; q * q <= r; q++)
+            while (r % q == 0) { e.rad[e.nrad++] = q; r /= q; }
+        if (r > 1) e.rad[e.nrad++] = r;
+    }
+    e.lines = rows_lines(N);
+    e.cols = cols_tile(N, e.pow2);
+    e.rows = sheet_rows(N);
+    e.sigma = g2mu_a / sqrt((double)Ns);
+    e.m2 = m_a * m_a;
+    e.lam2 = Lambda_a > 0 ? Lambda_a * Lambda_a : 0.0;
+    e.k0 = (uint32_t)seed;
+    e.k1 = (uint32_t)(seed >> 32);
+    char* s = (char*)scratch;
+    e.V = (double2*)(s + p.v);
+    e.tw = (double2*)(s + p.tw);
+    e.work = (double2*)(s + p.work);
+    e.green = (double*)(s + p.work + (size_t)p.S * 128 * V);
+    e.U64 = (double2*)(s + p.work);
+    e.comm = e.U64 + (size_t)12 * V;
+    e.fields = fields;
+    e.prec = prec;
+    e.bad = bad;
+    return e;
+}
+
+// the block's event and its block index there, for launch `k` of the table
+__device__ __forceinline__ const InitEv& init_find(const InitEv* evs, int ne, const InitEv& one, int k, int* blk) {
+    int lo = 0, hi = ne - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (evs[mid].begin[k] <= (int)blockIdx.x) lo = mid;
+        else hi = mid - 1;
+    }
+    const InitEv& d = evs ? evs[lo] : one;
+    *blk = blockIdx.x - (evs ? d.begin[k] : 0);
+    return d;
+}
+enum { IK_TABLES = 0, IK_ROWS, IK_COLS, IK_SHEETS, IK_SITES, IK_LINKS, IK_N };
+static_assert(IK_N <= InitEv::KINDS, "block table");
+
+// ------------------------------------------------------------ line transforms
+// `lines` lines of N points in shared memory, `ls` points apart, transformed in
+// place by the block (no barrier before, one after each pass).
+__device__ __forceinline__ double2 cmul(double2 a, double2 w) {
+    return make_double2(fma(a.x, w.x, -(a.y * w.y)), fma(a.x, w.y, a.y * w.x));
+}
+__device__ __forceinline__ double2 cmulc(double2 a, double2 w) {  // a conj(w)
+    return make_double2(fma(a.x, w.x, a.y * w.y), fma(a.y, w.x, -(a.x * w.y)));
+}
+__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+
+// powers of two: radix 4, and radix 2 on neighbours for odd log2 N
+__device__ __forceinline__ void pow2_radix2(double2* sh, int lines, int ls, int lN) {
+    for (int b = threadIdx.x; b < lines << (lN - 1); b += blockDim.x) {
+        double2* p = sh + (b >> (lN - 1)) * ls + 2 * (b & ((1 << (lN - 1)) - 1));
+        const double2 u = p[0], v = p[1];
+        p[0] = cadd(u, v);
+        p[1] = csub(u, v);
     }
     __syncthreads();
-    for (int len = 2; len <= N; len <<= 1) {
-        const int half = len >> 1;
-        for (int b = threadIdx.x; b < N / 2; b += blockDim.x) {
-            const int grp = b / half, k = b % half;
-            const int i0 = grp * len + k, i1 = i0 + half;
-            double sn, cs;
-            sincospi(sign * 2.0 * (double)k / (double)len, &sn, &cs);
-            const double2 u = sh[i0], v = sh[i1];
-            const double2 vw = make_double2(v.x * cs - v.y * sn, v.x * sn + v.y * cs);
-            sh[i0] = make_double2(u.x + vw.x, u.y + vw.y);
-            sh[i1] = make_double2(u.x - vw.x, u.y - vw.y);
+}
+__device__ __forceinline__ void pow2_forward(double2* sh, int lines, int ls, int lN, const double2* __restrict__ tw) {
+    for (int lb = lN; lb >= 2; lb -= 2) {
+        const int q = 1 << (lb - 2);
+        for (int b = threadIdx.x; b < lines << (lN - 2); b += blockDim.x) {
+            const int j = b & ((1 << (lN - 2)) - 1), n = j & (q - 1);
+            double2* p = sh + (b >> (lN - 2)) * ls + ((j >> (lb - 2)) << lb) + n;
+            const double2 a0 = p[0], a1 = p[q], a2 = p[2 * q], a3 = p[3 * q];
+            const double2 t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), t3 = csub(a1, a3);
+            p[0] = cadd(t0, t2);
+            // t1 -+ i t3
+            const double2 y1 = make_double2(t1.x + t3.y, t1.y - t3.x), y2 = csub(t0, t2),
+                          y3 = make_double2(t1.x - t3.y, t1.y + t3.x);
+            if (lb > 2) {
+                const int w = n << (lN - lb);
+                p[q] = cmulc(y1, __ldg(tw + w));
+                p[2 * q] = cmulc(y2, __ldg(tw + 2 * w));
+                p[3 * q] = cmulc(y3, __ldg(tw + 3 * w));
+            } else {
+                p[q] = y1;
+                p[2 * q] = y2;
+                p[3 * q] = y3;
+            }
         }
         __syncthreads();
     }
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        const int64_t idx = rows ? (int64_t)line * N + k : (int64_t)k * N + line;
-        base[idx] = sh[k];
-    }
+    if (lN & 1) pow2_radix2(sh, lines, ls, lN);
 }
-
-// direct DFT of one line (any N), used when N is not a power of two
-__global__ void dft_kernel(double2* data, int N, int sign, int rows, int64_t Vn) {
-    extern __shared__ double2 sh[];
-    double2* base = data + (size_t)blockIdx.y * Vn;
-    const int line = blockIdx.x;
-    for (int k = threadIdx.x; k < N; k += blockDim.x)
-        sh[k] = base[rows ? (int64_t)line * N + k : (int64_t)k * N + line];
-    __syncthreads();
-    for (int k = threadIdx.x; k < N; k += blockDim.x) {
-        double re = 0, im = 0;
-        for (int j = 0; j < N; j++) {
-            double sn, cs;
-            sincospi(sign * 2.0 * (double)((int64_t)j * k % N) / (double)N, &sn, &cs);
-            re += sh[j].x * cs - sh[j].y * sn;
-            im += sh[j].x * sn + sh[j].y * cs;
+__device__ __forceinline__ void pow2_inverse(double2* sh, int lines, int ls, int lN, const double2* __restrict__ tw) {
+    if (lN & 1) pow2_radix2(sh, lines, ls, lN);
+    for (int lb = 2 + (lN & 1); lb <= lN; lb += 2) {
+        const int q = 1 << (lb - 2);
+        for (int b = threadIdx.x; b < lines << (lN - 2); b += blockDim.x) {
+            const int j = b & ((1 << (lN - 2)) - 1), n = j & (q - 1);
+            double2* p = sh + (b >> (lN - 2)) * ls + ((j >> (lb - 2)) << lb) + n;
+            double2 x1 = p[q], x2 = p[2 * q], x3 = p[3 * q];
+            const double2 x0 = p[0];
+            if (lb > 2) {
+                const int w = n << (lN - lb);
+                x1 = cmul(x1, __ldg(tw + w));
+                x2 = cmul(x2, __ldg(tw + 2 * w));
+                x3 = cmul(x3, __ldg(tw + 3 * w));
+            }
+            const double2 t0 = cadd(x0, x2), t1 = csub(x0, x2), t2 = cadd(x1, x3), t3 = csub(x1, x3);
+            p[0] = cadd(t0, t2);
+            p[q] = make_double2(t1.x - t3.y, t1.y + t3.x);
+            p[2 * q] = csub(t0, t2);
+            p[3 * q] = make_double2(t1.x + t3.y, t1.y - t3.x);
         }
-        base[rows ? (int64_t)line * N + k : (int64_t)k * N + line] = make_double2(re, im);
+        __syncthreads();
     }
 }
 
-static void fft2(double2* data, int planes, int N, int sign, cudaStream_t st) {
-    const int64_t Vn = (int64_t)N * N;
-    int log2N = 0;
-    while ((1 << log2N) < N) log2N++;
-    const bool pow2 = (1 << log2N) == N;
-    const size_t shm = (size_t)N * sizeof(double2);
-    dim3 grid(N, planes);
-    const int threads = N >= 512 ? 256 : 128;
-    for (int rows = 1; rows >= 0; rows--) {
-        if (pow2) fft_pow2_kernel<<<grid, threads, shm, st>>>(data, N, log2N, sign, rows, Vn);
-        else dft_kernel<<<grid, threads, shm, st>>>(data, N, sign, rows, Vn);
+// any N: a direct transform of each prime factor in turn, one output point at
+// a time (a block's points, at most 256 x INIT_GEN_OUT, wait in registers for
+// the barrier before they replace the inputs)
+template <bool FORWARD>
+__device__ void prime_passes(double2* sh, int lines, int ls, const InitEv& d) {
+    const int N = d.N, total = lines * N;
+    int B = N;
+    if (!FORWARD)
+        for (int s = 0; s + 1 < d.nrad; s++) B /= d.rad[s];
+    for (int i = 0; i < d.nrad; i++) {
+        const int s = FORWARD ? i : d.nrad - 1 - i;
+        const int r = d.rad[s], m = B / r;
+        const int wr = N / r, wB = N / B;
+        double2 out[INIT_GEN_OUT];
+#pragma unroll
+        for (int c = 0; c < INIT_GEN_OUT; c++) {
+            const int idx = threadIdx.x + c * INIT_T;
+            if (idx < total) {
+                const int line = idx / N, p = idx - line * N, nb = p / B, k = (p - nb * B) / m, n = p % m;
+                const double2* x = sh + line * ls + nb * B + n;
+                double2 a = make_double2(0.0, 0.0);
+                int w = 0;               // (q k mod r) N / r
+                const int step = k * wr;
+                int tn = 0;              // inverse: n q N / B
+                for (int q = 0; q < r; q++) {
+                    const double2 v = x[q * m];
+                    if (FORWARD) {
+                        const double2 t = cmulc(v, __ldg(d.tw + w));
+                        a = cadd(a, t);
+                    } else {
+                        int u = w + tn;
+                        if (u >= N) u -= N;
+                        const double2 t = cmul(v, __ldg(d.tw + u));
+                        a = cadd(a, t);
+                        tn += n * wB;
+                        if (tn >= N) tn -= N;
+                    }
+                    w += step;
+                    if (w >= N) w -= N;
+                }
+                if (FORWARD) a = cmulc(a, __ldg(d.tw + n * k * wB));
+                out[c] = a;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < INIT_GEN_OUT; c++) {
+            const int idx = threadIdx.x + c * INIT_T;
+            if (idx < total) {
+                const int line = idx / N;
+                sh[line * ls + idx - line * N] = out[c];
+            }
+        }
+        __syncthreads();
+        if (FORWARD) B = m;
+        else B *= i + 1 < d.nrad ? d.rad[s - 1] : 1;
     }
 }
 
-__global__ void green_kernel(double2* rho, int N, double m2, double lam2, double invV) {
-    const int64_t Vn = (int64_t)N * N;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < Vn; s += (int64_t)gridDim.x * blockDim.x) {
-        const int kx = (int)(s % N), ky = (int)(s / N);
+__device__ __forceinline__ void lines_forward(double2* sh, int lines, int ls, const InitEv& d) {
+    if (d.pow2) pow2_forward(sh, lines, ls, d.log2N, d.tw);
+    else prime_passes<true>(sh, lines, ls, d);
+}
+__device__ __forceinline__ void lines_inverse(double2* sh, int lines, int ls, const InitEv& d) {
+    if (d.pow2) pow2_inverse(sh, lines, ls, d.log2N, d.tw);
+    else
+        for (int l = 0; l < lines;) {  // at most INIT_T x INIT_GEN_OUT points at a time
+            int c = INIT_T * INIT_GEN_OUT / d.N;
+            if (c > lines - l) c = lines - l;
+            prime_passes<false>(sh + (size_t)l * ls, c, ls, d);
+            l += c;
+        }
+}
+
+// ------------------------------------------------------------ kernels
+// the frequency at position p of a transformed line
+__device__ __forceinline__ int line_frequency(const InitEv& d, int p) {
+    int B = d.N, f = 0, scale = 1;
+    for (int s = 0; s < d.nrad; s++) {
+        const int m = B / d.rad[s], k = p / m;
+        p -= k * m;
+        f += k * scale;
+        scale *= d.rad[s];
+        B = m;
+    }
+    return f;
+}
+
+// the event's twiddles and its Green function over the number of sites, in the
+// order the transforms leave
+__global__ void __launch_bounds__(INIT_T) init_tables_kernel(const InitEv* evs, int ne, InitEv one) {
+    int blk;
+    const InitEv& d = init_find(evs, ne, one, IK_TABLES, &blk);
+    const int N = d.N;
+    const int64_t Vn = (int64_t)N * N, s = (int64_t)blk * INIT_T + threadIdx.x;
+    if (s == 0) *d.bad = 0;
+    if (s < N) {
+        double sn, cs;
+        sincospi(2.0 * (double)s / (double)N, &sn, &cs);
+        d.tw[s] = make_double2(cs, sn);
+    }
+    if (s < Vn) {
+        const int px = (int)(s % N), py = (int)(s / N);
+        const int kx = line_frequency(d, px), ky = line_frequency(d, py);
         const double sx = sinpi((double)kx / N), sy = sinpi((double)ky / N);
         const double k2 = 4.0 * (sx * sx + sy * sy);
-        double g = 1.0 / (k2 + m2);
+        double g = 1.0 / (k2 + d.m2);
         if (kx == 0 && ky == 0) g = 0.0;
-        if (lam2 > 0 && k2 > lam2) g = 0.0;
-        g *= invV;
-        for (int a = 0; a < 8; a++) {
-            double2 v = rho[(size_t)a * Vn + s];
-            rho[(size_t)a * Vn + s] = make_double2(v.x * g, v.y * g);
+        if (d.lam2 > 0 && k2 > d.lam2) g = 0.0;
+        d.green[s] = g * (1.0 / (double)Vn);
+    }
+}
+
+// rho of d.lines lattice rows of one or two planes and their forward transforms
+__global__ void __launch_bounds__(INIT_T) init_rows_kernel(const InitEv* evs, int ne, InitEv one, int round) {
+    extern __shared__ __align__(16) unsigned char init_smem[];
+    double2* sh = (double2*)init_smem;
+    int blk;
+    const InitEv& d = init_find(evs, ne, one, IK_ROWS, &blk);
+    const int N = d.N, S = d.S;
+    const int64_t all = (int64_t)2 * S * 4 * N, line0 = (int64_t)blk * d.lines;
+    const int nl = (int)(all - line0 < d.lines ? all - line0 : d.lines);
+    for (int idx = threadIdx.x; idx < nl * N; idx += INIT_T) {
+        const int l = idx / N, x = idx - l * N;
+        const int64_t line = line0 + l;
+        const int row = (int)(line % N), plane = (int)(line / N) & 3, slot = (int)(line / (4 * (int64_t)N));
+        const int nucleus = slot / S, sheet = round * S + slot - nucleus * S;
+        double2 z = make_double2(0.0, 0.0);
+        if (sheet < d.Ns) {
+            const U4 w = philox4x32_10(U4{(uint32_t)(row * N + x), (uint32_t)((nucleus * d.Ns + sheet) * 2 + (plane >> 1)),
+                                          1u, 0u}, d.k0, d.k1);
+            double z0, z1;
+            box_muller(u01((plane & 1) ? w.z : w.x), u01((plane & 1) ? w.w : w.y), z0, z1);
+            z = make_double2(d.sigma * z0, d.sigma * z1);
         }
+        sh[idx] = z;
+    }
+    __syncthreads();
+    lines_forward(sh, nl, N, d);
+    double2* out = d.work + (size_t)line0 * N;  // work[slot][plane][row][position]
+    for (int idx = threadIdx.x; idx < nl * N; idx += INIT_T) out[idx] = sh[idx];
+}
+
+// alpha = rho / (k^2 + m^2) along the columns of one plane
+__global__ void __launch_bounds__(INIT_T) init_cols_kernel(const InitEv* evs, int ne, InitEv one, int round) {
+    extern __shared__ __align__(16) unsigned char init_smem[];
+    double2* sh = (double2*)init_smem;
+    int blk;
+    const InitEv& d = init_find(evs, ne, one, IK_COLS, &blk);
+    const int N = d.N, S = d.S, C = d.cols, ls = N + 1;  // a point of padding: neighbouring columns in other banks
+    const int nt = (N + C - 1) / C;
+    const int c0 = (blk % nt) * C, sp = blk / nt, slot = sp >> 2;
+    if (round * S + slot % S >= d.Ns) return;
+    const int nc = N - c0 < C ? N - c0 : C;
+    double2* w = d.work + (size_t)sp * N * N + c0;
+    for (int idx = threadIdx.x; idx < nc * N; idx += INIT_T) {
+        const int r = idx / nc, c = idx - r * nc;
+        sh[c * ls + r] = w[(size_t)r * N + c];
+    }
+    __syncthreads();
+    lines_forward(sh, nc, ls, d);
+    const double* g = d.green + c0;
+    for (int idx = threadIdx.x; idx < nc * N; idx += INIT_T) {
+        const int r = idx / nc, c = idx - r * nc;
+        const double f = g[(size_t)r * N + c];
+        double2 v = sh[c * ls + r];
+        v.x *= f;
+        v.y *= f;
+        sh[c * ls + r] = v;
+    }
+    __syncthreads();
+    lines_inverse(sh, nc, ls, d);
+    for (int idx = threadIdx.x; idx < nc * N; idx += INIT_T) {
+        const int r = idx / nc, c = idx - r * nc;
+        w[(size_t)r * N + c] = sh[c * ls + r];
     }
 }
 
-__global__ void wilson_accum_kernel(double2* Vd, const double2* rho, int64_t Vn) {
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < Vn; s += (int64_t)gridDim.x * blockDim.x) {
-        A8<double> al;
-        for (int a = 0; a < 8; a++) al.v[a] = -rho[(size_t)a * Vn + s].x;
-        const M3<double> e = exp_i_alg<double>(al, 1.0);
-        const M3<double> v = load_link(Vd, 0, s, Vn);
-        store_link(Vd, 0, s, Vn, mul(v, e));
+// an SU(3) matrix of the scratch: rows 0 and 1 in six planes, row 2 rebuilt
+__device__ __forceinline__ M3<double> load_rows(const double2* V, int64_t s, int64_t Vn) {
+    M3<double> m;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const double2 v = V[(size_t)k * Vn + s];
+        m.re[k / 3][k % 3] = v.x;
+        m.im[k / 3][k % 3] = v.y;
+    }
+    rebuild_row2(m);
+    return m;
+}
+__device__ __forceinline__ void store_rows(double2* V, int64_t s, int64_t Vn, const M3<double>& m) {
+#pragma unroll
+    for (int k = 0; k < 6; k++) V[(size_t)k * Vn + s] = make_double2(m.re[k / 3][k % 3], m.im[k / 3][k % 3]);
+}
+// (rows 0 and 1 of) v m
+__device__ __forceinline__ M3<double> mul_rows(const M3<double>& v, const M3<double>& m) {
+    M3<double> c = m_zero<double>();
+#pragma unroll
+    for (int i = 0; i < 2; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                c.re[i][j] = fma(v.re[i][k], m.re[k][j], c.re[i][j]);
+                c.re[i][j] = fma(-v.im[i][k], m.im[k][j], c.re[i][j]);
+                c.im[i][j] = fma(v.re[i][k], m.im[k][j], c.im[i][j]);
+                c.im[i][j] = fma(v.im[i][k], m.re[k][j], c.im[i][j]);
+            }
+    return c;
+}
+
+// the inverse transforms of d.rows rows of a nucleus and the product over its
+// sheets of this round (of one group of them)
+__global__ void __launch_bounds__(INIT_T) init_sheets_kernel(const InitEv* evs, int ne, InitEv one, int round) {
+    extern __shared__ __align__(16) unsigned char init_smem[];
+    double2* sh = (double2*)init_smem;
+    int blk;
+    const InitEv& d = init_find(evs, ne, one, IK_SHEETS, &blk);
+    const int N = d.N, S = d.S;
+    const int64_t Vn = (int64_t)N * N;
+    const int nrb = (N + d.rows - 1) / d.rows;
+    const int r0 = (blk % nrb) * d.rows, g = (blk / nrb) % d.groups, nucleus = blk / (nrb * d.groups);
+    const int nr = N - r0 < d.rows ? N - r0 : d.rows, np = nr * N;
+    const int first = g * d.per_group;
+    int s0 = round * S, s1 = s0 + S < d.Ns ? s0 + S : d.Ns;
+    if (s0 < first) s0 = first;
+    if (s1 > first + d.per_group) s1 = first + d.per_group;
+    double2* V = d.V + (size_t)(nucleus * d.groups + g) * 6 * Vn + (int64_t)r0 * N;
+    for (int s = s0; s < s1; s++) {
+        const double2* w = d.work + (size_t)(nucleus * S + s - round * S) * 4 * Vn + (int64_t)r0 * N;
+        for (int idx = threadIdx.x; idx < 4 * np; idx += INIT_T) {
+            const int p = idx / np;
+            sh[idx] = w[(size_t)p * Vn + idx - p * np];
+        }
+        __syncthreads();
+        lines_inverse(sh, 4 * nr, N, d);
+        for (int i = threadIdx.x; i < np; i += INIT_T) {
+            A8<double> al;
+#pragma unroll
+            for (int p = 0; p < 4; p++) {
+                const double2 v = sh[p * np + i];
+                al.v[2 * p] = -v.x;
+                al.v[2 * p + 1] = -v.y;
+            }
+            const M3<double> e = exp_i_alg<double>(al, 1.0);
+            // only this thread reads and writes the site's line, sheet after sheet
+            if (s == first) store_rows(V, i, Vn, e);
+            else store_rows(V, i, Vn, mul_rows(load_rows(V, i, Vn), e));
+        }
+        __syncthreads();
     }
 }
 
-// tr(T^a M) for the eight generators, complex
-__device__ void tr_T(const M3<double>& M, double* re, double* im) {
+// the groups' partial products, in order, into the first
+__global__ void __launch_bounds__(128) init_groups_kernel(const InitEv* evs, int ne, InitEv one) {
+    int blk;
+    const InitEv& d = init_find(evs, ne, one, IK_SITES, &blk);
+    const int64_t Vn = (int64_t)d.N * d.N, t = (int64_t)blk * 128 + threadIdx.x;
+    if (d.groups < 2 || t >= 2 * Vn) return;
+    const int64_t s = t % Vn;
+    double2* V = d.V + (size_t)(t / Vn) * d.groups * 6 * Vn;
+    M3<double> v = load_rows(V, s, Vn);
+    for (int g = 1; g < d.groups; g++) v = mul_rows(v, load_rows(V + (size_t)g * 6 * Vn, s, Vn));
+    store_rows(V, s, Vn, v);
+}
+
+// Im tr(T^a M)
+__device__ __forceinline__ void im_tr_T(const M3<double>& M, double* f) {
     const double h = 0.5, s3 = 0.5 * inv_sqrt3<double>();
-    re[0] = h * (M.re[1][0] + M.re[0][1]);             im[0] = h * (M.im[1][0] + M.im[0][1]);
-    re[1] = h * (M.im[1][0] - M.im[0][1]);             im[1] = h * (-M.re[1][0] + M.re[0][1]);
-    re[2] = h * (M.re[0][0] - M.re[1][1]);             im[2] = h * (M.im[0][0] - M.im[1][1]);
-    re[3] = h * (M.re[2][0] + M.re[0][2]);             im[3] = h * (M.im[2][0] + M.im[0][2]);
-    re[4] = h * (M.im[2][0] - M.im[0][2]);             im[4] = h * (-M.re[2][0] + M.re[0][2]);
-    re[5] = h * (M.re[2][1] + M.re[1][2]);             im[5] = h * (M.im[2][1] + M.im[1][2]);
-    re[6] = h * (M.im[2][1] - M.im[1][2]);             im[6] = h * (-M.re[2][1] + M.re[1][2]);
-    re[7] = s3 * (M.re[0][0] + M.re[1][1] - 2 * M.re[2][2]);
-    im[7] = s3 * (M.im[0][0] + M.im[1][1] - 2 * M.im[2][2]);
+    f[0] = h * (M.im[1][0] + M.im[0][1]);
+    f[1] = h * (M.re[0][1] - M.re[1][0]);
+    f[2] = h * (M.im[0][0] - M.im[1][1]);
+    f[3] = h * (M.im[2][0] + M.im[0][2]);
+    f[4] = h * (M.re[0][2] - M.re[2][0]);
+    f[5] = h * (M.im[2][1] + M.im[1][2]);
+    f[6] = h * (M.re[1][2] - M.re[2][1]);
+    f[7] = s3 * (M.im[0][0] + M.im[1][1] - 2 * M.im[2][2]);
+}
+// Re tr(T^a M)
+__device__ __forceinline__ void re_tr_T(const M3<double>& M, double* f) {
+    const double h = 0.5, s3 = 0.5 * inv_sqrt3<double>();
+    f[0] = h * (M.re[1][0] + M.re[0][1]);
+    f[1] = h * (M.im[1][0] - M.im[0][1]);
+    f[2] = h * (M.re[0][0] - M.re[1][1]);
+    f[3] = h * (M.re[2][0] + M.re[0][2]);
+    f[4] = h * (M.im[2][0] - M.im[0][2]);
+    f[5] = h * (M.re[2][1] + M.re[1][2]);
+    f[6] = h * (M.im[2][1] - M.im[1][2]);
+    f[7] = s3 * (M.re[0][0] + M.re[1][1] - 2 * M.re[2][2]);
 }
 
-__device__ double match_residual(const M3<double>& W, const M3<double>& U, double* F) {
-    M3<double> one_ud = dag(U);
-    one_ud.re[0][0] += 1; one_ud.re[1][1] += 1; one_ud.re[2][2] += 1;
-    const M3<double> M = mul(W, one_ud);
-    double re[8];
-    tr_T(M, re, F);
-    double r = 0;
-    for (int a = 0; a < 8; a++) r = fmax(r, fabs(F[a]));
-    return r;
+// Jacobian of F^a = Im tr T^a (W + K), K = W U^+, under U -> exp(i x.T) U:
+// J_ab = -Re tr(T^a K T^b).  With T^b T^a = delta/6 + (d + i f)_bac T^c / 2,
+// J_ab = -(delta_ab Re tr K / 6 + d_abc r^c / 2 + f_abc i^c / 2) for tr(T^c K)
+// = r^c + i i^c: the sixteen independent d and nine f, instead of eight
+// matrix products.
+__device__ __forceinline__ void match_jacobian(const M3<double>& K, double J[8][8]) {
+    double r[8], q[8];
+    re_tr_T(K, r);
+    im_tr_T(K, q);
+    const double t = -(K.re[0][0] + K.re[1][1] + K.re[2][2]) * (1.0 / 6.0);
+    const double h = 0.25, s3 = 0.5 * inv_sqrt3<double>();  // d / 2 for d = 1/2, 1/sqrt 3
+    const double fh = 0.25, fs = 0.43301270189221932338;    // f / 2 for f = 1/2, sqrt(3)/2
+#pragma unroll
+    for (int a = 0; a < 8; a++)
+#pragma unroll
+        for (int b = 0; b < 8; b++) J[a][b] = 0.0;
+    // diagonal: delta term and d_aac r^c
+    const double e8 = s3 * r[7], h8 = 0.5 * e8, h3 = h * r[2];
+    J[0][0] = J[1][1] = J[2][2] = t - e8;
+    J[3][3] = J[4][4] = t - h3 + h8;
+    J[5][5] = J[6][6] = t + h3 + h8;
+    J[7][7] = t + e8;
+#define GL_D(a, b, v) J[a][b] -= (v), J[b][a] -= (v)
+    GL_D(0, 7, s3 * r[0]); GL_D(1, 7, s3 * r[1]); GL_D(2, 7, s3 * r[2]);         // d118 d228 d338
+    GL_D(0, 3, h * r[5]); GL_D(0, 5, h * r[3]); GL_D(3, 5, h * r[0]);            // d146
+    GL_D(0, 4, h * r[6]); GL_D(0, 6, h * r[4]); GL_D(4, 6, h * r[0]);            // d157
+    GL_D(1, 3, -h * r[6]); GL_D(1, 6, -h * r[3]); GL_D(3, 6, -h * r[1]);         // d247
+    GL_D(1, 4, h * r[5]); GL_D(1, 5, h * r[4]); GL_D(4, 5, h * r[1]);            // d256
+    GL_D(2, 3, h * r[3]); GL_D(2, 4, h * r[4]);                                  // d344 d355
+    GL_D(2, 5, -h * r[5]); GL_D(2, 6, -h * r[6]);                                // d366 d377
+    const double m8 = 0.5 * s3;
+    GL_D(3, 7, -m8 * r[3]); GL_D(4, 7, -m8 * r[4]); GL_D(5, 7, -m8 * r[5]); GL_D(6, 7, -m8 * r[6]);  // d448..d778
+#undef GL_D
+#define GL_F(a, b, c, v)                             \
+    {                                                \
+        const double va = (v) * q[a], vb = (v) * q[b], vc = (v) * q[c]; \
+        J[a][b] -= vc; J[b][a] += vc;                \
+        J[b][c] -= va; J[c][b] += va;                \
+        J[c][a] -= vb; J[a][c] += vb;                \
+    }
+    GL_F(0, 1, 2, 0.5);
+    GL_F(0, 3, 6, fh); GL_F(0, 4, 5, -fh); GL_F(1, 3, 5, fh); GL_F(1, 4, 6, fh); GL_F(2, 3, 4, fh);
+    GL_F(2, 5, 6, -fh);
+    GL_F(3, 4, 7, fs); GL_F(5, 6, 7, fs);
+#undef GL_F
 }
 
-__device__ int solve8(double J[8][8], double* b) {
+// J x = b with row exchanges (the links with a small leading pivot), 1 if singular
+__device__ __noinline__ int solve8_pivot(const double* J8, double* b) {
+    double J[8][8];
+    for (int r = 0; r < 8; r++)
+        for (int c = 0; c < 8; c++) J[r][c] = J8[8 * r + c];
     for (int c = 0; c < 8; c++) {
         int p = c;
         for (int r = c + 1; r < 8; r++) if (fabs(J[r][c]) > fabs(J[p][c])) p = r;
@@ -182,37 +597,88 @@ __device__ int solve8(double J[8][8], double* b) {
     return 0;
 }
 
+// the Newton step dx = -J^-1 F at K.  J is close to -1 for links near the
+// unit matrix, so the elimination runs in its own order, in registers; where a
+// pivot falls below 1/16 of the diagonal's scale it is done again with row
+// exchanges
+__device__ __forceinline__ int match_step(const M3<double>& K, const double* F, double* x) {
+    double J[8][8];
+    match_jacobian(K, J);
+#pragma unroll
+    for (int a = 0; a < 8; a++) x[a] = -F[a];
+    bool small = false;
+    double inv[8];
+#pragma unroll
+    for (int c = 0; c < 8; c++) {
+        small = small || !(fabs(J[c][c]) > 0.0625);
+        inv[c] = 1.0 / J[c][c];
+#pragma unroll
+        for (int r = c + 1; r < 8; r++) {
+            const double f = J[r][c] * inv[c];
+#pragma unroll
+            for (int k = c + 1; k < 8; k++) J[r][k] = fma(-f, J[c][k], J[r][k]);
+            x[r] = fma(-f, x[c], x[r]);
+        }
+    }
+#pragma unroll
+    for (int c = 7; c >= 0; c--) {
+#pragma unroll
+        for (int k = c + 1; k < 8; k++) x[c] = fma(-J[c][k], x[k], x[c]);
+        x[c] *= inv[c];
+    }
+    if (!small) return 0;
+    double Jp[64], b[8];
+    match_jacobian(K, J);
+#pragma unroll
+    for (int a = 0; a < 8; a++) {
+        b[a] = -F[a];
+#pragma unroll
+        for (int k = 0; k < 8; k++) Jp[8 * a + k] = J[a][k];
+    }
+    const int bad = solve8_pivot(Jp, b);
+#pragma unroll
+    for (int a = 0; a < 8; a++) x[a] = b[a];
+    return bad;
+}
+
+// F^a = Im tr T^a (W + K), K = W U^+, and its largest entry
+__device__ __forceinline__ double match_residual(const M3<double>& K, const double* fw, double* F) {
+    im_tr_T(K, F);
+    double r = 0;
+#pragma unroll
+    for (int a = 0; a < 8; a++) {
+        F[a] += fw[a];
+        r = fmax(r, fabs(F[a]));
+    }
+    return r;
+}
+
 // Newton solve for the Glasma link from the pure-gauge links of both nuclei
 __device__ int solve_link(const M3<double>& UA, const M3<double>& UB, M3<double>& U) {
     const M3<double> W = add(UA, UB);
+    double fw[8], F[8];
+    im_tr_T(W, fw);
     U = mul(UA, UB);
-    double F[8];
-    double r = match_residual(W, U, F);
+    M3<double> K = mul_nd(W, U);
+    double r = match_residual(K, fw, F);
     for (int it = 0; it < 100 && r > 1e-14; it++) {
-        // dF^a/dx^b for U -> exp(i x.T) U:  -Re tr(T^a W U^+ T^b)
-        const M3<double> K = mul_nd(W, U);
-        double J[8][8];
-        for (int b = 0; b < 8; b++) {
-            A8<double> eb = a_zero<double>();
-            eb.v[b] = 1.0;
-            const M3<double> KT = mul(K, alg_to_mat(eb));
-            double re[8], im[8];
-            tr_T(KT, re, im);
-            for (int a = 0; a < 8; a++) J[a][b] = -re[a];
-        }
         double dx[8];
-        for (int a = 0; a < 8; a++) dx[a] = -F[a];
-        if (solve8(J, dx)) break;
+        if (match_step(K, F, dx)) break;
         double lam = 1.0;
         for (int k = 0; k < 30; k++) {
             A8<double> st;
+#pragma unroll
             for (int a = 0; a < 8; a++) st.v[a] = lam * dx[a];
-            const M3<double> Un = mul(exp_i_alg<double>(st, 1.0), U);
+            M3<double> Un = mul_rows(exp_i_alg<double>(st, 1.0), U);
+            rebuild_row2(Un);
+            const M3<double> Kn = mul_nd(W, Un);
             double Fn[8];
-            const double rn = match_residual(W, Un, Fn);
+            const double rn = match_residual(Kn, fw, Fn);
             if (rn < r || k == 29) {
                 U = Un;
+                K = Kn;
                 r = rn;
+#pragma unroll
                 for (int a = 0; a < 8; a++) F[a] = Fn[a];
                 break;
             }
@@ -222,22 +688,25 @@ __device__ int solve_link(const M3<double>& UA, const M3<double>& UB, M3<double>
     return r > 1e-12;
 }
 
-__device__ __forceinline__ M3<double> nucleus_link(const double2* Vd, int d, int64_t s, int N, int64_t Vn) {
+// The Glasma link (d, s), as two rows, and i[-i[U^A]_ah, -i[U^B]_ah] of the
+// link, which E_eta(0) of both its ends needs.
+__global__ void __launch_bounds__(64) init_links_kernel(const InitEv* evs, int ne, InitEv one) {
+    int blk;
+    const InitEv& ev = init_find(evs, ne, one, IK_LINKS, &blk);
+    const int N = ev.N;
+    const int64_t Vn = (int64_t)N * N, l = (int64_t)blk * 64 + threadIdx.x;
+    if (l >= 2 * Vn) return;
+    const int d = (int)(l / Vn);
+    const int64_t s = l % Vn;
     const int x = (int)(s % N), y = (int)(s / N);
     const int64_t sn = d == 0 ? (int64_t)y * N + (x + 1 == N ? 0 : x + 1) : (int64_t)(y + 1 == N ? 0 : y + 1) * N + x;
-    return mul_dn(load_link(Vd, 0, s, Vn), load_link(Vd, 0, sn, Vn));
-}
-
-__global__ void glasma_link_kernel(const double2* VdA, const double2* VdB, double2* U64, int N, int* bad) {
-    const int64_t Vn = (int64_t)N * N;
-    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < 2 * Vn; l += (int64_t)gridDim.x * blockDim.x) {
-        const int d = (int)(l / Vn);
-        const int64_t s = l % Vn;
-        M3<double> U;
-        const int b = solve_link(nucleus_link(VdA, d, s, N, Vn), nucleus_link(VdB, d, s, N, Vn), U);
-        if (b) atomicAdd(bad, 1);
-        store_link(U64, d, s, Vn, U);
-    }
+    const double2* VB = ev.V + (size_t)ev.groups * 6 * Vn;
+    const M3<double> UA = mul_dn(load_rows(ev.V, s, Vn), load_rows(ev.V, sn, Vn));
+    const M3<double> UB = mul_dn(load_rows(VB, s, Vn), load_rows(VB, sn, Vn));
+    store_alg(ev.comm + (size_t)d * 4 * Vn, s, Vn, icomm(iah_to_alg(UA), iah_to_alg(UB)));
+    M3<double> U;
+    if (solve_link(UA, UB, U)) atomicAdd(ev.bad, 1);
+    store_rows(ev.U64 + (size_t)d * 6 * Vn, s, Vn, U);
 }
 
 template <typename R>
@@ -248,72 +717,102 @@ __device__ __forceinline__ M3<R> to_r(const M3<double>& m) {
     return o;
 }
 
+// pi(-1/2) = E_eta(0) = -sum over the four links at the site of the link's
+// commutator / 2 (the backward ones transported by the Glasma link), phi = e =
+// 0, and the links
 template <typename R>
-__global__ void initial_fields_kernel(const double2* VdA, const double2* VdB, const double2* U64, Fields<R> f,
-                                      int N) {
+__device__ __forceinline__ void initial_site(const InitEv& d, int64_t s) {
+    const int N = d.N;
     const int64_t Vn = (int64_t)N * N;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < Vn; s += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(s % N), y = (int)(s / N);
-        A8<double> pi = a_zero<double>();
-        for (int d = 0; d < 2; d++) {
-            const int64_t sb = d == 0 ? (int64_t)y * N + (x == 0 ? N - 1 : x - 1)
-                                      : (int64_t)(y == 0 ? N - 1 : y - 1) * N + x;
-            for (int k = 0; k < 2; k++) {
-                const int64_t sl = k == 0 ? s : sb;
-                A8<double> a = iah_to_alg(nucleus_link(VdA, d, sl, N, Vn));
-                A8<double> b = iah_to_alg(nucleus_link(VdB, d, sl, N, Vn));
-                for (int c = 0; c < 8; c++) { a.v[c] = -a.v[c]; b.v[c] = -b.v[c]; }  // -i[U]_ah
-                A8<double> c = icomm(a, b);                                          // i[a, b]
-                if (k == 1) c = adj_dag(load_link(U64, d, sb, Vn), c);
-                for (int q = 0; q < 8; q++) pi.v[q] -= 0.5 * c.v[q];
-            }
-        }
-        A8<R> pr, z;
-        for (int a = 0; a < 8; a++) { pr.v[a] = (R)pi.v[a]; z.v[a] = R(0); }
-        store_alg(f.pi, s, Vn, pr);
-        store_alg(f.phi, s, Vn, z);
-        store_alg(f.e, s, Vn, z);
-        store_alg(f.e + (size_t)Prec<R>::AP * Vn, s, Vn, z);
-        for (int d = 0; d < 2; d++) store_link(f.U, d, s, Vn, to_r<R>(load_link(U64, d, s, Vn)));
+    const Fields<R> f = carve_fields<R>(d.fields, Vn);
+    const int x = (int)(s % N), y = (int)(s / N);
+    A8<double> pi = a_zero<double>();
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        const int64_t sb = k == 0 ? (int64_t)y * N + (x == 0 ? N - 1 : x - 1) : (int64_t)(y == 0 ? N - 1 : y - 1) * N + x;
+        const double2* cm = d.comm + (size_t)k * 4 * Vn;
+        const A8<double> c = load_alg(cm, s, Vn);
+        const A8<double> b = conj_dn_t(load_rows(d.U64 + (size_t)k * 6 * Vn, sb, Vn), load_alg(cm, sb, Vn));
+#pragma unroll
+        for (int q = 0; q < 8; q++) pi.v[q] -= 0.5 * (c.v[q] + b.v[q]);
+    }
+    A8<R> pr;
+#pragma unroll
+    for (int a = 0; a < 8; a++) pr.v[a] = (R)pi.v[a];
+    const A8<R> z = a_zero<R>();
+    store_alg(f.pi, s, Vn, pr);
+    store_alg(f.phi, s, Vn, z);
+    store_alg(f.e, s, Vn, z);
+    store_alg(f.e + (size_t)Prec<R>::AP * Vn, s, Vn, z);
+#pragma unroll
+    for (int k = 0; k < 2; k++) store_link(f.U, k, s, Vn, to_r<R>(load_rows(d.U64 + (size_t)k * 6 * Vn, s, Vn)));
+}
+__global__ void __launch_bounds__(128) init_fields_kernel(const InitEv* evs, int ne, InitEv one) {
+    int blk;
+    const InitEv& d = init_find(evs, ne, one, IK_SITES, &blk);
+    const int64_t s = (int64_t)blk * 128 + threadIdx.x;
+    if (s >= (int64_t)d.N * d.N) return;
+    if (d.prec == 0) initial_site<double>(d, s);
+    else initial_site<float>(d, s);
+}
+
+// the blocks of event e in launch k
+static int64_t init_blocks(const InitEv& e, int k) {
+    const int64_t V = (int64_t)e.N * e.N;
+    switch (k) {
+        case IK_TABLES: return (V + INIT_T - 1) / INIT_T;
+        case IK_ROWS: return ((int64_t)8 * e.S * e.N + e.lines - 1) / e.lines;
+        case IK_COLS: return (int64_t)8 * e.S * ((e.N + e.cols - 1) / e.cols);
+        case IK_SHEETS: return (int64_t)2 * e.groups * ((e.N + e.rows - 1) / e.rows);
+        case IK_SITES: return (2 * V + 127) / 128;
+        default: return (2 * V + 63) / 64;
     }
 }
 
-static unsigned grid_for(int64_t n, int threads) {
-    int64_t b = (n + threads - 1) / threads;
-    if (b > 152 * 32) b = 152 * 32;
-    return (unsigned)(b < 1 ? 1 : b);
-}
+bool init_supported(int N) { return N <= INIT_MAX_N; }
 
-int launch_mv_init(int prec, void* buf, void* scratch, int N, int Ns, double g2mu_a, double m_a, double Lambda_a,
-                   uint64_t seed, int* d_bad, cudaStream_t st) {
-    const int64_t Vn = (int64_t)N * N;
-    char* sc = (char*)scratch;
-    double2* rho = (double2*)sc;
-    double2* U64 = (double2*)sc;  // reused after the Wilson lines are complete
-    double2* VdA = (double2*)(sc + init_region0(Vn));
-    double2* VdB = VdA + (size_t)9 * Vn;
-    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-    const double sigma = g2mu_a / sqrt((double)Ns);
-    const int T = 128;
-    for (int nucleus = 0; nucleus < 2; nucleus++) {
-        double2* Vd = nucleus == 0 ? VdA : VdB;
-        set_identity_kernel<<<grid_for(Vn, T), T, 0, st>>>(Vd, Vn);
-        for (int sheet = 0; sheet < Ns; sheet++) {
-            rho_kernel<<<grid_for(Vn, T), T, 0, st>>>(rho, Vn, Ns, nucleus, sheet, sigma, k0, k1);
-            fft2(rho, 8, N, -1, st);
-            green_kernel<<<grid_for(Vn, T), T, 0, st>>>(rho, N, m_a * m_a, Lambda_a > 0 ? Lambda_a * Lambda_a : 0.0,
-                                                          1.0 / (double)Vn);
-            fft2(rho, 8, N, +1, st);
-            wilson_accum_kernel<<<grid_for(Vn, T), T, 0, st>>>(Vd, rho, Vn);
+void init_block_table(InitEv* evs, int ne) {
+    for (int k = 0; k < IK_N; k++) {
+        int64_t b = 0;
+        for (int e = 0; e < ne; e++) {
+            evs[e].begin[k] = (int)b;
+            b += init_blocks(evs[e], k);
         }
     }
-    cudaMemsetAsync(d_bad, 0, sizeof(int), st);
-    glasma_link_kernel<<<grid_for(2 * Vn, 64), 64, 0, st>>>(VdA, VdB, U64, N, d_bad);
-    if (prec == 0)
-        initial_fields_kernel<double><<<grid_for(Vn, T), T, 0, st>>>(VdA, VdB, U64, carve_fields<double>(buf, Vn), N);
-    else
-        initial_fields_kernel<float><<<grid_for(Vn, T), T, 0, st>>>(VdA, VdB, U64, carve_fields<float>(buf, Vn), N);
-    return 0;
+}
+
+void launch_mv_init(const InitEv* h, const InitEv* d_ev, int ne, cudaStream_t st) {
+    const InitEv one = h[0];
+    const InitEv* ev = ne > 1 ? d_ev : nullptr;
+    unsigned nb[IK_N];
+    size_t rows = 0, cols = 0, sheets = 0;
+    int rounds = 1;
+    bool grouped = false;
+    for (int k = 0; k < IK_N; k++) nb[k] = (unsigned)(h[ne - 1].begin[k] + init_blocks(h[ne - 1], k));
+    for (int e = 0; e < ne; e++) {
+        const size_t r = (size_t)h[e].lines * h[e].N * 16, c = (size_t)h[e].cols * (h[e].N + 1) * 16,
+                     s = (size_t)4 * h[e].rows * h[e].N * 16;
+        rows = r > rows ? r : rows;
+        cols = c > cols ? c : cols;
+        sheets = s > sheets ? s : sheets;
+        const int n = (h[e].Ns + h[e].S - 1) / h[e].S;
+        rounds = n > rounds ? n : rounds;
+        grouped = grouped || h[e].groups > 1;
+    }
+    // per-device function attributes; set whenever a launch needs more than the default
+    if (rows > 48 * 1024) cudaFuncSetAttribute(init_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows);
+    if (cols > 48 * 1024) cudaFuncSetAttribute(init_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cols);
+    if (sheets > 48 * 1024)
+        cudaFuncSetAttribute(init_sheets_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sheets);
+    init_tables_kernel<<<nb[IK_TABLES], INIT_T, 0, st>>>(ev, ne, one);
+    for (int r = 0; r < rounds; r++) {
+        init_rows_kernel<<<nb[IK_ROWS], INIT_T, rows, st>>>(ev, ne, one, r);
+        init_cols_kernel<<<nb[IK_COLS], INIT_T, cols, st>>>(ev, ne, one, r);
+        init_sheets_kernel<<<nb[IK_SHEETS], INIT_T, sheets, st>>>(ev, ne, one, r);
+    }
+    if (grouped) init_groups_kernel<<<nb[IK_SITES], 128, 0, st>>>(ev, ne, one);
+    init_links_kernel<<<nb[IK_LINKS], 64, 0, st>>>(ev, ne, one);
+    init_fields_kernel<<<nb[IK_SITES], 128, 0, st>>>(ev, ne, one);
 }
 
 }  // namespace gl

@@ -49,9 +49,31 @@ void launch_push(int prec, const void* site, const void* bn1, void* parts, int64
 void launch_sample(int prec, void* parts, int64_t np, int N, uint64_t seed, const int64_t* offsets, int n_species,
                    const int* rep, const int* mom_mode, const double* p0, const double* p1,
                    const double q0[2][8], cudaStream_t st);
-// MV initial condition into field buffer b (FP64 scratch in `scratch`)
-int launch_mv_init(int prec, void* b, void* scratch, int N, int Ns, double g2mu_a, double m_a, double Lambda_a,
-                   uint64_t seed, int* d_bad, cudaStream_t st);
+// One event's MV initial conditions (init.cu): its parameters, the radices of
+// its line transforms, the split of the work, its scratch and the field slice
+// it fills.  begin[k]: its first block in launch k over several events.
+struct InitEv {
+    static constexpr int KINDS = 6;
+    int N, Ns, prec;
+    int pow2, log2N, nrad, rad[12];
+    int S, groups, per_group;  // sheets a round; groups of sheets multiplied apart
+    int lines, cols, rows;     // lines, columns and rows a block of the three launches takes
+    int begin[KINDS];
+    double sigma, m2, lam2;
+    uint32_t k0, k1;
+    double2 *V, *tw, *work, *U64, *comm;
+    double* green;
+    void* fields;
+    int* bad;                  // links whose matching did not converge
+};
+InitEv init_event(int prec, void* fields, void* scratch, int N, int Ns, double g2mu_a, double m_a, double Lambda_a,
+                  uint64_t seed, int* bad);
+// lattices whose lines fit the transforms
+bool init_supported(int N);
+// begin[] of every event, in order
+void init_block_table(InitEv* evs, int ne);
+// the initial conditions of ne events: h on the host, d_ev the same in device memory (not read for ne = 1)
+void launch_mv_init(const InitEv* h, const InitEv* d_ev, int ne, cudaStream_t st);
 // canonical FP64 <-> device layout conversions (staging buffer is FP64 canonical)
 void launch_parts_convert(int prec, void* parts, int64_t np, double* stg, int to_device, cudaStream_t st);
 // species and original indices of a native particle upload checked and
@@ -59,7 +81,7 @@ void launch_parts_convert(int prec, void* parts, int64_t np, double* stg, int to
 void launch_parts_validate(int prec, void* parts, int64_t np, int ns, int* d_bad, cudaStream_t st);
 // integrated p^tau of the particles <-> canonical [np] in the caller's order
 void launch_ptau_convert(int prec, void* parts, int64_t np, double* stg, int to_device, cudaStream_t st);
-size_t init_scratch_bytes(int64_t Vn);
+size_t init_scratch_bytes(int N, int Ns);
 void launch_convert(int prec, int which, int to_device, void* dev, double* staging, int N, int64_t np,
                     cudaStream_t st);
 // observables: per-species particle sums and field checks, FP64, fixed-order reductions
@@ -159,6 +181,9 @@ size_t site_bytes(int prec, int64_t Vn);
 size_t field_bytes(int prec, int64_t Vn);
 
 // context internals the batch reads and drives (capi.cu)
+InitEv ctx_init_event(const gl_ctx* c, int* bad);
+// after the initial conditions of a context were enqueued on its stream: site fields cleared, step 0
+void ctx_init_done(gl_ctx* c);
 struct CtxView {
     void* field[2];
     void* site[2];
