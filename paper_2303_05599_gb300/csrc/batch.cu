@@ -61,6 +61,7 @@ struct BatchArgs {
     const int64_t* clock;
     int push_chunk;  // particles per push block
     int seg_rows;    // FP32: rows per strip segment
+    int strip_wpb;   // FP32: warps per block of the field launch
 };
 
 // the last event whose first block is <= block (the prefix tables are
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(TX * TY, (Tile<R, TX, TY>::min_blocks)) batch_
     field_item<R, TX, TY>(b, blockIdx.x);
 }
 
-// FP32 field step of the whole batch: blocks of WPB warps take WPB
+// FP32 field step of the whole batch: blocks of up to WPB warps take as many
 // consecutive segments of the flat list per item (nseg segments, `items`
 // items strided over the grid)
 template <int WPB, int MINB>
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(WPB * 32, MINB) batch_strip_kernel(BatchArgs b
     const int64_t n = *b.clock;
     const StripStep a = strip_step(n, b.dt, b.reunit_every);
     for (int it = blockIdx.x; it < items; it += gridDim.x)
-        strip_seg_item(b, S[wib], n, a, (int64_t)it * WPB + wib, nseg);
+        strip_seg_item(b, S[wib], n, a, (int64_t)it * (blockDim.x >> 5) + wib, nseg);
 }
 
 // at most 64 FP32 registers (B threads, 1024 / B blocks per SM): enough
@@ -357,39 +358,36 @@ static void set_smem_attr() {
 // FP32 batch), warps per block x blocks per SM: 0 = 8 x 2 (16 warps per SM at
 // 128 registers), 1 = 12 x 1 (168 registers), 2 = 8 x 1 (255 registers)
 
-// resident blocks of a strip launch shape on this device (the kernel's own
-// occupancy on an idle GPU)
-template <int WPB, int MINB>
-static int batch_strip_blocks() {
-    static int blocks[64] = {};
-    int dev = 0;
+static int sm_count() {
+    int dev = 0, sms = 0;
     cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) dev = 0;
-    if (!blocks[dev]) {
-        const int smem = WPB * (int)sizeof(StripWarpSmem);
-        cudaFuncSetAttribute(batch_strip_kernel<WPB, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        int per_sm = 0, sms = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_strip_kernel<WPB, MINB>, WPB * 32, smem);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        blocks[dev] = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
-    }
-    return blocks[dev];
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms > 0 ? sms : 1;
 }
 
 template <int WPB, int MINB>
 static void launch_strip_shape(int64_t nseg, const BatchArgs& b, cudaStream_t st) {
     if (nseg < 1) return;
-    const int items = (int)((nseg + WPB - 1) / WPB);
-    int grid = batch_strip_blocks<WPB, MINB>();
+    // the dynamic shared-memory limit is a per-device function attribute
+    static bool attr[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr[dev]) {
+        cudaFuncSetAttribute(batch_strip_kernel<WPB, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             WPB * (int)sizeof(StripWarpSmem));
+        attr[dev] = true;
+    }
+    const int wpb = b.strip_wpb < WPB ? b.strip_wpb : WPB;
+    const int items = (int)((nseg + wpb - 1) / wpb);
+    int grid = sm_count() * (WPB * MINB / wpb);
     if (grid > items) grid = items;
-    batch_strip_kernel<WPB, MINB><<<grid, WPB * 32, WPB * sizeof(StripWarpSmem), st>>>(b, nseg, items);
+    batch_strip_kernel<WPB, MINB><<<grid, wpb * 32, wpb * sizeof(StripWarpSmem), st>>>(b, nseg, items);
 }
 
-// warps per block and resident blocks of FP32 strip launch shape `tile`
-static void strip_shape_geometry(int tile, int* wpb, int* blocks) {
-    if (tile == 1) { *wpb = 12; *blocks = batch_strip_blocks<12, 1>(); }
-    else if (tile == 2) { *wpb = 8; *blocks = batch_strip_blocks<8, 1>(); }
-    else { *wpb = 8; *blocks = batch_strip_blocks<8, 2>(); }
+// warps per block and per SM of FP32 strip launch shape `tile`
+static void strip_shape_geometry(int tile, int* wpb, int* warps_sm) {
+    *wpb = tile == 1 ? 12 : 8;
+    *warps_sm = tile == 1 ? 12 : tile == 2 ? 8 : 16;
 }
 
 template <typename R>
@@ -504,11 +502,13 @@ struct gl_batch {
     int field_blocks;      // FP64: tiles of all events
     int64_t field_segs;    // FP32: segments of all events' strips
     int seg_rows;          // FP32: rows per segment, for the current launch shape
+    int strip_wpb;         // FP32: warps per block of its launch
+    int plan_tile, plan_seg;  // the shape and fixed segment length (0: none) the two belong to
     int seg_tuned[N_TILES];  // FP32: the autotuner's segment length per launch shape (0: the cost model's)
     int push_blocks;
     cudaGraph_t graph;
     cudaGraphExec_t exec;
-    int graph_tile, graph_push_block, graph_push_chunk, graph_fused, graph_push_grid;
+    int graph_tile, graph_push_block, graph_push_chunk, graph_fused, graph_push_grid, graph_seg, graph_wpb;
     float tune_field_ms[N_TILES];
     float tune_push_ms[3];
     // trial steps: two streams; fused by push chunk; two streams with 1 and 2
@@ -542,23 +542,22 @@ static gl_status bfail(gl_batch* b, gl_status s, const char* m) {
 }
 
 extern "C" {
-// the strip segment length of the current launch shape: the one set or
-// tuned for it, else the one that spreads all events' strips evenly over its
-// resident warps (0: out of host memory)
-static int batch_seg_rows(const gl_batch* b) {
-    if (b->seg_tuned[b->tile] > 0) return b->seg_tuned[b->tile];
-    int wpb = 8, blocks = 1;
-    strip_shape_geometry(b->tile, &wpb, &blocks);
+// the strip segment length of the current launch shape (the one set or tuned
+// for it, else the one that spreads all events' strips evenly over its resident
+// warps; 0: out of host memory) and the warps a block of its launch
+static StripPlan batch_strip_plan(const gl_batch* b) {
+    int wpb = 8, warps_sm = 8;
+    strip_shape_geometry(b->tile, &wpb, &warps_sm);
     int* Ns = new (std::nothrow) int[b->ne];
-    if (!Ns) return 0;
+    if (!Ns) return StripPlan{0, wpb};
     for (int e = 0; e < b->ne; e++) {
         CtxView v;
         ctx_view(b->ev[e], &v);
         Ns[e] = v.N;
     }
-    const int rows = strip_seg_rows(Ns, b->ne, wpb, blocks);
+    const StripPlan p = strip_plan(Ns, b->ne, wpb, warps_sm, sm_count(), b->seg_tuned[b->tile]);
     delete[] Ns;
-    return rows;
+    return p;
 }
 
 static gl_status sync_desc(gl_batch* b);
@@ -689,6 +688,8 @@ gl_status gl_batch_create(const gl_config* cfgs, const gl_species* species, int3
     }
     b->tile = b->prec == GL_FP64 ? TILE_32x4 : 0;
     b->seg_rows = 16;  // replaced by the first descriptor sync
+    b->strip_wpb = 8;
+    b->plan_tile = -1;
     b->push_block = 128;
     b->push_chunk = PUSH_CHUNK;
     b->fused = 0;
@@ -791,7 +792,13 @@ static gl_status sync_desc(gl_batch* b) {
     const int TX = TILE_DIMS[b->tile][0], TY = TILE_DIMS[b->tile][1];
     int64_t step0 = -1;
     if (b->prec != GL_FP64) {
-        b->seg_rows = batch_seg_rows(b);
+        if (b->plan_tile != b->tile || b->plan_seg != b->seg_tuned[b->tile]) {
+            const StripPlan p = batch_strip_plan(b);
+            b->seg_rows = p.seg;
+            b->strip_wpb = p.wpb;
+            b->plan_tile = b->tile;
+            b->plan_seg = b->seg_tuned[b->tile];
+        }
         if (b->seg_rows < 1) return bfail(b, GL_ERR_ARG, "out of host memory");
     }
     for (int e = 0; e < b->ne; e++) {
@@ -843,20 +850,13 @@ static gl_status sync_desc(gl_batch* b) {
 }
 
 static BatchArgs batch_args(const gl_batch* b, int reunit_every) {
-    return BatchArgs{b->d_desc, b->ne, b->dt, reunit_every, b->d_clock, b->push_chunk, b->seg_rows};
+    return BatchArgs{b->d_desc, b->ne, b->dt, reunit_every, b->d_clock, b->push_chunk, b->seg_rows, b->strip_wpb};
 }
 
 static void launch_field(gl_batch* b, cudaStream_t st) {
     const BatchArgs a = batch_args(b, b->reunit_every);
     if (b->prec == GL_FP64) launch_batch_field<double>(b->tile, b->field_blocks, b->field_segs, a, st);
     else launch_batch_field<float>(b->tile, b->field_blocks, b->field_segs, a, st);
-}
-
-static int sm_count() {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 1;
 }
 
 // the separate push kernel: one block per chunk, or push_grid resident blocks per SM
@@ -934,7 +934,7 @@ gl_status gl_batch_autotune(gl_batch* b, int32_t* tile_out, int32_t* push_block_
             const int more[3] = {16, 2 * m, m / 2};
             cand[0] = m;
             for (int k = 0; k < 3; k++) {
-                bool dup = more[k] < 4;
+                bool dup = more[k] < 1;
                 for (int c = 0; c < nc; c++) dup = dup || cand[c] == more[k];
                 if (!dup) cand[nc++] = more[k];
             }
@@ -1144,7 +1144,8 @@ gl_status gl_batch_step(gl_batch* b, int32_t n_steps) {
     if (b->prec == GL_FP64) set_smem_attr<double, 32, 4>();
     // (re)capture the overlapped step when the launch shapes changed
     if (!b->exec || b->graph_tile != b->tile || b->graph_push_block != b->push_block ||
-        b->graph_push_chunk != b->push_chunk || b->graph_fused != b->fused || b->graph_push_grid != b->push_grid) {
+        b->graph_push_chunk != b->push_chunk || b->graph_fused != b->fused || b->graph_push_grid != b->push_grid ||
+        b->graph_seg != b->seg_rows || b->graph_wpb != b->strip_wpb) {
         if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
         if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
         if (cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
@@ -1160,6 +1161,8 @@ gl_status gl_batch_step(gl_batch* b, int32_t n_steps) {
         b->graph_push_chunk = b->push_chunk;
         b->graph_fused = b->fused;
         b->graph_push_grid = b->push_grid;
+        b->graph_seg = b->seg_rows;
+        b->graph_wpb = b->strip_wpb;
     }
     int64_t now = common_step(b);
     for (int32_t left = n_steps; left > 0;) {
@@ -1452,7 +1455,7 @@ gl_status gl_batch_set_launch(gl_batch* b, int32_t tile, int32_t push_block, int
 
 int32_t gl_batch_segment_rows(const gl_batch* b) {
     if (!b || b->prec == GL_FP64) return 0;
-    return b->desc_valid ? b->seg_rows : batch_seg_rows(b);  // the next launch's, also before it
+    return b->desc_valid ? b->seg_rows : batch_strip_plan(b).seg;  // the next launch's, also before it
 }
 
 gl_status gl_batch_set_segment_rows(gl_batch* b, int32_t rows) {

@@ -342,7 +342,7 @@ gl_status gl_create(const gl_config* cfg, const gl_species* sp, int32_t ns, void
     c->cur = 0;
     c->step = c->pstep = 0;
     site_forget(c);
-    c->tile = 0;
+    c->tile = c->prec == GL_FP32_2ROW ? -1 : 0;  // -1: the default shape, at the first step
     c->seg = 0;
     c->push_block = 128;
     *out = c;
@@ -551,6 +551,10 @@ gl_status gl_set_step(gl_ctx* c, int64_t step) {
 // an uninterrupted one does.
 static void one_field_step(gl_ctx* c, cudaStream_t st) {
     const int every = c->prec == GL_FP32_2ROW ? c->cfg.reunit_every : 0;
+    if (c->tile < 0) {
+        c->tile = strip_default_tile(c->N);
+        c->seg = strip_model_seg(c->N, c->tile);
+    }
     launch_fused_step(c->prec, c->field[c->cur], c->field[1 - c->cur], site_at(c, c->step), c->N, c->step, c->dt,
                       every, c->tile, c->seg, st);
     c->site_time[c->step & 1] = c->step;
@@ -687,7 +691,7 @@ gl_status gl_autotune(gl_ctx* c, int32_t* tile_out, int32_t* push_block_out) {
             const int more[3] = {16, 2 * m, m / 2};
             cand[0] = m;
             for (int j = 0; j < 3; j++) {
-                bool dup = more[j] < 4;
+                bool dup = more[j] < 1;
                 for (int q = 0; q < nc; q++) dup = dup || cand[q] == more[j];
                 if (!dup) cand[nc++] = more[j];
             }

@@ -40,6 +40,8 @@ void launch_fused_step(int prec, void* in, void* out, void* site, int N, int64_t
                        int tile, int seg, cudaStream_t st);
 // the cost model's segment length for an N x N lattice and FP32 launch shape `tile`
 int strip_model_seg(int N, int tile);
+// FP32 launch shape of an event that has not been tuned
+int strip_default_tile(int N);
 // site E, B at t_n from buffer n (U, phi, e(n-1/2), pi(n-1/2)) and buffer n+1 (e, pi at n+1/2)
 void launch_site_fields(int prec, const void* bn, const void* bn1, void* site, int N, double t, cudaStream_t st);
 // Euler + CPIC push of all particles active at t_n (bit s of active_mask)

@@ -30,8 +30,9 @@ static void launch_t(void* in, void* out, void* site, int N, int64_t n, double d
         carve_fields<R>(in, Vn), carve_fields<R>(out, Vn), (typename Prec<R>::V*)site, step_r<R>(a));
 }
 
-// FP32: blocks of WPB warps take WPB consecutive segments of the event's
-// strips per item and run them in step; `items` items strided over the grid
+// FP32: blocks of up to WPB warps take as many consecutive segments of the
+// event's strips per item and run them in step; `items` items strided over the
+// grid
 template <int WPB, int MINB>
 __global__ void __launch_bounds__(WPB * 32, MINB) strip_step_kernel(Fields<float> in, Fields<float> out, float4* site,
                                                                      int N, StripStep a, int items, int seg) {
@@ -40,40 +41,46 @@ __global__ void __launch_bounds__(WPB * 32, MINB) strip_step_kernel(Fields<float
     const int wib = threadIdx.x >> 5;
     const int64_t nseg = strip_segments(N, seg);
     for (int it = blockIdx.x; it < items; it += gridDim.x) {
-        const int64_t j = (int64_t)it * WPB + wib;
+        const int64_t j = (int64_t)it * (blockDim.x >> 5) + wib;
         strip_run_segment(S[wib], in, out, site, N, j < nseg ? j : nseg - 1, j < nseg, a, seg);
     }
 }
 
-// resident blocks of a strip launch shape on this device
-template <int WPB, int MINB>
-static int strip_blocks() {
-    static int blocks[64] = {};
+static int sm_count() {
+    static int sms[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
-    if (!blocks[dev]) {
-        const int smem = WPB * (int)sizeof(StripWarpSmem);
-        cudaFuncSetAttribute(strip_step_kernel<WPB, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        int per_sm = 0, sms = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, strip_step_kernel<WPB, MINB>, WPB * 32, smem);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        blocks[dev] = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
-    }
-    return blocks[dev];
+    if (!sms[dev]) cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
+    return sms[dev] > 0 ? sms[dev] : 1;
+}
+
+// warps a block and warps an SM of FP32 launch shape `tile`
+static void strip_shape(int tile, int* wpb, int* warps_sm) {
+    *wpb = tile == 1 ? 12 : 8;
+    *warps_sm = tile == 1 ? 12 : tile == 2 ? 8 : 16;
 }
 
 template <int WPB, int MINB>
 static void launch_strip(void* in, void* out, void* site, int N, int64_t n, double dt, int every, int seg,
                          cudaStream_t st) {
+    // the dynamic shared-memory limit is a per-device function attribute
+    static bool attr[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !attr[dev]) {
+        cudaFuncSetAttribute(strip_step_kernel<WPB, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             WPB * (int)sizeof(StripWarpSmem));
+        attr[dev] = true;
+    }
     const int64_t Vn = (int64_t)N * N;
-    int grid = strip_blocks<WPB, MINB>();
-    if (seg <= 0) seg = strip_seg_rows(&N, 1, WPB, grid);
-    const int items = (int)((strip_segments(N, seg) + WPB - 1) / WPB);
+    const StripPlan p = strip_plan(&N, 1, WPB, WPB * MINB, sm_count(), seg);
+    const int items = (int)((strip_segments(N, p.seg) + p.wpb - 1) / p.wpb);
+    int grid = sm_count() * (WPB * MINB / p.wpb);
     if (grid > items) grid = items;
-    strip_step_kernel<WPB, MINB><<<grid, WPB * 32, WPB * sizeof(StripWarpSmem), st>>>(
+    strip_step_kernel<WPB, MINB><<<grid, p.wpb * 32, p.wpb * sizeof(StripWarpSmem), st>>>(
         carve_fields<float>(in, Vn), carve_fields<float>(out, Vn), (float4*)site, N, strip_step(n, dt, every), items,
-        seg);
+        p.seg);
 }
 
 void launch_fused_step(int prec, void* in, void* out, void* site, int N, int64_t n, double dt, int reunit_every,
@@ -92,9 +99,15 @@ void launch_fused_step(int prec, void* in, void* out, void* site, int N, int64_t
 }
 
 int strip_model_seg(int N, int tile) {
-    if (tile == 1) return strip_seg_rows(&N, 1, 12, strip_blocks<12, 1>());
-    if (tile == 2) return strip_seg_rows(&N, 1, 8, strip_blocks<8, 1>());
-    return strip_seg_rows(&N, 1, 8, strip_blocks<8, 2>());
+    int wpb, warps_sm;
+    strip_shape(tile, &wpb, &warps_sm);
+    return strip_plan(&N, 1, wpb, warps_sm, sm_count(), 0).seg;
 }
+
+// Launch shape of an event that has not been tuned.  Lattices that leave the
+// SMs with one or two warps a scheduler take the 8-warp shape (203 registers a
+// thread), larger ones the 12-warp shape, which needs three to pay: 256^2 21
+// against 22 us, 1024^2 164 against 158 us.
+int strip_default_tile(int N) { return (int64_t)N * N <= (int64_t)sm_count() * 8 * 32 * 4 ? 2 : 1; }
 
 }  // namespace gl

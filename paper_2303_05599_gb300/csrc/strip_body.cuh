@@ -518,8 +518,8 @@ __device__ __forceinline__ void strip_segment(StripWarpSmem& S, const Fields<flo
 // consecutive segments of the flat list and run them in step (a barrier every
 // second row), read and write the same rows of each plane at the same time.
 // Warps beyond the list repeat its last segment without storing.  The segment
-// length is chosen per launch (below) so that the segments fill the resident
-// warps evenly.
+// length and W are chosen per launch (strip_plan) so that the segments fill the
+// resident warps evenly.
 __host__ __device__ inline int64_t strip_segments(int N, int seg) {
     return (int64_t)((N + STRIP_W - 1) / STRIP_W) * ((N + seg - 1) / seg);
 }
@@ -546,24 +546,44 @@ __device__ __forceinline__ void strip_run_segment(StripWarpSmem& S, const Fields
     strip_segment(S, in, out, site, N, g.x0, g.y0, g.y0 + seg, real ? g.y0 + g.len : g.y0, a, true);
 }
 
-// Segment length for lattices Ns[0..n) on `blocks` resident blocks of `wpb`
-// warps: the length S >= 4 that minimises the modelled time, rounds x (S rows
-// + the dry row + the halo passes), where rounds = the items of wpb segments
-// per resident block, rounded up.  The dry row costs about 0.6 of a row and a
-// halo pass (up to HALO_B rows of the left column) about 0.45.  Long segments
-// cost fewer dry rows and halo passes; short ones fill the last round.
-inline int strip_seg_rows(const int* Ns, int n, int wpb, int blocks) {
+// How a field launch splits the strips: rows a segment and warps a block.
+struct StripPlan {
+    int seg, wpb;
+};
+
+// The split of lattices Ns[0..n) on `sms` SMs for a launch shape of blocks of
+// wpb_max warps, warps_sm warps an SM: the one that minimises the modelled time
+//   rounds x row(w) x (S rows + the dry row + the halo passes)
+// with w the warps of a scheduler in a round.  The dry row costs about 0.6 of a
+// row and a halo pass (up to HALO_B rows of the left column) about 0.45.  A row
+// takes 3.9, 4.2 and 6.0 us with 1, 2 and 3 warps a scheduler (small lattices;
+// measured on 64^2 and 256^2), so lattices that cannot fill the chip spread
+// their segments over as many SMs as there are, down to one row each, in
+// blocks of one warp a scheduler: 64^2 takes 14.4 us in 4-warp blocks of 1-row
+// segments, 38 us in 12-warp blocks of 4-row ones; 256^2 22 us (2 rows)
+// against 43 us.  Full chips take the shape's own blocks, whose warps run in
+// step: separate blocks on one SM stall on instruction fetch, and beyond 8 rows
+// memory sets the time (1024^2 takes 164 us in 4-warp blocks of 27 rows, 147 us
+// in 12-warp blocks of 18).  seg > 0 fixes the segment length.
+inline StripPlan strip_plan(const int* Ns, int n, int wpb_max, int warps_sm, int sms, int seg) {
+    static const double row[4] = {1.0, 1.08, 1.54, 2.05};
     int nmax = 1;
     for (int e = 0; e < n; e++) nmax = Ns[e] > nmax ? Ns[e] : nmax;
-    int best = nmax < 4 ? nmax : 4;
+    StripPlan best = {seg > 0 ? seg : nmax, wpb_max};
     double best_cost = 1e300;
-    for (int S = 4; S <= (nmax > 4 ? nmax : 4); S++) {
+    for (int S = seg > 0 ? seg : 1; S <= (seg > 0 ? seg : nmax); S++) {
         int64_t nseg = 0;
         for (int e = 0; e < n; e++) nseg += strip_segments(Ns[e], S);
-        const int64_t items = (nseg + wpb - 1) / wpb;
-        const int64_t rounds = (items + blocks - 1) / (blocks > 0 ? blocks : 1);
-        const double cost = (double)rounds * (S + 0.6 + 0.45 * ((S + 1 + HALO_B - 1) / HALO_B));
-        if (cost < best_cost - 1e-9) { best_cost = cost; best = S; }
+        for (int k = 0; k < 2; k++) {
+            const int wpb = k ? 4 : wpb_max;
+            const int64_t items = (nseg + wpb - 1) / wpb, per_sm = (items + sms - 1) / sms, res = warps_sm / wpb;
+            const int64_t rounds = (per_sm + res - 1) / res;
+            const int blocks = (int)(per_sm < res ? per_sm : res), w = (blocks * wpb + 3) / 4;
+            if (k && (rounds > 1 || w > 2 || S > 8)) continue;
+            const double cost = (double)rounds * row[w < 4 ? w - 1 : 3] * (k ? 0.9 : 1.0) * (S + 0.6 +
+                                0.45 * ((S + 1 + HALO_B - 1) / HALO_B));
+            if (cost < best_cost - 1e-9) { best_cost = cost; best = StripPlan{S, wpb}; }
+        }
     }
     return best;
 }
