@@ -15,6 +15,9 @@
 #include <math.h>
 #include <string.h>
 
+#include <type_traits>
+
+#include "ff.cuh"
 #include "internal.h"
 #include "layout.cuh"
 #include "philox.cuh"
@@ -37,10 +40,13 @@ namespace gl {
 // direct pass per prime factor; the twiddles come from one table per event.
 //
 // What bounds it: FP64 arithmetic (GB300 issues one FP64 warp instruction per
-// 19 cycles of an SM), so the passes are arranged to do less of it.  Radix-2
+// 19 cycles of an SM), so the passes are arranged to do less of it: radix-2
 // transforms of eight complex planes with a sincospi per butterfly, a
 // 20-term exponential series and whole matrices took 105.7 ms for a 256^2
-// event of 50 sheets, 223 us a transform pass.
+// event of 50 sheets, 223 us a transform pass; these kernels in FP64 16.3 ms.
+// An FP32 event's fields keep 24 bits of the result, so its sheets (variates,
+// transforms, exponentials, products) run on pairs of FP32 values (ff.cuh,
+// about 48 bits) and only the links' matching in FP64.
 //
 // A sheet's planes wait in `work`, as many sheets a round as the scratch holds.
 // Small lattices (all sheets in one round) split each nucleus's product over
@@ -52,6 +58,7 @@ namespace gl {
 static constexpr int INIT_T = 256;                  // threads of the line kernels
 static constexpr int INIT_MAX_N = 3072;             // longest line
 static constexpr int INIT_GEN_OUT = 12;             // outputs a thread of a prime pass: 256 x 12 = 3072 points
+static_assert(sizeof(FFTables) % 16 == 0, "alignment of the tables behind it");
 static constexpr size_t INIT_ROUND_BYTES = (size_t)32 << 20;  // scratch small events may use for more sheets a round
 
 struct InitPlan {
@@ -62,7 +69,7 @@ struct InitPlan {
 static InitPlan init_plan(int N, int Ns) {
     const size_t V = (size_t)N * N;
     InitPlan p;
-    const size_t tw = ((size_t)N * 16 + 255) & ~(size_t)255;
+    const size_t tw = (((size_t)N * 16 + 255) & ~(size_t)255) + sizeof(FFTables);
     // per site: 128 B a sheet (both nuclei), 8 B Green function, 192 B a group
     // (two nuclei's lines as two rows); later 192 B links and 128 B commutators
     // in the place of work and Green function
@@ -127,13 +134,17 @@ InitEv init_event(int prec, void* fields, void* scratch, int N, int Ns, double g
     e.cols = cols_tile(N, e.pow2);
     e.rows = sheet_rows(N);
     e.sigma = g2mu_a / sqrt((double)Ns);
+    const ff sg = ff_of(e.sigma);
+    e.sigma_h = sg.h;
+    e.sigma_l = sg.l;
     e.m2 = m_a * m_a;
     e.lam2 = Lambda_a > 0 ? Lambda_a * Lambda_a : 0.0;
     e.k0 = (uint32_t)seed;
     e.k1 = (uint32_t)(seed >> 32);
     char* s = (char*)scratch;
     e.V = (double2*)(s + p.v);
-    e.tw = (double2*)(s + p.tw);
+    e.normal = (FFTables*)(s + p.tw);
+    e.tw = (double2*)(s + p.tw + sizeof(FFTables));
     e.work = (double2*)(s + p.work);
     e.green = (double*)(s + p.work + (size_t)p.S * 128 * V);
     e.U64 = (double2*)(s + p.work);
@@ -168,36 +179,56 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 w) {
 __device__ __forceinline__ double2 cmulc(double2 a, double2 w) {  // a conj(w)
     return make_double2(fma(a.x, w.x, a.y * w.y), fma(a.y, w.x, -(a.x * w.y)));
 }
-__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ double2 cxy(double x, double y) { return make_double2(x, y); }
+struct __align__(16) ff2 {
+    ff x, y;
+};
+__device__ __forceinline__ ff2 cxy(ff x, ff y) { return ff2{x, y}; }
+__device__ __forceinline__ ff2 cmul(ff2 a, ff2 w) {
+    return ff2{FDot(a.x, w.x).sub(a.y, w.y).get(), FDot(a.x, w.y).add(a.y, w.x).get()};
+}
+__device__ __forceinline__ ff2 cmulc(ff2 a, ff2 w) {
+    return ff2{FDot(a.x, w.x).add(a.y, w.y).get(), FDot(a.y, w.x).sub(a.x, w.y).get()};
+}
+__device__ __forceinline__ ff2 ldg16(const ff2* p) {
+    const float4 v = __ldg((const float4*)p);
+    return ff2{ff{v.x, v.y}, ff{v.z, v.w}};
+}
+__device__ __forceinline__ double2 ldg16(const double2* p) { return __ldg(p); }
+template <typename C>
+__device__ __forceinline__ C cadd(C a, C b) { return cxy(a.x + b.x, a.y + b.y); }
+template <typename C>
+__device__ __forceinline__ C csub(C a, C b) { return cxy(a.x - b.x, a.y - b.y); }
 
 // powers of two: radix 4, and radix 2 on neighbours for odd log2 N
-__device__ __forceinline__ void pow2_radix2(double2* sh, int lines, int ls, int lN) {
+template <typename C>
+__device__ __forceinline__ void pow2_radix2(C* sh, int lines, int ls, int lN) {
     for (int b = threadIdx.x; b < lines << (lN - 1); b += blockDim.x) {
-        double2* p = sh + (b >> (lN - 1)) * ls + 2 * (b & ((1 << (lN - 1)) - 1));
-        const double2 u = p[0], v = p[1];
+        C* p = sh + (b >> (lN - 1)) * ls + 2 * (b & ((1 << (lN - 1)) - 1));
+        const C u = p[0], v = p[1];
         p[0] = cadd(u, v);
         p[1] = csub(u, v);
     }
     __syncthreads();
 }
-__device__ __forceinline__ void pow2_forward(double2* sh, int lines, int ls, int lN, const double2* __restrict__ tw) {
+template <typename C>
+__device__ __forceinline__ void pow2_forward(C* sh, int lines, int ls, int lN, const C* __restrict__ tw) {
     for (int lb = lN; lb >= 2; lb -= 2) {
         const int q = 1 << (lb - 2);
         for (int b = threadIdx.x; b < lines << (lN - 2); b += blockDim.x) {
             const int j = b & ((1 << (lN - 2)) - 1), n = j & (q - 1);
-            double2* p = sh + (b >> (lN - 2)) * ls + ((j >> (lb - 2)) << lb) + n;
-            const double2 a0 = p[0], a1 = p[q], a2 = p[2 * q], a3 = p[3 * q];
-            const double2 t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), t3 = csub(a1, a3);
+            C* p = sh + (b >> (lN - 2)) * ls + ((j >> (lb - 2)) << lb) + n;
+            const C a0 = p[0], a1 = p[q], a2 = p[2 * q], a3 = p[3 * q];
+            const C t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), t3 = csub(a1, a3);
             p[0] = cadd(t0, t2);
             // t1 -+ i t3
-            const double2 y1 = make_double2(t1.x + t3.y, t1.y - t3.x), y2 = csub(t0, t2),
-                          y3 = make_double2(t1.x - t3.y, t1.y + t3.x);
+            const C y1 = cxy(t1.x + t3.y, t1.y - t3.x), y2 = csub(t0, t2),
+                          y3 = cxy(t1.x - t3.y, t1.y + t3.x);
             if (lb > 2) {
                 const int w = n << (lN - lb);
-                p[q] = cmulc(y1, __ldg(tw + w));
-                p[2 * q] = cmulc(y2, __ldg(tw + 2 * w));
-                p[3 * q] = cmulc(y3, __ldg(tw + 3 * w));
+                p[q] = cmulc(y1, ldg16(tw + w));
+                p[2 * q] = cmulc(y2, ldg16(tw + 2 * w));
+                p[3 * q] = cmulc(y3, ldg16(tw + 3 * w));
             } else {
                 p[q] = y1;
                 p[2 * q] = y2;
@@ -208,26 +239,27 @@ __device__ __forceinline__ void pow2_forward(double2* sh, int lines, int ls, int
     }
     if (lN & 1) pow2_radix2(sh, lines, ls, lN);
 }
-__device__ __forceinline__ void pow2_inverse(double2* sh, int lines, int ls, int lN, const double2* __restrict__ tw) {
+template <typename C>
+__device__ __forceinline__ void pow2_inverse(C* sh, int lines, int ls, int lN, const C* __restrict__ tw) {
     if (lN & 1) pow2_radix2(sh, lines, ls, lN);
     for (int lb = 2 + (lN & 1); lb <= lN; lb += 2) {
         const int q = 1 << (lb - 2);
         for (int b = threadIdx.x; b < lines << (lN - 2); b += blockDim.x) {
             const int j = b & ((1 << (lN - 2)) - 1), n = j & (q - 1);
-            double2* p = sh + (b >> (lN - 2)) * ls + ((j >> (lb - 2)) << lb) + n;
-            double2 x1 = p[q], x2 = p[2 * q], x3 = p[3 * q];
-            const double2 x0 = p[0];
+            C* p = sh + (b >> (lN - 2)) * ls + ((j >> (lb - 2)) << lb) + n;
+            C x1 = p[q], x2 = p[2 * q], x3 = p[3 * q];
+            const C x0 = p[0];
             if (lb > 2) {
                 const int w = n << (lN - lb);
-                x1 = cmul(x1, __ldg(tw + w));
-                x2 = cmul(x2, __ldg(tw + 2 * w));
-                x3 = cmul(x3, __ldg(tw + 3 * w));
+                x1 = cmul(x1, ldg16(tw + w));
+                x2 = cmul(x2, ldg16(tw + 2 * w));
+                x3 = cmul(x3, ldg16(tw + 3 * w));
             }
-            const double2 t0 = cadd(x0, x2), t1 = csub(x0, x2), t2 = cadd(x1, x3), t3 = csub(x1, x3);
+            const C t0 = cadd(x0, x2), t1 = csub(x0, x2), t2 = cadd(x1, x3), t3 = csub(x1, x3);
             p[0] = cadd(t0, t2);
-            p[q] = make_double2(t1.x - t3.y, t1.y + t3.x);
+            p[q] = cxy(t1.x - t3.y, t1.y + t3.x);
             p[2 * q] = csub(t0, t2);
-            p[3 * q] = make_double2(t1.x + t3.y, t1.y - t3.x);
+            p[3 * q] = cxy(t1.x + t3.y, t1.y - t3.x);
         }
         __syncthreads();
     }
@@ -236,8 +268,9 @@ __device__ __forceinline__ void pow2_inverse(double2* sh, int lines, int ls, int
 // any N: a direct transform of each prime factor in turn, one output point at
 // a time (a block's points, at most 256 x INIT_GEN_OUT, wait in registers for
 // the barrier before they replace the inputs)
-template <bool FORWARD>
-__device__ void prime_passes(double2* sh, int lines, int ls, const InitEv& d) {
+template <bool FORWARD, typename C>
+__device__ __noinline__ void prime_passes(C* sh, int lines, int ls, const InitEv& d) {
+    const C* tw = (const C*)d.tw;
     const int N = d.N, total = lines * N;
     int B = N;
     if (!FORWARD)
@@ -246,26 +279,26 @@ __device__ void prime_passes(double2* sh, int lines, int ls, const InitEv& d) {
         const int s = FORWARD ? i : d.nrad - 1 - i;
         const int r = d.rad[s], m = B / r;
         const int wr = N / r, wB = N / B;
-        double2 out[INIT_GEN_OUT];
+        C out[INIT_GEN_OUT];
 #pragma unroll
         for (int c = 0; c < INIT_GEN_OUT; c++) {
             const int idx = threadIdx.x + c * INIT_T;
             if (idx < total) {
                 const int line = idx / N, p = idx - line * N, nb = p / B, k = (p - nb * B) / m, n = p % m;
-                const double2* x = sh + line * ls + nb * B + n;
-                double2 a = make_double2(0.0, 0.0);
+                const C* x = sh + line * ls + nb * B + n;
+                C a = {};
                 int w = 0;               // (q k mod r) N / r
                 const int step = k * wr;
                 int tn = 0;              // inverse: n q N / B
                 for (int q = 0; q < r; q++) {
-                    const double2 v = x[q * m];
+                    const C v = x[q * m];
                     if (FORWARD) {
-                        const double2 t = cmulc(v, __ldg(d.tw + w));
+                        const C t = cmulc(v, ldg16(tw + w));
                         a = cadd(a, t);
                     } else {
                         int u = w + tn;
                         if (u >= N) u -= N;
-                        const double2 t = cmul(v, __ldg(d.tw + u));
+                        const C t = cmul(v, ldg16(tw + u));
                         a = cadd(a, t);
                         tn += n * wB;
                         if (tn >= N) tn -= N;
@@ -273,7 +306,7 @@ __device__ void prime_passes(double2* sh, int lines, int ls, const InitEv& d) {
                     w += step;
                     if (w >= N) w -= N;
                 }
-                if (FORWARD) a = cmulc(a, __ldg(d.tw + n * k * wB));
+                if (FORWARD) a = cmulc(a, ldg16(tw + n * k * wB));
                 out[c] = a;
             }
         }
@@ -292,12 +325,14 @@ __device__ void prime_passes(double2* sh, int lines, int ls, const InitEv& d) {
     }
 }
 
-__device__ __forceinline__ void lines_forward(double2* sh, int lines, int ls, const InitEv& d) {
-    if (d.pow2) pow2_forward(sh, lines, ls, d.log2N, d.tw);
+template <typename C>
+__device__ __forceinline__ void lines_forward(C* sh, int lines, int ls, const InitEv& d) {
+    if (d.pow2) pow2_forward(sh, lines, ls, d.log2N, (const C*)d.tw);
     else prime_passes<true>(sh, lines, ls, d);
 }
-__device__ __forceinline__ void lines_inverse(double2* sh, int lines, int ls, const InitEv& d) {
-    if (d.pow2) pow2_inverse(sh, lines, ls, d.log2N, d.tw);
+template <typename C>
+__device__ __forceinline__ void lines_inverse(C* sh, int lines, int ls, const InitEv& d) {
+    if (d.pow2) pow2_inverse(sh, lines, ls, d.log2N, (const C*)d.tw);
     else
         for (int l = 0; l < lines;) {  // at most INIT_T x INIT_GEN_OUT points at a time
             int c = INIT_T * INIT_GEN_OUT / d.N;
@@ -332,8 +367,13 @@ __global__ void __launch_bounds__(INIT_T) init_tables_kernel(const InitEv* evs, 
     if (s < N) {
         double sn, cs;
         sincospi(2.0 * (double)s / (double)N, &sn, &cs);
-        d.tw[s] = make_double2(cs, sn);
+        if (d.prec == 0) {
+            d.tw[s] = make_double2(cs, sn);
+        } else {
+            ((ff2*)d.tw)[s] = ff2{ff_of(cs), ff_of(sn)};
+        }
     }
+    if (d.prec != 0 && s < FF_ANGLES) ff_table_entry(d.normal, (int)s);
     if (s < Vn) {
         const int px = (int)(s % N), py = (int)(s / N);
         const int kx = line_frequency(d, px), ky = line_frequency(d, py);
@@ -342,66 +382,93 @@ __global__ void __launch_bounds__(INIT_T) init_tables_kernel(const InitEv* evs, 
         double g = 1.0 / (k2 + d.m2);
         if (kx == 0 && ky == 0) g = 0.0;
         if (d.lam2 > 0 && k2 > d.lam2) g = 0.0;
-        d.green[s] = g * (1.0 / (double)Vn);
+        g *= 1.0 / (double)Vn;
+        if (d.prec == 0) d.green[s] = g;
+        else ((ff*)d.green)[s] = ff_of(g);
     }
 }
 
+// two independent normal variates of standard deviation sigma
+__device__ __forceinline__ double2 normal_pair(const InitEv& d, uint32_t w1, uint32_t w2, double2*) {
+    double z0, z1;
+    box_muller(u01(w1), u01(w2), z0, z1);
+    return make_double2(d.sigma * z0, d.sigma * z1);
+}
+__device__ __forceinline__ ff2 normal_pair(const InitEv& d, uint32_t w1, uint32_t w2, ff2*) {
+    ff z0, z1;
+    ff_box_muller(w1, w2, d.normal, z0, z1);
+    const ff sigma{d.sigma_h, d.sigma_l};
+    return ff2{sigma * z0, sigma * z1};
+}
+
+// Blocks per SM of a line kernel: FP64 is bound by its pipe, which four warps
+// fill; pairs are bound by latency and take as many registers as the compiler
+// is given (2, 2 and 1 blocks of the three kernels without a cap, 5.4 ms a
+// 256^2 event; 4, 4 and 2 take 4.7 ms in spite of a few spills, 3, 3 and 3 5.8 ms).
+template <typename C>
+constexpr int line_blocks(int n) { return std::is_same<C, ff2>::value ? n : 1; }
+
 // rho of d.lines lattice rows of one or two planes and their forward transforms
-__global__ void __launch_bounds__(INIT_T) init_rows_kernel(const InitEv* evs, int ne, InitEv one, int round) {
-    extern __shared__ __align__(16) unsigned char init_smem[];
-    double2* sh = (double2*)init_smem;
-    int blk;
-    const InitEv& d = init_find(evs, ne, one, IK_ROWS, &blk);
+template <typename C>
+__device__ __forceinline__ void init_rows(const InitEv& d, int blk, int round, C* sh) {
     const int N = d.N, S = d.S;
     const int64_t all = (int64_t)2 * S * 4 * N, line0 = (int64_t)blk * d.lines;
     const int nl = (int)(all - line0 < d.lines ? all - line0 : d.lines);
+    // nothing to do beyond the last sheet (the other events of a batch may go on)
+    const int slot0 = (int)(line0 / (4 * (int64_t)N)), slot1 = (int)((line0 + nl - 1) / (4 * (int64_t)N));
+    if (round * S + slot0 % S >= d.Ns && round * S + slot1 % S >= d.Ns && slot1 - slot0 < 2) return;
     for (int idx = threadIdx.x; idx < nl * N; idx += INIT_T) {
         const int l = idx / N, x = idx - l * N;
         const int64_t line = line0 + l;
         const int row = (int)(line % N), plane = (int)(line / N) & 3, slot = (int)(line / (4 * (int64_t)N));
         const int nucleus = slot / S, sheet = round * S + slot - nucleus * S;
-        double2 z = make_double2(0.0, 0.0);
+        C z = {};
         if (sheet < d.Ns) {
             const U4 w = philox4x32_10(U4{(uint32_t)(row * N + x), (uint32_t)((nucleus * d.Ns + sheet) * 2 + (plane >> 1)),
                                           1u, 0u}, d.k0, d.k1);
-            double z0, z1;
-            box_muller(u01((plane & 1) ? w.z : w.x), u01((plane & 1) ? w.w : w.y), z0, z1);
-            z = make_double2(d.sigma * z0, d.sigma * z1);
+            z = normal_pair(d, (plane & 1) ? w.z : w.x, (plane & 1) ? w.w : w.y, (C*)nullptr);
         }
         sh[idx] = z;
     }
     __syncthreads();
     lines_forward(sh, nl, N, d);
-    double2* out = d.work + (size_t)line0 * N;  // work[slot][plane][row][position]
+    C* out = (C*)d.work + (size_t)line0 * N;  // work[slot][plane][row][position]
     for (int idx = threadIdx.x; idx < nl * N; idx += INIT_T) out[idx] = sh[idx];
+}
+template <typename C>
+__global__ void __launch_bounds__(INIT_T, line_blocks<C>(4)) init_rows_kernel(const InitEv* evs, int ne, InitEv one, int round) {
+    extern __shared__ __align__(16) unsigned char init_smem[];
+    int blk;
+    const InitEv& d = init_find(evs, ne, one, IK_ROWS, &blk);
+    init_rows<C>(d, blk, round, (C*)init_smem);
 }
 
 // alpha = rho / (k^2 + m^2) along the columns of one plane
-__global__ void __launch_bounds__(INIT_T) init_cols_kernel(const InitEv* evs, int ne, InitEv one, int round) {
+template <typename C>
+__global__ void __launch_bounds__(INIT_T, line_blocks<C>(4)) init_cols_kernel(const InitEv* evs, int ne, InitEv one, int round) {
+    using R = decltype(C::x);
     extern __shared__ __align__(16) unsigned char init_smem[];
-    double2* sh = (double2*)init_smem;
+    C* sh = (C*)init_smem;
     int blk;
     const InitEv& d = init_find(evs, ne, one, IK_COLS, &blk);
-    const int N = d.N, S = d.S, C = d.cols, ls = N + 1;  // a point of padding: neighbouring columns in other banks
-    const int nt = (N + C - 1) / C;
-    const int c0 = (blk % nt) * C, sp = blk / nt, slot = sp >> 2;
+    const int N = d.N, S = d.S, ls = N + 1;  // a point of padding: neighbouring columns in other banks
+    const int nt = (N + d.cols - 1) / d.cols;
+    const int c0 = (blk % nt) * d.cols, sp = blk / nt, slot = sp >> 2;
     if (round * S + slot % S >= d.Ns) return;
-    const int nc = N - c0 < C ? N - c0 : C;
-    double2* w = d.work + (size_t)sp * N * N + c0;
+    const int nc = N - c0 < d.cols ? N - c0 : d.cols;
+    C* w = (C*)d.work + (size_t)sp * N * N + c0;
     for (int idx = threadIdx.x; idx < nc * N; idx += INIT_T) {
         const int r = idx / nc, c = idx - r * nc;
         sh[c * ls + r] = w[(size_t)r * N + c];
     }
     __syncthreads();
     lines_forward(sh, nc, ls, d);
-    const double* g = d.green + c0;
+    const R* g = (const R*)d.green + c0;
     for (int idx = threadIdx.x; idx < nc * N; idx += INIT_T) {
         const int r = idx / nc, c = idx - r * nc;
-        const double f = g[(size_t)r * N + c];
-        double2 v = sh[c * ls + r];
-        v.x *= f;
-        v.y *= f;
-        sh[c * ls + r] = v;
+        const R f = g[(size_t)r * N + c];
+        const C v = sh[c * ls + r];
+        sh[c * ls + r] = cxy(v.x * f, v.y * f);
     }
     __syncthreads();
     lines_inverse(sh, nc, ls, d);
@@ -427,6 +494,35 @@ __device__ __forceinline__ void store_rows(double2* V, int64_t s, int64_t Vn, co
 #pragma unroll
     for (int k = 0; k < 6; k++) V[(size_t)k * Vn + s] = make_double2(m.re[k / 3][k % 3], m.im[k / 3][k % 3]);
 }
+__device__ __forceinline__ M3ff load_rows(const ff2* V, int64_t s, int64_t Vn) {  // row 2 is left alone
+    M3ff m;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        const ff2 v = V[(size_t)k * Vn + s];
+        m.re[k / 3][k % 3] = v.x;
+        m.im[k / 3][k % 3] = v.y;
+    }
+    return m;
+}
+__device__ __forceinline__ void store_rows(ff2* V, int64_t s, int64_t Vn, const M3ff& m) {
+#pragma unroll
+    for (int k = 0; k < 6; k++) V[(size_t)k * Vn + s] = ff2{m.re[k / 3][k % 3], m.im[k / 3][k % 3]};
+}
+// a line kept as pairs, in FP64
+__device__ __forceinline__ M3<double> load_line(const InitEv& d, const double2* V, int64_t s, int64_t Vn) {
+    if (d.prec == 0) return load_rows(V, s, Vn);
+    const M3ff f = load_rows((const ff2*)V, s, Vn);
+    M3<double> m;
+#pragma unroll
+    for (int k = 0; k < 6; k++) {
+        m.re[k / 3][k % 3] = to_double(f.re[k / 3][k % 3]);
+        m.im[k / 3][k % 3] = to_double(f.im[k / 3][k % 3]);
+    }
+    rebuild_row2(m);
+    return m;
+}
+__device__ __forceinline__ M3<double> sheet_exp(const A8<double>& al) { return exp_i_alg<double>(al, 1.0); }
+__device__ __forceinline__ M3ff sheet_exp(const A8<ff>& al) { return ff_exp_i(al.v); }
 // (rows 0 and 1 of) v m
 __device__ __forceinline__ M3<double> mul_rows(const M3<double>& v, const M3<double>& m) {
     M3<double> c = m_zero<double>();
@@ -443,12 +539,15 @@ __device__ __forceinline__ M3<double> mul_rows(const M3<double>& v, const M3<dou
             }
     return c;
 }
+__device__ __forceinline__ M3ff mul_rows(const M3ff& v, const M3ff& m) { return ff_mul<2>(v, m); }
 
 // the inverse transforms of d.rows rows of a nucleus and the product over its
 // sheets of this round (of one group of them)
-__global__ void __launch_bounds__(INIT_T) init_sheets_kernel(const InitEv* evs, int ne, InitEv one, int round) {
+template <typename C>
+__global__ void __launch_bounds__(INIT_T, line_blocks<C>(2)) init_sheets_kernel(const InitEv* evs, int ne, InitEv one, int round) {
+    using R = decltype(C::x);
     extern __shared__ __align__(16) unsigned char init_smem[];
-    double2* sh = (double2*)init_smem;
+    C* sh = (C*)init_smem;
     int blk;
     const InitEv& d = init_find(evs, ne, one, IK_SHEETS, &blk);
     const int N = d.N, S = d.S;
@@ -460,9 +559,9 @@ __global__ void __launch_bounds__(INIT_T) init_sheets_kernel(const InitEv* evs, 
     int s0 = round * S, s1 = s0 + S < d.Ns ? s0 + S : d.Ns;
     if (s0 < first) s0 = first;
     if (s1 > first + d.per_group) s1 = first + d.per_group;
-    double2* V = d.V + (size_t)(nucleus * d.groups + g) * 6 * Vn + (int64_t)r0 * N;
+    C* V = (C*)d.V + (size_t)(nucleus * d.groups + g) * 6 * Vn + (int64_t)r0 * N;
     for (int s = s0; s < s1; s++) {
-        const double2* w = d.work + (size_t)(nucleus * S + s - round * S) * 4 * Vn + (int64_t)r0 * N;
+        const C* w = (const C*)d.work + (size_t)(nucleus * S + s - round * S) * 4 * Vn + (int64_t)r0 * N;
         for (int idx = threadIdx.x; idx < 4 * np; idx += INIT_T) {
             const int p = idx / np;
             sh[idx] = w[(size_t)p * Vn + idx - p * np];
@@ -470,14 +569,14 @@ __global__ void __launch_bounds__(INIT_T) init_sheets_kernel(const InitEv* evs, 
         __syncthreads();
         lines_inverse(sh, 4 * nr, N, d);
         for (int i = threadIdx.x; i < np; i += INIT_T) {
-            A8<double> al;
+            A8<R> al;
 #pragma unroll
             for (int p = 0; p < 4; p++) {
-                const double2 v = sh[p * np + i];
+                const C v = sh[p * np + i];
                 al.v[2 * p] = -v.x;
                 al.v[2 * p + 1] = -v.y;
             }
-            const M3<double> e = exp_i_alg<double>(al, 1.0);
+            const auto e = sheet_exp(al);
             // only this thread reads and writes the site's line, sheet after sheet
             if (s == first) store_rows(V, i, Vn, e);
             else store_rows(V, i, Vn, mul_rows(load_rows(V, i, Vn), e));
@@ -494,14 +593,34 @@ __global__ void __launch_bounds__(128) init_groups_kernel(const InitEv* evs, int
     if (d.groups < 2 || t >= 2 * Vn) return;
     const int64_t s = t % Vn;
     double2* V = d.V + (size_t)(t / Vn) * d.groups * 6 * Vn;
-    M3<double> v = load_rows(V, s, Vn);
-    for (int g = 1; g < d.groups; g++) v = mul_rows(v, load_rows(V + (size_t)g * 6 * Vn, s, Vn));
-    store_rows(V, s, Vn, v);
+    if (d.prec == 0) {
+        M3<double> v = load_rows(V, s, Vn);
+        for (int g = 1; g < d.groups; g++) v = mul_rows(v, load_rows(V + (size_t)g * 6 * Vn, s, Vn));
+        store_rows(V, s, Vn, v);
+    } else {
+        ff2* W = (ff2*)V;
+        M3ff v = load_rows(W, s, Vn);
+        for (int g = 1; g < d.groups; g++) {
+            M3ff m = load_rows(W + (size_t)g * 6 * Vn, s, Vn);
+            // row 2: the conjugate cross product of rows 0 and 1
+#pragma unroll
+            for (int j = 0; j < 3; j++) {
+                const int p = (j + 1) % 3, q = (j + 2) % 3;
+                m.re[2][j] = FDot(m.re[0][p], m.re[1][q]).sub(m.im[0][p], m.im[1][q]).sub(m.re[0][q], m.re[1][p])
+                                 .add(m.im[0][q], m.im[1][p]).get();
+                m.im[2][j] = -FDot(m.re[0][p], m.im[1][q]).add(m.im[0][p], m.re[1][q]).sub(m.re[0][q], m.im[1][p])
+                                 .sub(m.im[0][q], m.re[1][p]).get();
+            }
+            v = mul_rows(v, m);
+        }
+        store_rows(W, s, Vn, v);
+    }
 }
 
 // Im tr(T^a M)
-__device__ __forceinline__ void im_tr_T(const M3<double>& M, double* f) {
-    const double h = 0.5, s3 = 0.5 * inv_sqrt3<double>();
+template <typename R>
+__device__ __forceinline__ void im_tr_T(const M3<R>& M, R* f) {
+    const R h = R(0.5), s3 = R(0.5) * inv_sqrt3<R>();
     f[0] = h * (M.im[1][0] + M.im[0][1]);
     f[1] = h * (M.re[0][1] - M.re[1][0]);
     f[2] = h * (M.im[0][0] - M.im[1][1]);
@@ -509,11 +628,12 @@ __device__ __forceinline__ void im_tr_T(const M3<double>& M, double* f) {
     f[4] = h * (M.re[0][2] - M.re[2][0]);
     f[5] = h * (M.im[2][1] + M.im[1][2]);
     f[6] = h * (M.re[1][2] - M.re[2][1]);
-    f[7] = s3 * (M.im[0][0] + M.im[1][1] - 2 * M.im[2][2]);
+    f[7] = s3 * (M.im[0][0] + M.im[1][1] - R(2) * M.im[2][2]);
 }
 // Re tr(T^a M)
-__device__ __forceinline__ void re_tr_T(const M3<double>& M, double* f) {
-    const double h = 0.5, s3 = 0.5 * inv_sqrt3<double>();
+template <typename R>
+__device__ __forceinline__ void re_tr_T(const M3<R>& M, R* f) {
+    const R h = R(0.5), s3 = R(0.5) * inv_sqrt3<R>();
     f[0] = h * (M.re[1][0] + M.re[0][1]);
     f[1] = h * (M.im[1][0] - M.im[0][1]);
     f[2] = h * (M.re[0][0] - M.re[1][1]);
@@ -521,7 +641,7 @@ __device__ __forceinline__ void re_tr_T(const M3<double>& M, double* f) {
     f[4] = h * (M.im[2][0] - M.im[0][2]);
     f[5] = h * (M.re[2][1] + M.re[1][2]);
     f[6] = h * (M.im[2][1] - M.im[1][2]);
-    f[7] = s3 * (M.re[0][0] + M.re[1][1] - 2 * M.re[2][2]);
+    f[7] = s3 * (M.re[0][0] + M.re[1][1] - R(2) * M.re[2][2]);
 }
 
 // Jacobian of F^a = Im tr T^a (W + K), K = W U^+, under U -> exp(i x.T) U:
@@ -529,19 +649,20 @@ __device__ __forceinline__ void re_tr_T(const M3<double>& M, double* f) {
 // J_ab = -(delta_ab Re tr K / 6 + d_abc r^c / 2 + f_abc i^c / 2) for tr(T^c K)
 // = r^c + i i^c: the sixteen independent d and nine f, instead of eight
 // matrix products.
-__device__ __forceinline__ void match_jacobian(const M3<double>& K, double J[8][8]) {
-    double r[8], q[8];
+template <typename R>
+__device__ __forceinline__ void match_jacobian(const M3<R>& K, R J[8][8]) {
+    R r[8], q[8];
     re_tr_T(K, r);
     im_tr_T(K, q);
-    const double t = -(K.re[0][0] + K.re[1][1] + K.re[2][2]) * (1.0 / 6.0);
-    const double h = 0.25, s3 = 0.5 * inv_sqrt3<double>();  // d / 2 for d = 1/2, 1/sqrt 3
-    const double fh = 0.25, fs = 0.43301270189221932338;    // f / 2 for f = 1/2, sqrt(3)/2
+    const R t = -(K.re[0][0] + K.re[1][1] + K.re[2][2]) * R(1.0 / 6.0);
+    const R h = R(0.25), s3 = R(0.5) * inv_sqrt3<R>();  // d / 2 for d = 1/2, 1/sqrt 3
+    const R fh = R(0.25), fs = R(0.43301270189221932338);    // f / 2 for f = 1/2, sqrt(3)/2
 #pragma unroll
     for (int a = 0; a < 8; a++)
 #pragma unroll
-        for (int b = 0; b < 8; b++) J[a][b] = 0.0;
+        for (int b = 0; b < 8; b++) J[a][b] = R(0);
     // diagonal: delta term and d_aac r^c
-    const double e8 = s3 * r[7], h8 = 0.5 * e8, h3 = h * r[2];
+    const R e8 = s3 * r[7], h8 = R(0.5) * e8, h3 = h * r[2];
     J[0][0] = J[1][1] = J[2][2] = t - e8;
     J[3][3] = J[4][4] = t - h3 + h8;
     J[5][5] = J[6][6] = t + h3 + h8;
@@ -554,28 +675,28 @@ __device__ __forceinline__ void match_jacobian(const M3<double>& K, double J[8][
     GL_D(1, 4, h * r[5]); GL_D(1, 5, h * r[4]); GL_D(4, 5, h * r[1]);            // d256
     GL_D(2, 3, h * r[3]); GL_D(2, 4, h * r[4]);                                  // d344 d355
     GL_D(2, 5, -h * r[5]); GL_D(2, 6, -h * r[6]);                                // d366 d377
-    const double m8 = 0.5 * s3;
+    const R m8 = R(0.5) * s3;
     GL_D(3, 7, -m8 * r[3]); GL_D(4, 7, -m8 * r[4]); GL_D(5, 7, -m8 * r[5]); GL_D(6, 7, -m8 * r[6]);  // d448..d778
 #undef GL_D
 #define GL_F(a, b, c, v)                             \
     {                                                \
-        const double va = (v) * q[a], vb = (v) * q[b], vc = (v) * q[c]; \
+        const R va = (v) * q[a], vb = (v) * q[b], vc = (v) * q[c]; \
         J[a][b] -= vc; J[b][a] += vc;                \
         J[b][c] -= va; J[c][b] += va;                \
         J[c][a] -= vb; J[a][c] += vb;                \
     }
-    GL_F(0, 1, 2, 0.5);
+    GL_F(0, 1, 2, R(0.5));
     GL_F(0, 3, 6, fh); GL_F(0, 4, 5, -fh); GL_F(1, 3, 5, fh); GL_F(1, 4, 6, fh); GL_F(2, 3, 4, fh);
     GL_F(2, 5, 6, -fh);
     GL_F(3, 4, 7, fs); GL_F(5, 6, 7, fs);
 #undef GL_F
 }
 
-// J x = b with row exchanges (the links with a small leading pivot), 1 if singular
-__device__ __noinline__ int solve8_pivot(const double* J8, double* b) {
+// the step in FP64 with row exchanges, 1 if J is singular
+__device__ __noinline__ int match_step_pivot(const M3<double>& K, const double* F, double* b) {
     double J[8][8];
-    for (int r = 0; r < 8; r++)
-        for (int c = 0; c < 8; c++) J[r][c] = J8[8 * r + c];
+    match_jacobian(K, J);
+    for (int c = 0; c < 8; c++) b[c] = -F[c];
     for (int c = 0; c < 8; c++) {
         int p = c;
         for (int r = c + 1; r < 8; r++) if (fabs(J[r][c]) > fabs(J[p][c])) p = r;
@@ -597,48 +718,45 @@ __device__ __noinline__ int solve8_pivot(const double* J8, double* b) {
     return 0;
 }
 
-// the Newton step dx = -J^-1 F at K.  J is close to -1 for links near the
-// unit matrix, so the elimination runs in its own order, in registers; where a
-// pivot falls below 1/16 of the diagonal's scale it is done again with row
-// exchanges
+// The Newton step dx = -J^-1 F at K.  Its direction needs no more than FP32: an
+// error of 1e-6 in it leaves 1e-6 of the residual, where the iteration's own
+// square would leave less only in its last step, so the Jacobian and its
+// elimination (half of the operations of an iteration) run on the FP32 pipe
+// and the residual, the step's exponential and the link in FP64.  J is close
+// to -1 for links near the unit matrix, so the elimination runs in its own
+// order, in registers; where a pivot falls below 1/16 of the diagonal's scale
+// it is done again in FP64 with row exchanges.
 __device__ __forceinline__ int match_step(const M3<double>& K, const double* F, double* x) {
-    double J[8][8];
-    match_jacobian(K, J);
+    float J[8][8], y[8], inv[8];
+    M3<float> Kf;
 #pragma unroll
-    for (int a = 0; a < 8; a++) x[a] = -F[a];
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) { Kf.re[i][j] = (float)K.re[i][j]; Kf.im[i][j] = (float)K.im[i][j]; }
+    match_jacobian(Kf, J);
+#pragma unroll
+    for (int a = 0; a < 8; a++) y[a] = -(float)F[a];
     bool small = false;
-    double inv[8];
 #pragma unroll
     for (int c = 0; c < 8; c++) {
-        small = small || !(fabs(J[c][c]) > 0.0625);
-        inv[c] = 1.0 / J[c][c];
+        small = small || !(fabsf(J[c][c]) > 0.0625f);
+        inv[c] = 1.0f / J[c][c];
 #pragma unroll
         for (int r = c + 1; r < 8; r++) {
-            const double f = J[r][c] * inv[c];
+            const float f = J[r][c] * inv[c];
 #pragma unroll
-            for (int k = c + 1; k < 8; k++) J[r][k] = fma(-f, J[c][k], J[r][k]);
-            x[r] = fma(-f, x[c], x[r]);
+            for (int k = c + 1; k < 8; k++) J[r][k] = fmaf(-f, J[c][k], J[r][k]);
+            y[r] = fmaf(-f, y[c], y[r]);
         }
     }
 #pragma unroll
     for (int c = 7; c >= 0; c--) {
 #pragma unroll
-        for (int k = c + 1; k < 8; k++) x[c] = fma(-J[c][k], x[k], x[c]);
-        x[c] *= inv[c];
+        for (int k = c + 1; k < 8; k++) y[c] = fmaf(-J[c][k], y[k], y[c]);
+        y[c] *= inv[c];
+        x[c] = (double)y[c];
     }
-    if (!small) return 0;
-    double Jp[64], b[8];
-    match_jacobian(K, J);
-#pragma unroll
-    for (int a = 0; a < 8; a++) {
-        b[a] = -F[a];
-#pragma unroll
-        for (int k = 0; k < 8; k++) Jp[8 * a + k] = J[a][k];
-    }
-    const int bad = solve8_pivot(Jp, b);
-#pragma unroll
-    for (int a = 0; a < 8; a++) x[a] = b[a];
-    return bad;
+    return small ? match_step_pivot(K, F, x) : 0;
 }
 
 // F^a = Im tr T^a (W + K), K = W U^+, and its largest entry
@@ -701,8 +819,8 @@ __global__ void __launch_bounds__(64) init_links_kernel(const InitEv* evs, int n
     const int x = (int)(s % N), y = (int)(s / N);
     const int64_t sn = d == 0 ? (int64_t)y * N + (x + 1 == N ? 0 : x + 1) : (int64_t)(y + 1 == N ? 0 : y + 1) * N + x;
     const double2* VB = ev.V + (size_t)ev.groups * 6 * Vn;
-    const M3<double> UA = mul_dn(load_rows(ev.V, s, Vn), load_rows(ev.V, sn, Vn));
-    const M3<double> UB = mul_dn(load_rows(VB, s, Vn), load_rows(VB, sn, Vn));
+    const M3<double> UA = mul_dn(load_line(ev, ev.V, s, Vn), load_line(ev, ev.V, sn, Vn));
+    const M3<double> UB = mul_dn(load_line(ev, VB, s, Vn), load_line(ev, VB, sn, Vn));
     store_alg(ev.comm + (size_t)d * 4 * Vn, s, Vn, icomm(iah_to_alg(UA), iah_to_alg(UB)));
     M3<double> U;
     if (solve_link(UA, UB, U)) atomicAdd(ev.bad, 1);
@@ -760,7 +878,7 @@ __global__ void __launch_bounds__(128) init_fields_kernel(const InitEv* evs, int
 static int64_t init_blocks(const InitEv& e, int k) {
     const int64_t V = (int64_t)e.N * e.N;
     switch (k) {
-        case IK_TABLES: return (V + INIT_T - 1) / INIT_T;
+        case IK_TABLES: return ((V > FF_ANGLES ? V : FF_ANGLES) + INIT_T - 1) / INIT_T;
         case IK_ROWS: return ((int64_t)8 * e.S * e.N + e.lines - 1) / e.lines;
         case IK_COLS: return (int64_t)8 * e.S * ((e.N + e.cols - 1) / e.cols);
         case IK_SHEETS: return (int64_t)2 * e.groups * ((e.N + e.rows - 1) / e.rows);
@@ -778,6 +896,22 @@ void init_block_table(InitEv* evs, int ne) {
             evs[e].begin[k] = (int)b;
             b += init_blocks(evs[e], k);
         }
+    }
+}
+
+template <typename C>
+static void launch_sheets(const unsigned* nb, size_t rows, size_t cols, size_t sheets, int rounds, const InitEv* ev,
+                          int ne, const InitEv& one, cudaStream_t st) {
+    // per-device function attributes; set whenever a launch needs more than the default
+    const size_t most = 48 * 1024;
+    if (rows > most) cudaFuncSetAttribute(init_rows_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows);
+    if (cols > most) cudaFuncSetAttribute(init_cols_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cols);
+    if (sheets > most)
+        cudaFuncSetAttribute(init_sheets_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sheets);
+    for (int r = 0; r < rounds; r++) {
+        init_rows_kernel<C><<<nb[IK_ROWS], INIT_T, rows, st>>>(ev, ne, one, r);
+        init_cols_kernel<C><<<nb[IK_COLS], INIT_T, cols, st>>>(ev, ne, one, r);
+        init_sheets_kernel<C><<<nb[IK_SHEETS], INIT_T, sheets, st>>>(ev, ne, one, r);
     }
 }
 
@@ -799,17 +933,10 @@ void launch_mv_init(const InitEv* h, const InitEv* d_ev, int ne, cudaStream_t st
         rounds = n > rounds ? n : rounds;
         grouped = grouped || h[e].groups > 1;
     }
-    // per-device function attributes; set whenever a launch needs more than the default
-    if (rows > 48 * 1024) cudaFuncSetAttribute(init_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows);
-    if (cols > 48 * 1024) cudaFuncSetAttribute(init_cols_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cols);
-    if (sheets > 48 * 1024)
-        cudaFuncSetAttribute(init_sheets_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sheets);
     init_tables_kernel<<<nb[IK_TABLES], INIT_T, 0, st>>>(ev, ne, one);
-    for (int r = 0; r < rounds; r++) {
-        init_rows_kernel<<<nb[IK_ROWS], INIT_T, rows, st>>>(ev, ne, one, r);
-        init_cols_kernel<<<nb[IK_COLS], INIT_T, cols, st>>>(ev, ne, one, r);
-        init_sheets_kernel<<<nb[IK_SHEETS], INIT_T, sheets, st>>>(ev, ne, one, r);
-    }
+    // the events of a launch have one precision
+    if (one.prec == 0) launch_sheets<double2>(nb, rows, cols, sheets, rounds, ev, ne, one, st);
+    else launch_sheets<ff2>(nb, rows, cols, sheets, rounds, ev, ne, one, st);
     if (grouped) init_groups_kernel<<<nb[IK_SITES], 128, 0, st>>>(ev, ne, one);
     init_links_kernel<<<nb[IK_LINKS], 64, 0, st>>>(ev, ne, one);
     init_fields_kernel<<<nb[IK_SITES], 128, 0, st>>>(ev, ne, one);

@@ -51,6 +51,7 @@ void launch_push(int prec, const void* site, const void* bn1, void* parts, int64
 void launch_sample(int prec, void* parts, int64_t np, int N, uint64_t seed, const int64_t* offsets, int n_species,
                    const int* rep, const int* mom_mode, const double* p0, const double* p1,
                    const double q0[2][8], cudaStream_t st);
+struct FFTables;  // ff.cuh
 // One event's MV initial conditions (init.cu): its parameters, the radices of
 // its line transforms, the split of the work, its scratch and the field slice
 // it fills.  begin[k]: its first block in launch k over several events.
@@ -62,9 +63,12 @@ struct InitEv {
     int lines, cols, rows;     // lines, columns and rows a block of the three launches takes
     int begin[KINDS];
     double sigma, m2, lam2;
+    float sigma_h, sigma_l;
     uint32_t k0, k1;
+    // FP32 events keep V, tw, work and green as pairs of FP32 values in the place of each double
     double2 *V, *tw, *work, *U64, *comm;
     double* green;
+    FFTables* normal;   // FP32 events: tables of the normal variates
     void* fields;
     int* bad;                  // links whose matching did not converge
 };

@@ -37,6 +37,21 @@ def test_initial_fields_against_the_oracle(N, Ns):
     assert ev.observables().unitarity_max < 1e-13
 
 
+@pytest.mark.parametrize("N,Ns", [(4, 3), (32, 50), (45, 4), (53, 2), (64, 6), (128, 16)])
+def test_fp32_initial_fields_are_the_rounded_fp64_ones(N, Ns):
+    """An FP32 event's sheets run on pairs of FP32 values (48 bits), so that
+    its links and E_eta(0) are off by the rounding of their storage alone:
+    half a unit in the last place of an entry below 1 is 2^-25."""
+    w = wl(N, Ns, W.FP32_2ROW)
+    ev = B.Event(w)
+    ev.glasma_init()
+    st, bad = O.mv_init(w.N, w.Ns, w.g2mu_a, w.m_a, w.Lambda_a, w.seed)
+    assert bad == 0
+    U, pi = ev.download(B.GL_BUF_LINKS)[:, :, :12], ev.download(B.GL_BUF_PI)
+    assert np.abs(U - st.U.reshape(2, N * N, 18)[:, :, :12]).max() < 2.0 ** -25 + 1e-10
+    assert (np.abs(pi - st.pi.reshape(pi.shape)) <= np.abs(st.pi.reshape(pi.shape)) * 2.0 ** -24 + 1e-10).all()
+
+
 @pytest.mark.parametrize("prec", [W.FP64, W.FP32_2ROW])
 def test_batch_init_equals_single_events(prec):
     ws = [wl(N, Ns, prec, seed=20 + e) for e, (N, Ns) in enumerate([(64, 3), (16, 5), (37, 2), (128, 16), (8, 1)])]
