@@ -4,17 +4,27 @@
 // single-event launch (obs.cu) and the one launch over all events of a batch.
 // The maxima leave the kernels as squared norms; the host takes their roots.
 #pragma once
+#include "ff.cuh"
 #include "internal.h"
 #include "layout.cuh"
 #include "obs_body.cuh"
 
 namespace gl {
 
+// an FP32 value in FP64, by integer operations: the conversion instruction runs
+// at the FP64 pipe's rate (64 cycles a warp and scheduler), and the checks of an
+// FP32 state convert about 70 values a site
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x), e = u & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) return (double)x;  // zero, denormal, infinite, NaN
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
 template <typename R>
 __device__ __forceinline__ A8<double> to_d(const A8<R>& a) {
     A8<double> o;
 #pragma unroll
-    for (int k = 0; k < 8; k++) o.v[k] = (double)a.v[k];
+    for (int k = 0; k < 8; k++) o.v[k] = widen(a.v[k]);
     return o;
 }
 template <typename R>
@@ -23,19 +33,112 @@ __device__ __forceinline__ M3<double> to_d(const M3<R>& a) {
 #pragma unroll
     for (int i = 0; i < 3; i++)
 #pragma unroll
-        for (int j = 0; j < 3; j++) { o.re[i][j] = a.re[i][j]; o.im[i][j] = a.im[i][j]; }
+        for (int j = 0; j < 3; j++) { o.re[i][j] = widen(a.re[i][j]); o.im[i][j] = widen(a.im[i][j]); }
     return o;
+}
+
+// ||U U^+ - 1||_F^2 from the Gram matrix of the rows (Hermitian: upper
+// triangle, off-diagonal twice; the diagonal is real)
+__device__ __forceinline__ double gram_deviation(const M3<double>& u) {
+    double n2 = 0;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = i; j < 3; j++) {
+            double gr = 0, gi = 0;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                gr = fma(u.re[i][k], u.re[j][k], gr);
+                gr = fma(u.im[i][k], u.im[j][k], gr);
+                if (i != j) {
+                    gi = fma(u.im[i][k], u.re[j][k], gi);
+                    gi = fma(-u.re[i][k], u.im[j][k], gi);
+                }
+            }
+            const double r = gr - (i == j ? 1.0 : 0.0);
+            n2 += (i == j ? 1.0 : 2.0) * (r * r + gi * gi);
+        }
+    return n2;
+}
+
+// sum of products of FP32 values in three FP32 parts (every product and every
+// rounding of the sum and of its first correction is kept: the error is below
+// 2^-68 of the largest product, against FP64's 2^-53)
+struct Sum3 {
+    float s, c, d;
+    __device__ __forceinline__ Sum3(float a, float b) {
+        s = __fmul_rn(a, b);
+        c = fmaf(a, b, -s);
+        d = 0.f;
+    }
+    __device__ __forceinline__ void add(float a, float b) {
+        const float p = __fmul_rn(a, b), e = fmaf(a, b, -p);
+        const ff t = ff_sum(s, p), u = ff_sum(c, t.l), v = ff_sum(u.h, e);
+        s = t.h;
+        c = v.h;
+        d = __fadd_rn(d, __fadd_rn(u.l, v.l));
+    }
+    // the sum less `one` (0, or 1 with s within a factor 2 of it, else rounded)
+    __device__ __forceinline__ ff less(float one) const {
+        const ff t = ff_sum(s, -one), u = ff_sum(t.h, c);
+        return ff_quick(u.h, __fadd_rn(t.l, __fadd_rn(u.l, d)));
+    }
+};
+// the same of an FP32 link, on the FP32 pipe: the Gram matrix in three parts,
+// its deviation and the sum of squares in pairs.  54 FP64 operations a link
+// less, with a smaller error.  Links with entries whose products would leave
+// the FP32 range, or that are not finite, take the FP64 form.
+__device__ __forceinline__ double gram_deviation(const M3<float>& u) {
+    float big = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = 0; j < 3; j++) big += fabsf(u.re[i][j]) + fabsf(u.im[i][j]);
+    if (!(big < 1e9f)) return gram_deviation(to_d(u));
+    ff n2{0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = i; j < 3; j++) {
+            Sum3 gr(u.re[i][0], u.re[j][0]);
+            gr.add(u.im[i][0], u.im[j][0]);
+#pragma unroll
+            for (int k = 1; k < 3; k++) {
+                gr.add(u.re[i][k], u.re[j][k]);
+                gr.add(u.im[i][k], u.im[j][k]);
+            }
+            const ff r = gr.less(i == j ? 1.f : 0.f);
+            ff q = r * r;
+            if (i != j) {
+                Sum3 gi(u.im[i][0], u.re[j][0]);
+                gi.add(-u.re[i][0], u.im[j][0]);
+#pragma unroll
+                for (int k = 1; k < 3; k++) {
+                    gi.add(u.im[i][k], u.re[j][k]);
+                    gi.add(-u.re[i][k], u.im[j][k]);
+                }
+                const ff m = gi.less(0.f);
+                q = ff_scale(ff_fma(m, m, q), 2.f);
+            }
+            n2 = n2 + q;
+        }
+    return (double)n2.h + (double)n2.l;
 }
 
 // Site s = (x, y) into the accumulators v[FO_N]:
 //   G(x) = sum_i [e_i(x) - U_i(x-i)^+ e_i(x-i) U_i(x-i)] + i[phi(x), pi(x)]
 // (with the full transport: for a link that is not unitary, which is what the
-// check is for, U^+ e U has a trace) and ||U U^+ - 1||_F of both links at s,
-// in FP64; the maxima are kept as squared norms (the root, monotonic, is taken
-// once of the maximum).  The sums of squares of the six site fields, whose
-// halves are tr X^2 = X^a X^a / 2, go into SquareSum<R> slots: an FP32
+// check is for, U^+ e U has a trace) and ||U U^+ - 1||_F of the two links it
+// transports by, U_i(x-i) (every link is that of one site); the maxima are kept
+// as squared norms (the root, monotonic, is taken once of the maximum).  The
+// Gauss residual is FP64 throughout; an FP32 link's unitarity takes three-part
+// FP32 sums, which are more exact.  The sums of squares of the six site fields,
+// whose halves are tr X^2 = X^a X^a / 2, go into SquareSum<R> slots: an FP32
 // state's squares are exact as float pairs, so its sums cost no FP64 issue
 // (field_obs_finish turns the slots into FP64 values).
+// Bound by the FP64 pipe (87 % of its cycles): 18 events of 64/128/256, FP32,
+// 540 FP64 warp instructions a site, 559 us under ncu; with FP64 Gram matrices,
+// converted inputs and one block reduction a site the call took 786 us, now 612.
 template <typename R>
 __device__ __forceinline__ void field_obs_site(const Fields<R>& f, const typename Prec<R>::V* __restrict__ site,
                                                int N, int64_t Vn, int64_t s, double* v) {
@@ -47,28 +150,11 @@ __device__ __forceinline__ void field_obs_site(const Fields<R>& f, const typenam
     for (int d = 0; d < 2; d++) {
         const typename Prec<R>::V* e = f.e + (size_t)d * AP * Vn;
         const A8<double> eh = to_d(load_alg(e, s, Vn));
-        const A8<double> eb = conj_dn(to_d(load_link(f.U, d, sb[d], Vn)), to_d(load_alg(e, sb[d], Vn)));
+        const M3<R> u = load_link(f.U, d, sb[d], Vn);
+        const A8<double> eb = conj_dn(to_d(u), to_d(load_alg(e, sb[d], Vn)));
+#pragma unroll
         for (int a = 0; a < 8; a++) G.v[a] += eh.v[a] - eb.v[a];
-        // unitarity of the link at (d, s): ||U U^+ - 1||_F^2 from the Gram
-        // matrix of the rows (Hermitian: upper triangle, off-diagonal twice;
-        // the diagonal is real)
-        const M3<double> u = to_d(load_link(f.U, d, s, Vn));
-        double n2 = 0;
-        for (int i = 0; i < 3; i++)
-            for (int j = i; j < 3; j++) {
-                double gr = 0, gi = 0;
-                for (int k = 0; k < 3; k++) {
-                    gr = fma(u.re[i][k], u.re[j][k], gr);
-                    gr = fma(u.im[i][k], u.im[j][k], gr);
-                    if (i != j) {
-                        gi = fma(u.im[i][k], u.re[j][k], gi);
-                        gi = fma(-u.re[i][k], u.im[j][k], gi);
-                    }
-                }
-                const double r = gr - (i == j ? 1.0 : 0.0);
-                n2 += (i == j ? 1.0 : 2.0) * (r * r + gi * gi);
-            }
-        v[FO_UMAX] = nanmax(v[FO_UMAX], n2);
+        v[FO_UMAX] = nanmax(v[FO_UMAX], gram_deviation(u));
     }
     const double g2 = a_dot(G, G);
     v[FO_GMAX] = nanmax(v[FO_GMAX], g2);

@@ -109,11 +109,15 @@ struct FieldObsEv {
     double* out;
 };
 static constexpr int FIELD_OBS_MAX_BLOCKS = 1024;
-// blocks of an N x N event's field checks: one site a thread in blocks of
-// 256, at most FIELD_OBS_MAX_BLOCKS (then grid-strided)
+// blocks of an N x N event's field checks: one site a thread, at most
+// FIELD_OBS_BLOCKS (then grid-strided: a block's FP64 reduction costs a tenth of
+// a site's arithmetic, and 512 blocks fill the chip).  Blocks of 64: two warps do not yet
+// share an SM's FP64 pipe, so a 32^2 event spreads over 16 SMs (27 us against 49
+// in blocks of 256)
+static constexpr int FIELD_OBS_THREADS = 64, FIELD_OBS_BLOCKS = 512;
 inline int field_obs_blocks(int N) {
-    const int64_t b = ((int64_t)N * N + 255) / 256;
-    return (int)(b < FIELD_OBS_MAX_BLOCKS ? b : FIELD_OBS_MAX_BLOCKS);
+    const int64_t b = ((int64_t)N * N + FIELD_OBS_THREADS - 1) / FIELD_OBS_THREADS;
+    return (int)(b < FIELD_OBS_BLOCKS ? b : FIELD_OBS_BLOCKS);
 }
 // The field checks of ne events in one launch of `blocks` blocks (the sum of
 // their nblocks), their descriptors `stride` bytes apart from the device
@@ -139,8 +143,8 @@ struct ObsEvent {
 // energy density per site, tr of the squared site fields (FP64 out[N*N])
 void launch_energy(int prec, const void* site, int N, double* out, cudaStream_t st);
 
-// light-like jet-correlator probes (Sec. 5.2), [n][JET_LEN] in the state's
-// precision: x0, y0, W (18), X_x, X_y, X_z (8 each)
+// light-like jet-correlator probes (Sec. 5.2), JET_LEN planes of n values in the
+// state's precision: x0, y0, W (18), X_x, X_y, X_z (8 each)
 static constexpr int JET_LEN = 44;
 void launch_jets_init(int prec, void* jets, int64_t n, int N, uint64_t seed, cudaStream_t st);
 // one step of every probe from t_n = t: site fields at t_n, links at t_{n+1} (bn1)

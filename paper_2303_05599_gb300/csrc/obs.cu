@@ -15,7 +15,7 @@ __device__ __forceinline__ FieldObsEv field_obs_event(const FieldObsEv& one, con
 // Block b is block b - block_begin of its event, grid-strided over that
 // event's sites; one row of partial results per block.
 template <typename R>
-__global__ void __launch_bounds__(256) field_obs_kernel(FieldObsEv one, const char* evs, size_t stride, int ne) {
+__global__ void __launch_bounds__(FIELD_OBS_THREADS) field_obs_kernel(FieldObsEv one, const char* evs, size_t stride, int ne) {
     int e = 0;
     if (ne > 0) {
         int lo = 0, hi = ne - 1;
@@ -49,8 +49,8 @@ void launch_field_obs_events(int prec, const FieldObsEv& one, const void* evs, s
                              bool finalize, cudaStream_t st) {
     if (blocks < 1) return;
     const char* p = (const char*)evs;
-    if (prec == 0) field_obs_kernel<double><<<blocks, 256, 0, st>>>(one, p, stride, ne);
-    else field_obs_kernel<float><<<blocks, 256, 0, st>>>(one, p, stride, ne);
+    if (prec == 0) field_obs_kernel<double><<<blocks, FIELD_OBS_THREADS, 0, st>>>(one, p, stride, ne);
+    else field_obs_kernel<float><<<blocks, FIELD_OBS_THREADS, 0, st>>>(one, p, stride, ne);
     if (finalize) field_obs_finalize<<<ne > 0 ? ne : 1, OBS_FINAL_WARPS * 32, 0, st>>>(one, p, stride, ne);
 }
 

@@ -278,6 +278,8 @@ template <typename IsMax>
 __device__ __forceinline__ void obs_finalize_block(const double* partials, int nblocks, int width, IsMax is_max,
                                                    double* out, double* copy = nullptr) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int top = 16;
+    while (top > 0 && top >= nblocks) top >>= 1;
     double acc[OBS_FINAL_V];
 #pragma unroll
     for (int j = 0; j < OBS_FINAL_V; j++) acc[j] = 0.0;
@@ -299,8 +301,8 @@ __device__ __forceinline__ void obs_finalize_block(const double* partials, int n
     for (int j = 0; j < OBS_FINAL_V; j++) {
         const int k = w + j * OBS_FINAL_WARPS;
         const bool mx = k < width && is_max(k);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+        // lanes beyond the rows hold zeros: the levels that would add them are skipped
+        for (int o = top; o > 0; o >>= 1) {
             const double oth = __shfl_down_sync(0xffffffffu, acc[j], o);
             acc[j] = mx ? nanmax(acc[j], oth) : acc[j] + oth;
         }
