@@ -28,6 +28,7 @@
 #include "internal.h"
 #include "obs_body.cuh"
 #include "push_body.cuh"
+#include "small_body.cuh"
 #include "strip_body.cuh"
 
 namespace gl {
@@ -50,7 +51,7 @@ struct EvDesc {
     double t_form[GL_MAX_SPECIES];
     int ptau_diag;
     int n_species;
-    int pad;
+    int small_begin; // FP64: first block of this event in the launch of the small lattices
 };
 
 struct BatchArgs {
@@ -69,12 +70,14 @@ struct BatchArgs {
 // reads one event's entry and a ballot counts those at or before the block,
 // 32 events per round, so a block starts after one round of loads instead of
 // a chain of dependent ones
-__device__ __forceinline__ int find_event_warp(const EvDesc* ev, int ne, int block, bool tiles) {
+enum { FIND_CHUNKS = 0, FIND_TILES, FIND_SMALL };
+__device__ __forceinline__ int find_event_warp(const EvDesc* ev, int ne, int block, int kind) {
     const int lane = threadIdx.x & 31;
     int cnt = 0;
     for (int g = 0; g < ne; g += 32) {
         const int k = g + lane;
-        const bool le = k < ne && (tiles ? ev[k].tile_begin : ev[k].chunk_begin) <= block;
+        const bool le = k < ne && (kind == FIND_TILES ? ev[k].tile_begin : kind == FIND_SMALL ? ev[k].small_begin
+                                                                                              : ev[k].chunk_begin) <= block;
         const unsigned m = __ballot_sync(0xffffffffu, le);
         cnt += __popc(m);
         if (m != 0xffffffffu) break;
@@ -109,8 +112,9 @@ __device__ __forceinline__ void strip_seg_item(const BatchArgs& b, StripWarpSmem
                       (float4*)d.site[n & 1], d.N, j - d.seg_begin, real, a, b.seg_rows);
 }
 
-// one field tile (block `blk` of the tile prefix table) of step n = clock
-template <typename R, int TX, int TY>
+// one field tile (block `blk` of the tile prefix table) of step n = clock;
+// SMALL: of the small FP64 lattices (small_body.cuh) and their table
+template <typename R, int TX, int TY, bool SMALL = false>
 __device__ __forceinline__ void field_item(const BatchArgs& b, int blk) {
     // the block's event and step scalars, once per block
     __shared__ int s_e;
@@ -118,7 +122,7 @@ __device__ __forceinline__ void field_item(const BatchArgs& b, int blk) {
     __shared__ StepR<R> s_a;
     if (threadIdx.x < 32) {
         const int64_t n = *b.clock;
-        const int e = find_event_warp(b.ev, b.ne, blk, true);
+        const int e = find_event_warp(b.ev, b.ne, blk, SMALL ? FIND_SMALL : FIND_TILES);
         if (threadIdx.x == 0) {
             const int reunit = b.reunit_every > 0 && (n + 1) % b.reunit_every == 0;
             s_e = e;
@@ -130,8 +134,10 @@ __device__ __forceinline__ void field_item(const BatchArgs& b, int blk) {
     const EvDesc& d = b.ev[s_e];
     const int64_t n = s_n;
     const int64_t Vn = (int64_t)d.N * d.N;
-    fused_tile<R, TX, TY>(carve_fields<R>(d.field[n & 1], Vn), carve_fields<R>(d.field[(n + 1) & 1], Vn),
-                                (typename Prec<R>::V*)d.site[n & 1], s_a, blk - d.tile_begin);
+    const Fields<R> in = carve_fields<R>(d.field[n & 1], Vn), out = carve_fields<R>(d.field[(n + 1) & 1], Vn);
+    typename Prec<R>::V* site = (typename Prec<R>::V*)d.site[n & 1];
+    if constexpr (SMALL) small_tile(in, out, site, s_a, blk - d.small_begin);
+    else fused_tile<R, TX, TY>(in, out, site, s_a, blk - d.tile_begin);
 }
 
 // one chunk of b.push_chunk particles (block `blk` of the chunk prefix table),
@@ -147,7 +153,7 @@ __device__ __forceinline__ void push_item(const BatchArgs& b, int lag, int blk) 
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
         const int64_t n = *b.clock - lag;
-        const int e = find_event_warp(b.ev, b.ne, blk, false);
+        const int e = find_event_warp(b.ev, b.ne, blk, FIND_CHUNKS);
         const EvDesc& d = b.ev[e];
         const double t = n * b.dt;
         // species k on lane k
@@ -187,6 +193,10 @@ __device__ __forceinline__ void push_item(const BatchArgs& b, int lag, int blk) 
 template <typename R, int TX, int TY>
 __global__ void __launch_bounds__(TX * TY, (Tile<R, TX, TY>::min_blocks)) batch_field_kernel(BatchArgs b) {
     field_item<R, TX, TY>(b, blockIdx.x);
+}
+
+__global__ void __launch_bounds__(SmallTile::NT) batch_small_kernel(BatchArgs b) {
+    field_item<double, 32, 4, true>(b, blockIdx.x);
 }
 
 // FP32 field step of the whole batch: blocks of up to WPB warps take as many
@@ -258,11 +268,12 @@ __global__ void __launch_bounds__(256, 1) batch_fused_strip_kernel(BatchArgs b, 
 
 template <typename R, int TX, int TY>
 __global__ void __launch_bounds__(TX * TY, (Tile<R, TX, TY>::min_blocks))
-    batch_fused_kernel(BatchArgs b, int lag, int n_field, int n_push) {
-    const int64_t total = (int64_t)n_field + n_push;
+    batch_fused_kernel(BatchArgs b, int lag, int n_field, int n_small, int n_push) {
+    const int64_t fields = (int64_t)n_field + n_small, total = fields + n_push;
     for (int64_t w = blockIdx.x; w < total; w += gridDim.x) {
-        const int64_t f0 = w * n_field / total, f1 = (w + 1) * n_field / total;
-        if (f1 > f0) field_item<R, TX, TY>(b, (int)f0);
+        const int64_t f0 = w * fields / total, f1 = (w + 1) * fields / total;
+        if (f1 > f0 && f0 < n_field) field_item<R, TX, TY>(b, (int)f0);
+        else if (f1 > f0) field_item<R, TX, TY, true>(b, (int)(f0 - n_field));
         else push_item<R>(b, lag, (int)(w - f0));
         __syncthreads();  // shared memory is reused by the next item
     }
@@ -393,11 +404,12 @@ static void strip_shape_geometry(int tile, int* wpb, int* warps_sm) {
 template <typename R>
 static void launch_batch_field(int tile, int blocks, int64_t nseg, const BatchArgs& b, cudaStream_t st) {
     if constexpr (sizeof(R) == 8) {
-        // FP64: the 32x4 tile only (shared memory)
+        // FP64: the 32x4 tile only (shared memory), and the small lattices'
+        // tiles (nseg of them) in a launch of their own, six blocks an SM
         (void)tile;
-        (void)nseg;
         set_smem_attr<R, 32, 4>();
-        batch_field_kernel<R, 32, 4><<<blocks, 128, Tile<R, 32, 4>::bytes, st>>>(b);
+        if (blocks > 0) batch_field_kernel<R, 32, 4><<<blocks, 128, Tile<R, 32, 4>::bytes, st>>>(b);
+        if (nseg > 0) batch_small_kernel<<<(unsigned)nseg, SmallTile::NT, sizeof(SmallTile), st>>>(b);
     } else if (tile == 1) {
         launch_strip_shape<12, 1>(nseg, b, st);
     } else if (tile == 2) {
@@ -426,12 +438,12 @@ static int fused_grid() {
 }
 
 template <typename R, int TX, int TY>
-static void launch_fused_t(const BatchArgs& b, int lag, int n_field, int n_push, cudaStream_t st) {
+static void launch_fused_t(const BatchArgs& b, int lag, int n_field, int n_small, int n_push, cudaStream_t st) {
     int g = fused_grid<R, TX, TY>();
-    const int total = n_field + n_push;
+    const int total = n_field + n_small + n_push;
     if (g > total) g = total;
     if (g < 1) return;
-    batch_fused_kernel<R, TX, TY><<<g, TX * TY, Tile<R, TX, TY>::bytes, st>>>(b, lag, n_field, n_push);
+    batch_fused_kernel<R, TX, TY><<<g, TX * TY, Tile<R, TX, TY>::bytes, st>>>(b, lag, n_field, n_small, n_push);
 }
 
 // FP32: the persistent fused launch over strip items and push chunks
@@ -460,8 +472,7 @@ static void launch_batch_fused(int tile, const BatchArgs& b, int lag, int n_fiel
                                cudaStream_t st) {
     if constexpr (sizeof(R) == 8) {
         (void)tile;
-        (void)nseg;
-        launch_fused_t<R, 32, 4>(b, lag, n_field, n_push, st);
+        launch_fused_t<R, 32, 4>(b, lag, n_field, (int)nseg, n_push, st);
     } else {
         (void)tile;
         (void)n_field;
@@ -500,7 +511,7 @@ struct gl_batch {
     int fused;        // 1: one persistent fused launch per step; 0: field and push on two streams
     int push_grid;    // two streams: 0 = one push block per chunk, k > 0 = k resident 128-thread blocks per SM
     int field_blocks;      // FP64: tiles of all events
-    int64_t field_segs;    // FP32: segments of all events' strips
+    int64_t field_segs;    // FP32: segments of all events' strips; FP64: tiles of the small lattices
     int seg_rows;          // FP32: rows per segment, for the current launch shape
     int strip_wpb;         // FP32: warps per block of its launch
     int plan_tile, plan_seg;  // the shape and fixed segment length (0: none) the two belong to
@@ -790,7 +801,13 @@ static gl_status sync_desc(gl_batch* b) {
     int tb = 0, cb = 0;
     int64_t rb = 0;
     const int TX = TILE_DIMS[b->tile][0], TY = TILE_DIMS[b->tile][1];
-    int64_t step0 = -1;
+    int64_t step0 = -1, tiles_all = 0;
+    const int sms = b->prec == GL_FP64 ? sm_count() : 0;
+    for (int e = 0; e < b->ne && b->prec == GL_FP64; e++) {
+        CtxView v;
+        ctx_view(b->ev[e], &v);
+        tiles_all += tiles64(v.N);
+    }
     if (b->prec != GL_FP64) {
         if (b->plan_tile != b->tile || b->plan_seg != b->seg_tuned[b->tile]) {
             const StripPlan p = batch_strip_plan(b);
@@ -815,11 +832,13 @@ static gl_status sync_desc(gl_batch* b) {
         d.site[1] = v.site[1];
         d.parts = v.parts;
         d.N = v.N;
-        d.tiles_x = (v.N + TX - 1) / TX;
+        const bool small = b->prec == GL_FP64 && small64(tiles_all, sms);
+        d.tiles_x = small ? small_tiles_x(v.N) : (v.N + TX - 1) / TX;
         d.tile_begin = tb;
-        tb += d.tiles_x * ((v.N + TY - 1) / TY);
+        tb += small ? 0 : d.tiles_x * ((v.N + TY - 1) / TY);
         d.seg_begin = rb;
-        rb += b->prec != GL_FP64 ? strip_segments(v.N, b->seg_rows) : 0;
+        d.small_begin = (int)rb;
+        rb += b->prec != GL_FP64 ? strip_segments(v.N, b->seg_rows) : small ? d.tiles_x * d.tiles_x : 0;
         d.chunk_begin = cb;
         cb += (int)((v.np + b->push_chunk - 1) / b->push_chunk);
         d.np = v.np;

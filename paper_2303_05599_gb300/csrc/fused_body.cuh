@@ -208,6 +208,13 @@ __host__ __device__ inline StepR<R> step_r(const StepArgs& a) {
     return r;
 }
 
+// e(n+1/2) = e(n-1/2) + dt (t F + c / t), F the plaquette force and c the scalar
+// current (shared with the small tiles, one rounding order)
+template <typename R>
+__device__ __forceinline__ R next_e(R e, R F, R c, R t, R dt, R inv_t) {
+    return fma(dt, fma(t, F, mul_rn(inv_t, c)), e);
+}
+
 // one tile (index `tile` of a lattice with tiles_x tiles per row); the caller
 // provides the dynamic shared memory of Tile<R, TX, TY>::bytes
 template <typename R, int TX, int TY>
@@ -319,7 +326,7 @@ __device__ __forceinline__ void fused_tile(const Fields<R>& in, const Fields<R>&
             A8<R> ex_n, sx;
 #pragma unroll
             for (int c = 0; c < 8; c++) {
-                ex_n.v[c] = eox.v[c] + dt * (t * (A0.v[c] - Dn.v[c]) + inv_t * cx.v[c]);
+                ex_n.v[c] = next_e(eox.v[c], A0.v[c] - Dn.v[c], cx.v[c], t, dt, inv_t);
                 sx.v[c] = eox.v[c] + ex_n.v[c];
             }
             // only this thread reads site e of sEs before the barrier
@@ -338,7 +345,7 @@ __device__ __forceinline__ void fused_tile(const Fields<R>& in, const Fields<R>&
             A8<R> ey_n, sy;
 #pragma unroll
             for (int c = 0; c < 8; c++) {
-                ey_n.v[c] = eoy.v[c] + dt * (t * (Lf.v[c] - A0.v[c]) + inv_t * cy.v[c]);
+                ey_n.v[c] = next_e(eoy.v[c], Lf.v[c] - A0.v[c], cy.v[c], t, dt, inv_t);
                 sy.v[c] = eoy.v[c] + ey_n.v[c];
             }
             s_alg_put(sEs + AP * EN, e, EN, sy);
@@ -367,8 +374,8 @@ __device__ __forceinline__ void fused_tile(const Fields<R>& in, const Fields<R>&
 #pragma unroll
         for (int c = 0; c < 8; c++) {
             const R lap = my_tx.v[c] + my_ty.v[c] + bx.v[c] + by.v[c] - R(4) * ph.v[c];
-            p_new.v[c] = p_old.v[c] + dt * inv_t * lap;
-            ph_new.v[c] = ph.v[c] + a.dt_th * p_new.v[c];
+            p_new.v[c] = fma(mul_rn(dt, inv_t), lap, p_old.v[c]);
+            ph_new.v[c] = fma(a.dt_th, p_new.v[c], ph.v[c]);
         }
         // the site fields of t_n, written by every field step (one code path for
         // every caller, so the fields evolve bitwise alike whether or not the

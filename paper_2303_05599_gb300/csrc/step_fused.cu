@@ -1,6 +1,7 @@
 // Single-event launch of the field step: the FP32 strip kernel
 // (strip_body.cuh) or the FP64 tile kernel (fused_body.cuh), both writing the
 // site E, B of t_n beside the fields of step n + 1.
+#include "small_body.cuh"
 #include "strip_body.cuh"
 
 namespace gl {
@@ -83,11 +84,23 @@ static void launch_strip(void* in, void* out, void* site, int N, int64_t n, doub
         p.seg);
 }
 
+__global__ void __launch_bounds__(SmallTile::NT) small_step_kernel(Fields<double> in, Fields<double> out, double2* site,
+                                                                  StepR<double> a) {
+    small_tile(in, out, site, a, blockIdx.x);
+}
+
 void launch_fused_step(int prec, void* in, void* out, void* site, int N, int64_t n, double dt, int reunit_every,
                        int tile, int seg, cudaStream_t st) {
     if (prec == 0) {
-        // FP64 tiles: 32x4 (139 KB of shared memory) or 32x2
-        if (tile == 2) launch_t<double, 32, 2>(in, out, site, N, n, dt, st);
+        // FP64: 4x4 tiles of four warps for small lattices, else 32x4 (139 KB of
+        // shared memory) or 32x2
+        if (small64(tiles64(N), sm_count())) {
+            const int64_t Vn = (int64_t)N * N;
+            const int nt = small_tiles_x(N);
+            small_step_kernel<<<nt * nt, SmallTile::NT, sizeof(SmallTile), st>>>(
+                carve_fields<double>(in, Vn), carve_fields<double>(out, Vn), (double2*)site,
+                step_r<double>(step_args(N, nt, n, dt, 0)));
+        } else if (tile == 2) launch_t<double, 32, 2>(in, out, site, N, n, dt, st);
         else launch_t<double, 32, 4>(in, out, site, N, n, dt, st);
     } else if (tile == 1) {
         launch_strip<12, 1>(in, out, site, N, n, dt, reunit_every, seg, st);

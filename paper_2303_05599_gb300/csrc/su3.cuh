@@ -25,6 +25,13 @@ struct A8 {
 template <typename R>
 __host__ __device__ __forceinline__ R inv_sqrt3() { return R(0.57735026918962576451); }
 
+// A product that the compiler does not fuse into a later sum.  The FP64 field
+// step has two kernels (tiles of 128 and of 16 sites) whose results are the
+// same bits: every operation whose fusion would depend on what surrounds it is
+// either this or an explicit fma.  FP32 has one kernel body and lets it fuse.
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return a * b; }
+
 template <typename R>
 __device__ __forceinline__ M3<R> m_zero() {
     M3<R> m;
@@ -226,11 +233,11 @@ __device__ __forceinline__ A8<R> adj_dag(const M3<R>& U, const A8<R>& x) {
 // themselves (no factor 1/2)
 template <typename R>
 __device__ __forceinline__ M3<R> alg_to_mat2(const A8<R>& x) {
-    const R s3 = inv_sqrt3<R>();
+    const R p = mul_rn(x.v[7], inv_sqrt3<R>());
     M3<R> m;
-    m.re[0][0] = x.v[2] + x.v[7] * s3; m.im[0][0] = R(0);
-    m.re[1][1] = -x.v[2] + x.v[7] * s3; m.im[1][1] = R(0);
-    m.re[2][2] = R(-2) * (x.v[7] * s3); m.im[2][2] = R(0);
+    m.re[0][0] = x.v[2] + p; m.im[0][0] = R(0);
+    m.re[1][1] = p - x.v[2]; m.im[1][1] = R(0);
+    m.re[2][2] = R(-2) * p; m.im[2][2] = R(0);
     m.re[0][1] = x.v[0]; m.im[0][1] = -x.v[1];
     m.re[1][0] = x.v[0]; m.im[1][0] = x.v[1];
     m.re[0][2] = x.v[3]; m.im[0][2] = -x.v[4];
@@ -343,13 +350,13 @@ __device__ __forceinline__ A8<R> conj_dn_t(const M3<R>& V, const A8<R>& x) {
     A8<R> o;
     o.v[0] = zr[0][1];
     o.v[1] = -zi[0][1];
-    o.v[2] = R(0.5) * (zr[0][0] - zr[1][1]);
+    o.v[2] = mul_rn(R(0.5), zr[0][0] - zr[1][1]);
     o.v[3] = zr[0][2];
     o.v[4] = -zi[0][2];
     o.v[5] = zr[1][2];
     o.v[6] = -zi[1][2];
     // (Z00 + Z11 - 2 Z22) / sqrt 3 with Z22 = -(Z00 + Z11), halved for 2X
-    o.v[7] = (zr[0][0] + zr[1][1]) * R(0.86602540378443864676);
+    o.v[7] = mul_rn(zr[0][0] + zr[1][1], R(0.86602540378443864676));
     return o;
 }
 
@@ -568,10 +575,14 @@ __device__ __forceinline__ M3<R> exp_i_alg(const A8<R>& x, R s) {
     for (int i = 0; i < 3; i++)
 #pragma unroll
         for (int j = 0; j < 3; j++) {
-            const R d = (i == j) ? R(1) : R(0);
-            // (f0 + f1 X + f2 X2)_ij, complex coefficients
-            U.re[i][j] = fr[0] * d + fr[1] * X.re[i][j] - fi[1] * X.im[i][j] + fr[2] * X2.re[i][j] - fi[2] * X2.im[i][j];
-            U.im[i][j] = fi[0] * d + fr[1] * X.im[i][j] + fi[1] * X.re[i][j] + fr[2] * X2.im[i][j] + fi[2] * X2.re[i][j];
+            // (f0 + f1 X + f2 X2)_ij, complex coefficients; X and X2 have real diagonals
+            if (i == j) {
+                U.re[i][j] = fma(fr[1], X.re[i][j], fma(fr[2], X2.re[i][j], fr[0]));
+                U.im[i][j] = fma(fi[1], X.re[i][j], fma(fi[2], X2.re[i][j], fi[0]));
+            } else {
+                U.re[i][j] = fma(fr[1], X.re[i][j], fma(-fi[1], X.im[i][j], fma(fr[2], X2.re[i][j], -(fi[2] * X2.im[i][j]))));
+                U.im[i][j] = fma(fr[1], X.im[i][j], fma(fi[1], X.re[i][j], fma(fr[2], X2.im[i][j], fi[2] * X2.re[i][j])));
+            }
         }
     for (int k = 0; k < sc.nsq; k++) U = mul(U, U);
     return U;
