@@ -141,7 +141,7 @@ static Carve carve(const gl_config* cfg, int64_t np, int ns) {
     const size_t nj = cfg->n_jets > 0 ? (size_t)cfg->n_jets : 0;
     c.jets = o; o += nj ? a256(nj * JET_LEN * (prec == 0 ? 8 : 4)) : 0;
     c.jet_partials = o; o += nj ? a256((1024 * 3 + 3) * sizeof(double)) : 0;
-    size_t sc = init_scratch_bytes(cfg->N, cfg->Ns);
+    size_t sc = init_scratch_bytes(prec, cfg->N, cfg->Ns);
     size_t stg = (size_t)Vn * 6 * 8 * sizeof(double);
     if (stg > sc) sc = stg;
     if ((size_t)np * 16 * sizeof(double) > sc) sc = (size_t)np * 16 * sizeof(double);

@@ -1,5 +1,5 @@
 // McLerran-Venugopalan initial conditions on the GPU (Sec. 2.1 of
-// arXiv:2303.05599), all in FP64:
+// arXiv:2303.05599):
 //   rho^a_n(x) ~ N(0, (g^2 mu a)^2 / Ns) per sheet n, colour a, site x
 //   alpha_n = rho_n / (k^2 + m^2) in Fourier space (lattice k^2, zero mode
 //             removed, modes with k > Lambda removed)
@@ -14,8 +14,6 @@
 // literature it builds on.
 #include <math.h>
 #include <string.h>
-
-#include <type_traits>
 
 #include "ff.cuh"
 #include "internal.h"
@@ -46,7 +44,8 @@ namespace gl {
 // event of 50 sheets, 223 us a transform pass; these kernels in FP64 16.3 ms.
 // An FP32 event's fields keep 24 bits of the result, so its sheets (variates,
 // transforms, exponentials, products) run on pairs of FP32 values (ff.cuh,
-// about 48 bits) and only the links' matching in FP64.
+// about 48 bits) and only the links' matching in FP64.  FP64 events have
+// kernels of their own, in one fixed order of roundings (init64.cuh).
 //
 // A sheet's planes wait in `work`, as many sheets a round as the scratch holds.
 // Small lattices (all sheets in one round) split each nucleus's product over
@@ -63,12 +62,29 @@ static constexpr size_t INIT_ROUND_BYTES = (size_t)32 << 20;  // scratch small e
 
 struct InitPlan {
     int S, groups, per_group;  // sheets a round, groups of sheets, sheets a group
-    size_t v, tw, work, total; // byte offsets
+    size_t v, tw, work, green, total; // byte offsets
 };
 
-static InitPlan init_plan(int N, int Ns) {
+static InitPlan init_plan(int prec, int N, int Ns) {
     const size_t V = (size_t)N * N;
     InitPlan p;
+    if (prec == 0) {
+        // per site: 288 B a sheet (both nuclei), 288 B lines, 8 B Green
+        // function; the commutators, 128 B, later in the place of the sheets
+        const size_t lines = 288 * V, tables = ((size_t)2 * N * 16 + 255) & ~(size_t)255;
+        size_t room = lines + tables + 296 * V;
+        if (room < INIT_ROUND_BYTES) room = INIT_ROUND_BYTES;
+        const size_t most = (room - lines - tables - 8 * V) / (288 * V);
+        p.groups = 1;
+        p.per_group = Ns;
+        p.S = most < (size_t)Ns ? (int)most : Ns;
+        p.v = 0;
+        p.tw = lines;
+        p.work = p.tw + tables;
+        p.green = p.work + (size_t)p.S * 288 * V;
+        p.total = p.green + 8 * V;
+        return p;
+    }
     const size_t tw = (((size_t)N * 16 + 255) & ~(size_t)255) + sizeof(FFTables);
     // per site: 128 B a sheet (both nuclei), 8 B Green function, 192 B a group
     // (two nuclei's lines as two rows); later 192 B links and 128 B commutators
@@ -92,11 +108,12 @@ static InitPlan init_plan(int N, int Ns) {
     p.v = 0;
     p.tw = (size_t)p.groups * 192 * V;
     p.work = p.tw + tw;
+    p.green = p.work + (size_t)p.S * 128 * V;
     p.total = p.work + w;
     return p;
 }
 
-size_t init_scratch_bytes(int N, int Ns) { return init_plan(N, Ns).total; }
+size_t init_scratch_bytes(int prec, int N, int Ns) { return init_plan(prec, N, Ns).total; }
 
 // blocks of the kernels of one event
 static inline int rows_lines(int N) { return N >= 1024 ? 1 : 1024 / N; }          // lines a block of `rows`
@@ -106,11 +123,18 @@ static inline int cols_tile(int N, bool pow2) {                                 
 }
 static inline int sheet_rows(int N) { return N >= 256 ? 1 : 256 / N; }             // rows a block of `sheets`
 
+// FP64: lines of each of two planes a block of `rows`, columns a block of `columns`
+static inline int rows64(int N) { return N >= 512 ? 1 : 512 / N; }
+static inline int cols64(int N) {
+    const int c = N >= 2048 ? 1 : N >= 512 ? 2 : N >= 256 ? 4 : 1024 / N;
+    return c > N ? N : c;
+}
+
 InitEv init_event(int prec, void* fields, void* scratch, int N, int Ns, double g2mu_a, double m_a, double Lambda_a,
                   uint64_t seed, int* bad) {
     InitEv e;
     memset(&e, 0, sizeof e);
-    const InitPlan p = init_plan(N, Ns);
+    const InitPlan p = init_plan(prec, N, Ns);
     const int64_t V = (int64_t)N * N;
     e.N = N;
     e.Ns = Ns;
@@ -130,8 +154,8 @@ InitEv init_event(int prec, void* fields, void* scratch, int N, int Ns, double g
             while (r % q == 0) { e.rad[e.nrad++] = q; r /= q; }
         if (r > 1) e.rad[e.nrad++] = r;
     }
-    e.lines = rows_lines(N);
-    e.cols = cols_tile(N, e.pow2);
+    e.lines = prec == 0 ? rows64(N) : rows_lines(N);
+    e.cols = prec == 0 ? cols64(N) : cols_tile(N, e.pow2);
     e.rows = sheet_rows(N);
     e.sigma = g2mu_a / sqrt((double)Ns);
     const ff sg = ff_of(e.sigma);
@@ -144,11 +168,11 @@ InitEv init_event(int prec, void* fields, void* scratch, int N, int Ns, double g
     char* s = (char*)scratch;
     e.V = (double2*)(s + p.v);
     e.normal = (FFTables*)(s + p.tw);
-    e.tw = (double2*)(s + p.tw + sizeof(FFTables));
+    e.tw = (double2*)(s + p.tw + (prec == 0 ? 0 : sizeof(FFTables)));
     e.work = (double2*)(s + p.work);
-    e.green = (double*)(s + p.work + (size_t)p.S * 128 * V);
+    e.green = (double*)(s + p.green);
     e.U64 = (double2*)(s + p.work);
-    e.comm = e.U64 + (size_t)12 * V;
+    e.comm = prec == 0 ? e.work : e.U64 + (size_t)12 * V;
     e.fields = fields;
     e.prec = prec;
     e.bad = bad;
@@ -167,19 +191,12 @@ __device__ __forceinline__ const InitEv& init_find(const InitEv* evs, int ne, co
     *blk = blockIdx.x - (evs ? d.begin[k] : 0);
     return d;
 }
-enum { IK_TABLES = 0, IK_ROWS, IK_COLS, IK_SHEETS, IK_SITES, IK_LINKS, IK_N };
+enum { IK_TABLES = 0, IK_ROWS, IK_COLS, IK_SHEETS, IK_SITES, IK_LINKS, IK_PRODUCTS, IK_N };
 static_assert(IK_N <= InitEv::KINDS, "block table");
 
 // ------------------------------------------------------------ line transforms
 // `lines` lines of N points in shared memory, `ls` points apart, transformed in
 // place by the block (no barrier before, one after each pass).
-__device__ __forceinline__ double2 cmul(double2 a, double2 w) {
-    return make_double2(fma(a.x, w.x, -(a.y * w.y)), fma(a.x, w.y, a.y * w.x));
-}
-__device__ __forceinline__ double2 cmulc(double2 a, double2 w) {  // a conj(w)
-    return make_double2(fma(a.x, w.x, a.y * w.y), fma(a.y, w.x, -(a.x * w.y)));
-}
-__device__ __forceinline__ double2 cxy(double x, double y) { return make_double2(x, y); }
 struct __align__(16) ff2 {
     ff x, y;
 };
@@ -187,42 +204,37 @@ __device__ __forceinline__ ff2 cxy(ff x, ff y) { return ff2{x, y}; }
 __device__ __forceinline__ ff2 cmul(ff2 a, ff2 w) {
     return ff2{FDot(a.x, w.x).sub(a.y, w.y).get(), FDot(a.x, w.y).add(a.y, w.x).get()};
 }
-__device__ __forceinline__ ff2 cmulc(ff2 a, ff2 w) {
+__device__ __forceinline__ ff2 cmulc(ff2 a, ff2 w) {  // a conj(w)
     return ff2{FDot(a.x, w.x).add(a.y, w.y).get(), FDot(a.y, w.x).sub(a.x, w.y).get()};
 }
 __device__ __forceinline__ ff2 ldg16(const ff2* p) {
     const float4 v = __ldg((const float4*)p);
     return ff2{ff{v.x, v.y}, ff{v.z, v.w}};
 }
-__device__ __forceinline__ double2 ldg16(const double2* p) { return __ldg(p); }
-template <typename C>
-__device__ __forceinline__ C cadd(C a, C b) { return cxy(a.x + b.x, a.y + b.y); }
-template <typename C>
-__device__ __forceinline__ C csub(C a, C b) { return cxy(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ ff2 cadd(ff2 a, ff2 b) { return cxy(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ ff2 csub(ff2 a, ff2 b) { return cxy(a.x - b.x, a.y - b.y); }
 
 // powers of two: radix 4, and radix 2 on neighbours for odd log2 N
-template <typename C>
-__device__ __forceinline__ void pow2_radix2(C* sh, int lines, int ls, int lN) {
+__device__ __forceinline__ void pow2_radix2(ff2* sh, int lines, int ls, int lN) {
     for (int b = threadIdx.x; b < lines << (lN - 1); b += blockDim.x) {
-        C* p = sh + (b >> (lN - 1)) * ls + 2 * (b & ((1 << (lN - 1)) - 1));
-        const C u = p[0], v = p[1];
+        ff2* p = sh + (b >> (lN - 1)) * ls + 2 * (b & ((1 << (lN - 1)) - 1));
+        const ff2 u = p[0], v = p[1];
         p[0] = cadd(u, v);
         p[1] = csub(u, v);
     }
     __syncthreads();
 }
-template <typename C>
-__device__ __forceinline__ void pow2_forward(C* sh, int lines, int ls, int lN, const C* __restrict__ tw) {
+__device__ __forceinline__ void pow2_forward(ff2* sh, int lines, int ls, int lN, const ff2* __restrict__ tw) {
     for (int lb = lN; lb >= 2; lb -= 2) {
         const int q = 1 << (lb - 2);
         for (int b = threadIdx.x; b < lines << (lN - 2); b += blockDim.x) {
             const int j = b & ((1 << (lN - 2)) - 1), n = j & (q - 1);
-            C* p = sh + (b >> (lN - 2)) * ls + ((j >> (lb - 2)) << lb) + n;
-            const C a0 = p[0], a1 = p[q], a2 = p[2 * q], a3 = p[3 * q];
-            const C t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), t3 = csub(a1, a3);
+            ff2* p = sh + (b >> (lN - 2)) * ls + ((j >> (lb - 2)) << lb) + n;
+            const ff2 a0 = p[0], a1 = p[q], a2 = p[2 * q], a3 = p[3 * q];
+            const ff2 t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), t3 = csub(a1, a3);
             p[0] = cadd(t0, t2);
             // t1 -+ i t3
-            const C y1 = cxy(t1.x + t3.y, t1.y - t3.x), y2 = csub(t0, t2),
+            const ff2 y1 = cxy(t1.x + t3.y, t1.y - t3.x), y2 = csub(t0, t2),
                           y3 = cxy(t1.x - t3.y, t1.y + t3.x);
             if (lb > 2) {
                 const int w = n << (lN - lb);
@@ -239,23 +251,22 @@ __device__ __forceinline__ void pow2_forward(C* sh, int lines, int ls, int lN, c
     }
     if (lN & 1) pow2_radix2(sh, lines, ls, lN);
 }
-template <typename C>
-__device__ __forceinline__ void pow2_inverse(C* sh, int lines, int ls, int lN, const C* __restrict__ tw) {
+__device__ __forceinline__ void pow2_inverse(ff2* sh, int lines, int ls, int lN, const ff2* __restrict__ tw) {
     if (lN & 1) pow2_radix2(sh, lines, ls, lN);
     for (int lb = 2 + (lN & 1); lb <= lN; lb += 2) {
         const int q = 1 << (lb - 2);
         for (int b = threadIdx.x; b < lines << (lN - 2); b += blockDim.x) {
             const int j = b & ((1 << (lN - 2)) - 1), n = j & (q - 1);
-            C* p = sh + (b >> (lN - 2)) * ls + ((j >> (lb - 2)) << lb) + n;
-            C x1 = p[q], x2 = p[2 * q], x3 = p[3 * q];
-            const C x0 = p[0];
+            ff2* p = sh + (b >> (lN - 2)) * ls + ((j >> (lb - 2)) << lb) + n;
+            ff2 x1 = p[q], x2 = p[2 * q], x3 = p[3 * q];
+            const ff2 x0 = p[0];
             if (lb > 2) {
                 const int w = n << (lN - lb);
                 x1 = cmul(x1, ldg16(tw + w));
                 x2 = cmul(x2, ldg16(tw + 2 * w));
                 x3 = cmul(x3, ldg16(tw + 3 * w));
             }
-            const C t0 = cadd(x0, x2), t1 = csub(x0, x2), t2 = cadd(x1, x3), t3 = csub(x1, x3);
+            const ff2 t0 = cadd(x0, x2), t1 = csub(x0, x2), t2 = cadd(x1, x3), t3 = csub(x1, x3);
             p[0] = cadd(t0, t2);
             p[q] = cxy(t1.x - t3.y, t1.y + t3.x);
             p[2 * q] = csub(t0, t2);
@@ -268,9 +279,9 @@ __device__ __forceinline__ void pow2_inverse(C* sh, int lines, int ls, int lN, c
 // any N: a direct transform of each prime factor in turn, one output point at
 // a time (a block's points, at most 256 x INIT_GEN_OUT, wait in registers for
 // the barrier before they replace the inputs)
-template <bool FORWARD, typename C>
-__device__ __noinline__ void prime_passes(C* sh, int lines, int ls, const InitEv& d) {
-    const C* tw = (const C*)d.tw;
+template <bool FORWARD>
+__device__ __noinline__ void prime_passes(ff2* sh, int lines, int ls, const InitEv& d) {
+    const ff2* tw = (const ff2*)d.tw;
     const int N = d.N, total = lines * N;
     int B = N;
     if (!FORWARD)
@@ -279,26 +290,26 @@ __device__ __noinline__ void prime_passes(C* sh, int lines, int ls, const InitEv
         const int s = FORWARD ? i : d.nrad - 1 - i;
         const int r = d.rad[s], m = B / r;
         const int wr = N / r, wB = N / B;
-        C out[INIT_GEN_OUT];
+        ff2 out[INIT_GEN_OUT];
 #pragma unroll
         for (int c = 0; c < INIT_GEN_OUT; c++) {
             const int idx = threadIdx.x + c * INIT_T;
             if (idx < total) {
                 const int line = idx / N, p = idx - line * N, nb = p / B, k = (p - nb * B) / m, n = p % m;
-                const C* x = sh + line * ls + nb * B + n;
-                C a = {};
+                const ff2* x = sh + line * ls + nb * B + n;
+                ff2 a = {};
                 int w = 0;               // (q k mod r) N / r
                 const int step = k * wr;
                 int tn = 0;              // inverse: n q N / B
                 for (int q = 0; q < r; q++) {
-                    const C v = x[q * m];
+                    const ff2 v = x[q * m];
                     if (FORWARD) {
-                        const C t = cmulc(v, ldg16(tw + w));
+                        const ff2 t = cmulc(v, ldg16(tw + w));
                         a = cadd(a, t);
                     } else {
                         int u = w + tn;
                         if (u >= N) u -= N;
-                        const C t = cmul(v, ldg16(tw + u));
+                        const ff2 t = cmul(v, ldg16(tw + u));
                         a = cadd(a, t);
                         tn += n * wB;
                         if (tn >= N) tn -= N;
@@ -325,14 +336,12 @@ __device__ __noinline__ void prime_passes(C* sh, int lines, int ls, const InitEv
     }
 }
 
-template <typename C>
-__device__ __forceinline__ void lines_forward(C* sh, int lines, int ls, const InitEv& d) {
-    if (d.pow2) pow2_forward(sh, lines, ls, d.log2N, (const C*)d.tw);
+__device__ __forceinline__ void lines_forward(ff2* sh, int lines, int ls, const InitEv& d) {
+    if (d.pow2) pow2_forward(sh, lines, ls, d.log2N, (const ff2*)d.tw);
     else prime_passes<true>(sh, lines, ls, d);
 }
-template <typename C>
-__device__ __forceinline__ void lines_inverse(C* sh, int lines, int ls, const InitEv& d) {
-    if (d.pow2) pow2_inverse(sh, lines, ls, d.log2N, (const C*)d.tw);
+__device__ __forceinline__ void lines_inverse(ff2* sh, int lines, int ls, const InitEv& d) {
+    if (d.pow2) pow2_inverse(sh, lines, ls, d.log2N, (const ff2*)d.tw);
     else
         for (int l = 0; l < lines;) {  // at most INIT_T x INIT_GEN_OUT points at a time
             int c = INIT_T * INIT_GEN_OUT / d.N;
@@ -357,7 +366,8 @@ __device__ __forceinline__ int line_frequency(const InitEv& d, int p) {
 }
 
 // the event's twiddles and its Green function over the number of sites, in the
-// order the transforms leave
+// order the transforms leave (FP64: the order of the frequencies, and the
+// twiddles of either sign)
 __global__ void __launch_bounds__(INIT_T) init_tables_kernel(const InitEv* evs, int ne, InitEv one) {
     int blk;
     const InitEv& d = init_find(evs, ne, one, IK_TABLES, &blk);
@@ -369,6 +379,8 @@ __global__ void __launch_bounds__(INIT_T) init_tables_kernel(const InitEv* evs, 
         sincospi(2.0 * (double)s / (double)N, &sn, &cs);
         if (d.prec == 0) {
             d.tw[s] = make_double2(cs, sn);
+            sincospi(-2.0 * (double)s / (double)N, &sn, &cs);
+            d.tw[N + s] = make_double2(cs, sn);
         } else {
             ((ff2*)d.tw)[s] = ff2{ff_of(cs), ff_of(sn)};
         }
@@ -376,7 +388,7 @@ __global__ void __launch_bounds__(INIT_T) init_tables_kernel(const InitEv* evs, 
     if (d.prec != 0 && s < FF_ANGLES) ff_table_entry(d.normal, (int)s);
     if (s < Vn) {
         const int px = (int)(s % N), py = (int)(s / N);
-        const int kx = line_frequency(d, px), ky = line_frequency(d, py);
+        const int kx = d.prec == 0 ? px : line_frequency(d, px), ky = d.prec == 0 ? py : line_frequency(d, py);
         const double sx = sinpi((double)kx / N), sy = sinpi((double)ky / N);
         const double k2 = 4.0 * (sx * sx + sy * sy);
         double g = 1.0 / (k2 + d.m2);
@@ -389,28 +401,20 @@ __global__ void __launch_bounds__(INIT_T) init_tables_kernel(const InitEv* evs, 
 }
 
 // two independent normal variates of standard deviation sigma
-__device__ __forceinline__ double2 normal_pair(const InitEv& d, uint32_t w1, uint32_t w2, double2*) {
-    double z0, z1;
-    box_muller(u01(w1), u01(w2), z0, z1);
-    return make_double2(d.sigma * z0, d.sigma * z1);
-}
-__device__ __forceinline__ ff2 normal_pair(const InitEv& d, uint32_t w1, uint32_t w2, ff2*) {
+__device__ __forceinline__ ff2 normal_pair(const InitEv& d, uint32_t w1, uint32_t w2) {
     ff z0, z1;
     ff_box_muller(w1, w2, d.normal, z0, z1);
     const ff sigma{d.sigma_h, d.sigma_l};
     return ff2{sigma * z0, sigma * z1};
 }
 
-// Blocks per SM of a line kernel: FP64 is bound by its pipe, which four warps
-// fill; pairs are bound by latency and take as many registers as the compiler
-// is given (2, 2 and 1 blocks of the three kernels without a cap, 5.4 ms a
-// 256^2 event; 4, 4 and 2 take 4.7 ms in spite of a few spills, 3, 3 and 3 5.8 ms).
-template <typename C>
-constexpr int line_blocks(int n) { return std::is_same<C, ff2>::value ? n : 1; }
+// Blocks per SM of the line kernels: pairs are bound by latency and take as many
+// registers as the compiler is given (2, 2 and 1 blocks of the three kernels
+// without a cap, 5.4 ms a 256^2 event; 4, 4 and 2 take 4.7 ms in spite of a few
+// spills, 3, 3 and 3 5.8 ms).
 
 // rho of d.lines lattice rows of one or two planes and their forward transforms
-template <typename C>
-__device__ __forceinline__ void init_rows(const InitEv& d, int blk, int round, C* sh) {
+__device__ __forceinline__ void init_rows(const InitEv& d, int blk, int round, ff2* sh) {
     const int N = d.N, S = d.S;
     const int64_t all = (int64_t)2 * S * 4 * N, line0 = (int64_t)blk * d.lines;
     const int nl = (int)(all - line0 < d.lines ? all - line0 : d.lines);
@@ -422,33 +426,30 @@ __device__ __forceinline__ void init_rows(const InitEv& d, int blk, int round, C
         const int64_t line = line0 + l;
         const int row = (int)(line % N), plane = (int)(line / N) & 3, slot = (int)(line / (4 * (int64_t)N));
         const int nucleus = slot / S, sheet = round * S + slot - nucleus * S;
-        C z = {};
+        ff2 z = {};
         if (sheet < d.Ns) {
             const U4 w = philox4x32_10(U4{(uint32_t)(row * N + x), (uint32_t)((nucleus * d.Ns + sheet) * 2 + (plane >> 1)),
                                           1u, 0u}, d.k0, d.k1);
-            z = normal_pair(d, (plane & 1) ? w.z : w.x, (plane & 1) ? w.w : w.y, (C*)nullptr);
+            z = normal_pair(d, (plane & 1) ? w.z : w.x, (plane & 1) ? w.w : w.y);
         }
         sh[idx] = z;
     }
     __syncthreads();
     lines_forward(sh, nl, N, d);
-    C* out = (C*)d.work + (size_t)line0 * N;  // work[slot][plane][row][position]
+    ff2* out = (ff2*)d.work + (size_t)line0 * N;  // work[slot][plane][row][position]
     for (int idx = threadIdx.x; idx < nl * N; idx += INIT_T) out[idx] = sh[idx];
 }
-template <typename C>
-__global__ void __launch_bounds__(INIT_T, line_blocks<C>(4)) init_rows_kernel(const InitEv* evs, int ne, InitEv one, int round) {
+__global__ void __launch_bounds__(INIT_T, 4) init_rows_kernel(const InitEv* evs, int ne, InitEv one, int round) {
     extern __shared__ __align__(16) unsigned char init_smem[];
     int blk;
     const InitEv& d = init_find(evs, ne, one, IK_ROWS, &blk);
-    init_rows<C>(d, blk, round, (C*)init_smem);
+    init_rows(d, blk, round, (ff2*)init_smem);
 }
 
 // alpha = rho / (k^2 + m^2) along the columns of one plane
-template <typename C>
-__global__ void __launch_bounds__(INIT_T, line_blocks<C>(4)) init_cols_kernel(const InitEv* evs, int ne, InitEv one, int round) {
-    using R = decltype(C::x);
+__global__ void __launch_bounds__(INIT_T, 4) init_cols_kernel(const InitEv* evs, int ne, InitEv one, int round) {
     extern __shared__ __align__(16) unsigned char init_smem[];
-    C* sh = (C*)init_smem;
+    ff2* sh = (ff2*)init_smem;
     int blk;
     const InitEv& d = init_find(evs, ne, one, IK_COLS, &blk);
     const int N = d.N, S = d.S, ls = N + 1;  // a point of padding: neighbouring columns in other banks
@@ -456,18 +457,18 @@ __global__ void __launch_bounds__(INIT_T, line_blocks<C>(4)) init_cols_kernel(co
     const int c0 = (blk % nt) * d.cols, sp = blk / nt, slot = sp >> 2;
     if (round * S + slot % S >= d.Ns) return;
     const int nc = N - c0 < d.cols ? N - c0 : d.cols;
-    C* w = (C*)d.work + (size_t)sp * N * N + c0;
+    ff2* w = (ff2*)d.work + (size_t)sp * N * N + c0;
     for (int idx = threadIdx.x; idx < nc * N; idx += INIT_T) {
         const int r = idx / nc, c = idx - r * nc;
         sh[c * ls + r] = w[(size_t)r * N + c];
     }
     __syncthreads();
     lines_forward(sh, nc, ls, d);
-    const R* g = (const R*)d.green + c0;
+    const ff* g = (const ff*)d.green + c0;
     for (int idx = threadIdx.x; idx < nc * N; idx += INIT_T) {
         const int r = idx / nc, c = idx - r * nc;
-        const R f = g[(size_t)r * N + c];
-        const C v = sh[c * ls + r];
+        const ff f = g[(size_t)r * N + c];
+        const ff2 v = sh[c * ls + r];
         sh[c * ls + r] = cxy(v.x * f, v.y * f);
     }
     __syncthreads();
@@ -509,8 +510,7 @@ __device__ __forceinline__ void store_rows(ff2* V, int64_t s, int64_t Vn, const 
     for (int k = 0; k < 6; k++) V[(size_t)k * Vn + s] = ff2{m.re[k / 3][k % 3], m.im[k / 3][k % 3]};
 }
 // a line kept as pairs, in FP64
-__device__ __forceinline__ M3<double> load_line(const InitEv& d, const double2* V, int64_t s, int64_t Vn) {
-    if (d.prec == 0) return load_rows(V, s, Vn);
+__device__ __forceinline__ M3<double> load_line(const double2* V, int64_t s, int64_t Vn) {
     const M3ff f = load_rows((const ff2*)V, s, Vn);
     M3<double> m;
 #pragma unroll
@@ -521,9 +521,7 @@ __device__ __forceinline__ M3<double> load_line(const InitEv& d, const double2* 
     rebuild_row2(m);
     return m;
 }
-__device__ __forceinline__ M3<double> sheet_exp(const A8<double>& al) { return exp_i_alg<double>(al, 1.0); }
-__device__ __forceinline__ M3ff sheet_exp(const A8<ff>& al) { return ff_exp_i(al.v); }
-// (rows 0 and 1 of) v m
+// rows 0 and 1 of v m
 __device__ __forceinline__ M3<double> mul_rows(const M3<double>& v, const M3<double>& m) {
     M3<double> c = m_zero<double>();
 #pragma unroll
@@ -539,15 +537,12 @@ __device__ __forceinline__ M3<double> mul_rows(const M3<double>& v, const M3<dou
             }
     return c;
 }
-__device__ __forceinline__ M3ff mul_rows(const M3ff& v, const M3ff& m) { return ff_mul<2>(v, m); }
 
 // the inverse transforms of d.rows rows of a nucleus and the product over its
 // sheets of this round (of one group of them)
-template <typename C>
-__global__ void __launch_bounds__(INIT_T, line_blocks<C>(2)) init_sheets_kernel(const InitEv* evs, int ne, InitEv one, int round) {
-    using R = decltype(C::x);
+__global__ void __launch_bounds__(INIT_T, 2) init_sheets_kernel(const InitEv* evs, int ne, InitEv one, int round) {
     extern __shared__ __align__(16) unsigned char init_smem[];
-    C* sh = (C*)init_smem;
+    ff2* sh = (ff2*)init_smem;
     int blk;
     const InitEv& d = init_find(evs, ne, one, IK_SHEETS, &blk);
     const int N = d.N, S = d.S;
@@ -559,9 +554,9 @@ __global__ void __launch_bounds__(INIT_T, line_blocks<C>(2)) init_sheets_kernel(
     int s0 = round * S, s1 = s0 + S < d.Ns ? s0 + S : d.Ns;
     if (s0 < first) s0 = first;
     if (s1 > first + d.per_group) s1 = first + d.per_group;
-    C* V = (C*)d.V + (size_t)(nucleus * d.groups + g) * 6 * Vn + (int64_t)r0 * N;
+    ff2* V = (ff2*)d.V + (size_t)(nucleus * d.groups + g) * 6 * Vn + (int64_t)r0 * N;
     for (int s = s0; s < s1; s++) {
-        const C* w = (const C*)d.work + (size_t)(nucleus * S + s - round * S) * 4 * Vn + (int64_t)r0 * N;
+        const ff2* w = (const ff2*)d.work + (size_t)(nucleus * S + s - round * S) * 4 * Vn + (int64_t)r0 * N;
         for (int idx = threadIdx.x; idx < 4 * np; idx += INIT_T) {
             const int p = idx / np;
             sh[idx] = w[(size_t)p * Vn + idx - p * np];
@@ -569,17 +564,17 @@ __global__ void __launch_bounds__(INIT_T, line_blocks<C>(2)) init_sheets_kernel(
         __syncthreads();
         lines_inverse(sh, 4 * nr, N, d);
         for (int i = threadIdx.x; i < np; i += INIT_T) {
-            A8<R> al;
+            A8<ff> al;
 #pragma unroll
             for (int p = 0; p < 4; p++) {
-                const C v = sh[p * np + i];
+                const ff2 v = sh[p * np + i];
                 al.v[2 * p] = -v.x;
                 al.v[2 * p + 1] = -v.y;
             }
-            const auto e = sheet_exp(al);
+            const M3ff e = ff_exp_i(al.v);
             // only this thread reads and writes the site's line, sheet after sheet
             if (s == first) store_rows(V, i, Vn, e);
-            else store_rows(V, i, Vn, mul_rows(load_rows(V, i, Vn), e));
+            else store_rows(V, i, Vn, ff_mul<2>(load_rows(V, i, Vn), e));
         }
         __syncthreads();
     }
@@ -592,29 +587,22 @@ __global__ void __launch_bounds__(128) init_groups_kernel(const InitEv* evs, int
     const int64_t Vn = (int64_t)d.N * d.N, t = (int64_t)blk * 128 + threadIdx.x;
     if (d.groups < 2 || t >= 2 * Vn) return;
     const int64_t s = t % Vn;
-    double2* V = d.V + (size_t)(t / Vn) * d.groups * 6 * Vn;
-    if (d.prec == 0) {
-        M3<double> v = load_rows(V, s, Vn);
-        for (int g = 1; g < d.groups; g++) v = mul_rows(v, load_rows(V + (size_t)g * 6 * Vn, s, Vn));
-        store_rows(V, s, Vn, v);
-    } else {
-        ff2* W = (ff2*)V;
-        M3ff v = load_rows(W, s, Vn);
-        for (int g = 1; g < d.groups; g++) {
-            M3ff m = load_rows(W + (size_t)g * 6 * Vn, s, Vn);
-            // row 2: the conjugate cross product of rows 0 and 1
+    ff2* V = (ff2*)d.V + (size_t)(t / Vn) * d.groups * 6 * Vn;
+    M3ff v = load_rows(V, s, Vn);
+    for (int g = 1; g < d.groups; g++) {
+        M3ff m = load_rows(V + (size_t)g * 6 * Vn, s, Vn);
+        // row 2: the conjugate cross product of rows 0 and 1
 #pragma unroll
-            for (int j = 0; j < 3; j++) {
-                const int p = (j + 1) % 3, q = (j + 2) % 3;
-                m.re[2][j] = FDot(m.re[0][p], m.re[1][q]).sub(m.im[0][p], m.im[1][q]).sub(m.re[0][q], m.re[1][p])
-                                 .add(m.im[0][q], m.im[1][p]).get();
-                m.im[2][j] = -FDot(m.re[0][p], m.im[1][q]).add(m.im[0][p], m.re[1][q]).sub(m.re[0][q], m.im[1][p])
-                                 .sub(m.im[0][q], m.re[1][p]).get();
-            }
-            v = mul_rows(v, m);
+        for (int j = 0; j < 3; j++) {
+            const int p = (j + 1) % 3, q = (j + 2) % 3;
+            m.re[2][j] = FDot(m.re[0][p], m.re[1][q]).sub(m.im[0][p], m.im[1][q]).sub(m.re[0][q], m.re[1][p])
+                             .add(m.im[0][q], m.im[1][p]).get();
+            m.im[2][j] = -FDot(m.re[0][p], m.im[1][q]).add(m.im[0][p], m.re[1][q]).sub(m.re[0][q], m.im[1][p])
+                             .sub(m.im[0][q], m.re[1][p]).get();
         }
-        store_rows(W, s, Vn, v);
+        v = ff_mul<2>(v, m);
     }
+    store_rows(V, s, Vn, v);
 }
 
 // Im tr(T^a M)
@@ -643,6 +631,12 @@ __device__ __forceinline__ void re_tr_T(const M3<R>& M, R* f) {
     f[6] = h * (M.im[2][1] - M.im[1][2]);
     f[7] = s3 * (M.re[0][0] + M.re[1][1] - R(2) * M.re[2][2]);
 }
+
+}  // namespace gl
+
+#include "init64.cuh"
+
+namespace gl {
 
 // Jacobian of F^a = Im tr T^a (W + K), K = W U^+, under U -> exp(i x.T) U:
 // J_ab = -Re tr(T^a K T^b).  With T^b T^a = delta/6 + (d + i f)_bac T^c / 2,
@@ -819,20 +813,30 @@ __global__ void __launch_bounds__(64) init_links_kernel(const InitEv* evs, int n
     const int x = (int)(s % N), y = (int)(s / N);
     const int64_t sn = d == 0 ? (int64_t)y * N + (x + 1 == N ? 0 : x + 1) : (int64_t)(y + 1 == N ? 0 : y + 1) * N + x;
     const double2* VB = ev.V + (size_t)ev.groups * 6 * Vn;
-    const M3<double> UA = mul_dn(load_line(ev, ev.V, s, Vn), load_line(ev, ev.V, sn, Vn));
-    const M3<double> UB = mul_dn(load_line(ev, VB, s, Vn), load_line(ev, VB, sn, Vn));
+    const M3<double> UA = mul_dn(load_line(ev.V, s, Vn), load_line(ev.V, sn, Vn));
+    const M3<double> UB = mul_dn(load_line(VB, s, Vn), load_line(VB, sn, Vn));
     store_alg(ev.comm + (size_t)d * 4 * Vn, s, Vn, icomm(iah_to_alg(UA), iah_to_alg(UB)));
     M3<double> U;
     if (solve_link(UA, UB, U)) atomicAdd(ev.bad, 1);
     store_rows(ev.U64 + (size_t)d * 6 * Vn, s, Vn, U);
 }
 
-template <typename R>
-__device__ __forceinline__ M3<R> to_r(const M3<double>& m) {
-    M3<R> o;
+// the Glasma link: an FP64 event's is in its fields already, an FP32 event's in the scratch
+__device__ __forceinline__ M3<double> matched_link(const InitEv&, const Fields<double>& f, int k, int64_t s, int64_t Vn) {
+    return load_link(f.U, k, s, Vn);
+}
+__device__ __forceinline__ M3<double> matched_link(const InitEv& d, const Fields<float>&, int k, int64_t s, int64_t Vn) {
+    return load_rows(d.U64 + (size_t)k * 6 * Vn, s, Vn);
+}
+__device__ __forceinline__ void put_link(const InitEv&, const Fields<double>&, int, int64_t, int64_t) {}
+__device__ __forceinline__ void put_link(const InitEv& d, const Fields<float>& f, int k, int64_t s, int64_t Vn) {
+    const M3<double> m = matched_link(d, f, k, s, Vn);
+    M3<float> o;
+#pragma unroll
     for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++) { o.re[i][j] = (R)m.re[i][j]; o.im[i][j] = (R)m.im[i][j]; }
-    return o;
+#pragma unroll
+        for (int j = 0; j < 3; j++) { o.re[i][j] = (float)m.re[i][j]; o.im[i][j] = (float)m.im[i][j]; }
+    store_link(f.U, k, s, Vn, o);
 }
 
 // pi(-1/2) = E_eta(0) = -sum over the four links at the site of the link's
@@ -850,7 +854,7 @@ __device__ __forceinline__ void initial_site(const InitEv& d, int64_t s) {
         const int64_t sb = k == 0 ? (int64_t)y * N + (x == 0 ? N - 1 : x - 1) : (int64_t)(y == 0 ? N - 1 : y - 1) * N + x;
         const double2* cm = d.comm + (size_t)k * 4 * Vn;
         const A8<double> c = load_alg(cm, s, Vn);
-        const A8<double> b = conj_dn_t(load_rows(d.U64 + (size_t)k * 6 * Vn, sb, Vn), load_alg(cm, sb, Vn));
+        const A8<double> b = conj_dn_t(matched_link(d, f, k, sb, Vn), load_alg(cm, sb, Vn));
 #pragma unroll
         for (int q = 0; q < 8; q++) pi.v[q] -= 0.5 * (c.v[q] + b.v[q]);
     }
@@ -863,7 +867,7 @@ __device__ __forceinline__ void initial_site(const InitEv& d, int64_t s) {
     store_alg(f.e, s, Vn, z);
     store_alg(f.e + (size_t)Prec<R>::AP * Vn, s, Vn, z);
 #pragma unroll
-    for (int k = 0; k < 2; k++) store_link(f.U, k, s, Vn, to_r<R>(load_rows(d.U64 + (size_t)k * 6 * Vn, s, Vn)));
+    for (int k = 0; k < 2; k++) put_link(d, f, k, s, Vn);
 }
 __global__ void __launch_bounds__(128) init_fields_kernel(const InitEv* evs, int ne, InitEv one) {
     int blk;
@@ -877,6 +881,13 @@ __global__ void __launch_bounds__(128) init_fields_kernel(const InitEv* evs, int
 // the blocks of event e in launch k
 static int64_t init_blocks(const InitEv& e, int k) {
     const int64_t V = (int64_t)e.N * e.N;
+    if (e.prec == 0) switch (k) {
+        case IK_ROWS: return (int64_t)8 * e.S * ((e.N + e.lines - 1) / e.lines);
+        case IK_COLS: return (int64_t)16 * e.S * ((e.N + e.cols - 1) / e.cols);
+        case IK_SHEETS: return (2 * e.S * V + 127) / 128;
+        case IK_PRODUCTS: return 2 * ((V + 31) / 32);
+        default: break;
+    }
     switch (k) {
         case IK_TABLES: return ((V > FF_ANGLES ? V : FF_ANGLES) + INIT_T - 1) / INIT_T;
         case IK_ROWS: return ((int64_t)8 * e.S * e.N + e.lines - 1) / e.lines;
@@ -899,32 +910,23 @@ void init_block_table(InitEv* evs, int ne) {
     }
 }
 
-template <typename C>
-static void launch_sheets(const unsigned* nb, size_t rows, size_t cols, size_t sheets, int rounds, const InitEv* ev,
-                          int ne, const InitEv& one, cudaStream_t st) {
-    // per-device function attributes; set whenever a launch needs more than the default
-    const size_t most = 48 * 1024;
-    if (rows > most) cudaFuncSetAttribute(init_rows_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows);
-    if (cols > most) cudaFuncSetAttribute(init_cols_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cols);
-    if (sheets > most)
-        cudaFuncSetAttribute(init_sheets_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sheets);
-    for (int r = 0; r < rounds; r++) {
-        init_rows_kernel<C><<<nb[IK_ROWS], INIT_T, rows, st>>>(ev, ne, one, r);
-        init_cols_kernel<C><<<nb[IK_COLS], INIT_T, cols, st>>>(ev, ne, one, r);
-        init_sheets_kernel<C><<<nb[IK_SHEETS], INIT_T, sheets, st>>>(ev, ne, one, r);
-    }
+// what the launches of one kind need beyond the default is a per-device function attribute, set on every call
+template <typename K>
+static void line_smem(K* kernel, size_t bytes) {
+    if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 void launch_mv_init(const InitEv* h, const InitEv* d_ev, int ne, cudaStream_t st) {
     const InitEv one = h[0];
     const InitEv* ev = ne > 1 ? d_ev : nullptr;
+    const bool wide = one.prec == 0;  // the events of a launch have one precision
     unsigned nb[IK_N];
     size_t rows = 0, cols = 0, sheets = 0;
     int rounds = 1;
     bool grouped = false;
     for (int k = 0; k < IK_N; k++) nb[k] = (unsigned)(h[ne - 1].begin[k] + init_blocks(h[ne - 1], k));
     for (int e = 0; e < ne; e++) {
-        const size_t r = (size_t)h[e].lines * h[e].N * 16, c = (size_t)h[e].cols * (h[e].N + 1) * 16,
+        const size_t r = (size_t)h[e].lines * h[e].N * (wide ? 32 : 16), c = (size_t)h[e].cols * (h[e].N + 1) * 16,
                      s = (size_t)4 * h[e].rows * h[e].N * 16;
         rows = r > rows ? r : rows;
         cols = c > cols ? c : cols;
@@ -934,11 +936,32 @@ void launch_mv_init(const InitEv* h, const InitEv* d_ev, int ne, cudaStream_t st
         grouped = grouped || h[e].groups > 1;
     }
     init_tables_kernel<<<nb[IK_TABLES], INIT_T, 0, st>>>(ev, ne, one);
-    // the events of a launch have one precision
-    if (one.prec == 0) launch_sheets<double2>(nb, rows, cols, sheets, rounds, ev, ne, one, st);
-    else launch_sheets<ff2>(nb, rows, cols, sheets, rounds, ev, ne, one, st);
-    if (grouped) init_groups_kernel<<<nb[IK_SITES], 128, 0, st>>>(ev, ne, one);
-    init_links_kernel<<<nb[IK_LINKS], 64, 0, st>>>(ev, ne, one);
+    if (wide) {
+        line_smem(init64_rows_kernel<true>, rows);
+        line_smem(init64_rows_kernel<false>, rows);
+        line_smem(init64_cols_kernel<true>, cols);
+        line_smem(init64_cols_kernel<false>, cols);
+        for (int r = 0; r < rounds; r++) {
+            init64_rows_kernel<true><<<nb[IK_ROWS], 256, rows, st>>>(ev, ne, one, r);
+            init64_cols_kernel<true><<<nb[IK_COLS], 256, cols, st>>>(ev, ne, one, r);
+            init64_rows_kernel<false><<<nb[IK_ROWS], 256, rows, st>>>(ev, ne, one, r);
+            init64_cols_kernel<false><<<nb[IK_COLS], 256, cols, st>>>(ev, ne, one, r);
+            init64_exp_kernel<<<nb[IK_SHEETS], 128, 0, st>>>(ev, ne, one, r);
+            init64_products_kernel<<<nb[IK_PRODUCTS], 96, 0, st>>>(ev, ne, one, r);
+        }
+        init64_links_kernel<<<nb[IK_LINKS], 64, 0, st>>>(ev, ne, one);
+    } else {
+        line_smem(init_rows_kernel, rows);
+        line_smem(init_cols_kernel, cols);
+        line_smem(init_sheets_kernel, sheets);
+        for (int r = 0; r < rounds; r++) {
+            init_rows_kernel<<<nb[IK_ROWS], INIT_T, rows, st>>>(ev, ne, one, r);
+            init_cols_kernel<<<nb[IK_COLS], INIT_T, cols, st>>>(ev, ne, one, r);
+            init_sheets_kernel<<<nb[IK_SHEETS], INIT_T, sheets, st>>>(ev, ne, one, r);
+        }
+        if (grouped) init_groups_kernel<<<nb[IK_SITES], 128, 0, st>>>(ev, ne, one);
+        init_links_kernel<<<nb[IK_LINKS], 64, 0, st>>>(ev, ne, one);
+    }
     init_fields_kernel<<<nb[IK_SITES], 128, 0, st>>>(ev, ne, one);
 }
 

@@ -56,7 +56,7 @@ struct FFTables;  // ff.cuh
 // its line transforms, the split of the work, its scratch and the field slice
 // it fills.  begin[k]: its first block in launch k over several events.
 struct InitEv {
-    static constexpr int KINDS = 6;
+    static constexpr int KINDS = 7;
     int N, Ns, prec;
     int pow2, log2N, nrad, rad[12];
     int S, groups, per_group;  // sheets a round; groups of sheets multiplied apart
@@ -87,7 +87,7 @@ void launch_parts_convert(int prec, void* parts, int64_t np, double* stg, int to
 void launch_parts_validate(int prec, void* parts, int64_t np, int ns, int* d_bad, cudaStream_t st);
 // integrated p^tau of the particles <-> canonical [np] in the caller's order
 void launch_ptau_convert(int prec, void* parts, int64_t np, double* stg, int to_device, cudaStream_t st);
-size_t init_scratch_bytes(int N, int Ns);
+size_t init_scratch_bytes(int prec, int N, int Ns);
 void launch_convert(int prec, int which, int to_device, void* dev, double* staging, int N, int64_t np,
                     cudaStream_t st);
 // observables: per-species particle sums and field checks, FP64, fixed-order reductions

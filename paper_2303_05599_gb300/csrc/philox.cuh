@@ -36,7 +36,7 @@ __device__ __forceinline__ double u01(uint32_t r) { return ((double)r + 0.5) * (
 __device__ __forceinline__ void box_muller(double u1, double u2, double& z0, double& z1) {
     const double rad = sqrt(-2.0 * log(u1));
     double s, c;
-    sincospi(2.0 * u2, &s, &c);
+    sincos(2.0 * 3.14159265358979323846 * u2, &s, &c);
     z0 = rad * c;
     z1 = rad * s;
 }

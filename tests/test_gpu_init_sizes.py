@@ -19,8 +19,8 @@ def wl(N, Ns, prec=W.FP64, seed=9):
                       species=[W.Species(W.M_CHARM, 0.0, 50, W.REP_F, W.MOM_FIXED_PT, 0.5)])
 
 
-# (128, 16) takes two rounds of sheets; below 128 sites a side all sheets fit
-# one round and are multiplied in groups
+# (128, 16) takes several rounds of sheets; an FP32 event below 128 sites a side
+# takes one and multiplies groups of sheets apart
 @pytest.mark.parametrize("N,Ns", [(4, 3), (5, 1), (8, 50), (12, 7), (32, 50), (45, 4), (53, 2), (64, 6), (90, 2),
                                   (128, 16)])
 def test_initial_fields_against_the_oracle(N, Ns):
@@ -73,3 +73,14 @@ def test_init_beyond_the_longest_line_is_an_error():
     with pytest.raises(B.GlasmaError) as err:
         ev.glasma_init()
     assert err.value.status == B.GL_ERR_CUDA
+
+
+@pytest.mark.parametrize("N,Ns,value", [(8, 50, "0x1.94a390714d34ap-47"), (33, 1, "0x1.6ea1164352606p-48"),
+                                        (64, 6, "0x1.63c18e857b809p-47")])
+def test_fp64_links_keep_their_roundings(N, Ns, value):
+    """The unitarity a check reports for an FP64 event right after its initial
+    conditions is the sum of their roundings, so it is the same number as long
+    as the order of the operations is."""
+    ev = B.Event(wl(N, Ns))
+    ev.glasma_init()
+    assert ev.observables(B.GL_OBS_FIELDS).unitarity_max.hex() == value
