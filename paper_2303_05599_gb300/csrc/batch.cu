@@ -320,26 +320,26 @@ __global__ void __launch_bounds__(OBS_THREADS) batch_obs_kernel(const BObs* ev, 
                           d.partials + (size_t)b * GL_MAX_SPECIES * PO_N);
 }
 
-// One block per event: the final reductions of the requested parts (the
+// One warp per event and value: the final reductions of the requested parts (the
 // particle values, or zeros for an event without particles; the field checks)
 // into the event's obs row, by the function the single-event launches use,
 // and into all[n_events][OBS_W], so that the host reads every event's row
 // with one copy (the parts not requested are not copied: the host does not
 // read them).
 static constexpr int OBS_W = GL_MAX_SPECIES * PO_N + FO_N;
-static_assert(GL_MAX_SPECIES * PO_N <= OBS_FINAL_WARPS * OBS_FINAL_V && FO_N <= OBS_FINAL_WARPS * OBS_FINAL_V,
-              "obs_finalize_block takes at most OBS_FINAL_WARPS x OBS_FINAL_V values");
 __global__ void __launch_bounds__(OBS_FINAL_WARPS * 32) batch_obs_finish(const BObs* ev, uint32_t what, double* all) {
-    const BObs& d = ev[blockIdx.x];
-    double* row = all + (size_t)blockIdx.x * OBS_W;
-    if (what & GL_OBS_PARTICLES) {
-        if (d.nblocks > 0)
-            obs_finalize_block(d.partials, d.nblocks, GL_MAX_SPECIES * PO_N, ParticleObsKind(), d.out, row);
-        else
-            for (int k = threadIdx.x; k < GL_MAX_SPECIES * PO_N; k += blockDim.x) row[k] = 0.0;
+    constexpr int per_event = obs_final_blocks(OBS_W);
+    const int e = blockIdx.x / per_event;
+    const int k = (blockIdx.x - e * per_event) * OBS_FINAL_WARPS + (threadIdx.x >> 5), f = k - GL_MAX_SPECIES * PO_N;
+    if (k >= OBS_W) return;
+    const BObs& d = ev[e];
+    double* row = all + (size_t)e * OBS_W + k;
+    if (f < 0) {
+        if (what & GL_OBS_PARTICLES)
+            particle_finalize_value(d.partials, d.nblocks, d.nblocks > 0 ? d.oa.sp.n_species : 0, k, d.out + k, row);
+    } else if (what & GL_OBS_FIELDS) {
+        field_finalize_value(d.fo.partials, d.fo.nblocks, f, d.fo.out + f, row);
     }
-    if (what & GL_OBS_FIELDS)
-        obs_finalize_block(d.fo.partials, d.fo.nblocks, FO_N, FieldObsKind(), d.fo.out, row + GL_MAX_SPECIES * PO_N);
 }
 
 // tile shapes the autotuner chooses from
@@ -1410,7 +1410,7 @@ static gl_status obs_enqueue(gl_batch* b, uint32_t what, int k) {
     if (what & GL_OBS_FIELDS)
         launch_field_obs_events(b->prec, b->h_obs[0].fo, (const char*)b->d_obs + offsetof(BObs, fo), sizeof(BObs),
                                 b->ne, fblocks, false, b->stream);
-    batch_obs_finish<<<b->ne, OBS_FINAL_WARPS * 32, 0, b->stream>>>(b->d_obs, what, b->d_obs_all);
+    batch_obs_finish<<<b->ne * obs_final_blocks(OBS_W), OBS_FINAL_WARPS * 32, 0, b->stream>>>(b->d_obs, what, b->d_obs_all);
     cudaMemcpyAsync(b->p_rows[k], b->d_obs_all, sizeof(double) * OBS_W * b->ne, cudaMemcpyDeviceToHost, b->stream);
     cudaEventRecord(b->obs_done[k], b->stream);
     b->obs_what[k] = what;

@@ -39,10 +39,12 @@ __global__ void __launch_bounds__(FIELD_OBS_THREADS) field_obs_kernel(FieldObsEv
     field_obs_block_reduce(v, d.partials + (size_t)blk * FO_N);
 }
 
-// the FO_N values of event e in block e
+// the FO_N values of event e in block e, a warp each
 __global__ void __launch_bounds__(OBS_FINAL_WARPS * 32) field_obs_finalize(FieldObsEv one, const char* evs, size_t stride, int ne) {
     const FieldObsEv d = field_obs_event(one, ne > 0 ? evs : nullptr, stride, blockIdx.x);
-    obs_finalize_block(d.partials, d.nblocks, FO_N, FieldObsKind(), d.out);
+    const int k = threadIdx.x >> 5;
+    static_assert(FO_N <= OBS_FINAL_WARPS, "a warp each");
+    if (k < FO_N) field_finalize_value(d.partials, d.nblocks, k, d.out + k);
 }
 
 void launch_field_obs_events(int prec, const FieldObsEv& one, const void* evs, size_t stride, int ne, int blocks,

@@ -367,7 +367,7 @@ void launch_parts_convert(int prec, void* parts, int64_t np, double* stg, int to
 }
 
 // ------------------------------------------------------------ particle observables
-// one block per chunk of obs_chunk(np) particles, then one block for the final reduction
+// one block per chunk of obs_chunk(np) particles, then one warp per value for the final reduction
 template <typename R>
 __global__ void __launch_bounds__(OBS_THREADS) particle_obs_kernel(Parts<R> P, double t, uint32_t active, ObsArgs oa,
                                                                    double* partials) {
@@ -377,8 +377,10 @@ __global__ void __launch_bounds__(OBS_THREADS) particle_obs_kernel(Parts<R> P, d
     particle_obs_block<R>(P, t, active, oa, c0, c1, partials + (size_t)blockIdx.x * GL_MAX_SPECIES * PO_N);
 }
 
-__global__ void __launch_bounds__(OBS_FINAL_WARPS * 32) particle_obs_finalize(const double* partials, int nblocks, double* out) {
-    obs_finalize_block(partials, nblocks, GL_MAX_SPECIES * PO_N, ParticleObsKind(), out);
+__global__ void __launch_bounds__(OBS_FINAL_WARPS * 32) particle_obs_finalize(const double* partials, int nblocks,
+                                                                               int n_species, double* out) {
+    const int k = blockIdx.x * OBS_FINAL_WARPS + (threadIdx.x >> 5);
+    if (k < GL_MAX_SPECIES * PO_N) particle_finalize_value(partials, nblocks, n_species, k, out + k);
 }
 
 void launch_particle_obs(int prec, const void* parts, int64_t np, double t, uint32_t active_mask,
@@ -402,7 +404,7 @@ void launch_particle_obs(int prec, const void* parts, int64_t np, double t, uint
         particle_obs_kernel<float><<<blocks, OBS_THREADS, smem, st>>>(carve_parts<float>((void*)parts, np), t,
                                                                       active_mask, oa, partials);
     }
-    particle_obs_finalize<<<1, OBS_FINAL_WARPS * 32, 0, st>>>(partials, blocks, out);
+    particle_obs_finalize<<<obs_final_blocks(GL_MAX_SPECIES * PO_N), OBS_FINAL_WARPS * 32, 0, st>>>(partials, blocks, sp.n_species, out);
 }
 
 }  // namespace gl
