@@ -25,6 +25,14 @@ __device__ __forceinline__ double fmod_r<double>(double a, double b) { return fm
 template <>
 __device__ __forceinline__ float fmod_r<float>(float a, float b) { return fmodf(a, b); }
 
+// x on the periodic lattice; positions within it, nearly all, are what fmod would give them
+template <typename R>
+__device__ __forceinline__ R wrap_position(R x, R N) {
+    if (x >= R(0) && x < N) return x;
+    x = fmod_r<R>(x, N);
+    return x < R(0) ? x + N : x;
+}
+
 // temporal constraint (Sec. 3.1): one Euler step of p^tau from its own
 // equation of motion, started at the mass shell at the particle's first push
 // (NaN before).  Kept out of line, so that the arithmetic of the push itself
@@ -34,6 +42,36 @@ __device__ __noinline__ R ptau_step(R pt, R shell, R w, R t, R dt, R work) {
     if (pt != pt) pt = shell;
     const R drift = (t > R(0) && shell > R(0)) ? w * w / (t * shell) : R(0);
     return pt + dt * (work - drift);
+}
+
+// e^{-i s phi} Q e^{i s phi}.  FP64: the exponential and the transport.
+__device__ __forceinline__ A8<double> rapidity_rotation(const A8<double>& ph, double s, const A8<double>& q) {
+    return conj_up_t(exp_i_alg<double>(ph, -s), q);
+}
+// FP32: the rotation is that of Q's eight components by exp(s ad), whose series
+// Q - s i[phi, Q] + ... needs K terms where |s phi|^(K+1) / (K+1)! <= 2^-25 (ad's
+// largest eigenvalue is at most |phi|, the length of SU(3)'s roots being 1).  A
+// step turns Q by dt / t v_w phi, 1e-4 .. 1e-2 for most particles, and a term
+// takes 80 operations, the exponential and the transport about 320, so angles
+// to 0.08 (four terms) take the series.  The push is bound by memory where the
+// particles are few a cell (30 x 256^2: 0.216 ms with either), and by issue as
+// well on 1024^2 with 4 a cell: 0.212 -> 0.203 ms.
+__device__ __forceinline__ A8<float> rapidity_rotation(const A8<float>& ph, float s, const A8<float>& q) {
+    const float x2 = s * s * a_dot(ph, ph);
+    if (!(x2 <= 6.6e-3f)) return conj_up_t(exp_i_alg<float>(ph, -s), q);
+    const float terms = x2 <= 5.9e-8f ? 1.f : x2 <= 3.1e-5f ? 2.f : x2 <= 8.4e-4f ? 3.f : 4.f;
+    A8<float> o = q, t = q;
+#pragma unroll 1
+    for (float k = 1.f; k <= terms; k += 1.f) {
+        const float f = k == 1.f ? -s : k == 2.f ? -0.5f * s : k == 3.f ? s * (-1.f / 3) : -0.25f * s;
+        t = icomm(ph, t);
+#pragma unroll
+        for (int a = 0; a < 8; a++) {
+            t.v[a] *= f;
+            o.v[a] += t.v[a];
+        }
+    }
+    return o;
 }
 
 // Euler + CPIC update of particle i (Sec. 3.1 and 3.2); site: site fields at
@@ -73,11 +111,9 @@ __device__ __forceinline__ void push_one(const typename Prec<R>::V* __restrict__
         p.px += dt * qEx;
         p.py += dt * (qEy - qBe);
         p.Pe += dt * (qEe + qBy);
-        R xn = p.x + dt;
+        const R xn = p.x + dt;
         const int jxu = (int)floor_r<R>(xn + R(0.5));
-        xn = fmod_r<R>(xn, (R)N);
-        if (xn < R(0)) xn += (R)N;
-        p.x = xn;
+        p.x = wrap_position(xn, (R)N);
         if (jxu != ixu) p.q = conj_dn(load_link(bn1.U, 0, cell, Vn), p.q);
         P.store_cs(i, p);
         return;
@@ -96,18 +132,14 @@ __device__ __forceinline__ void push_one(const typename Prec<R>::V* __restrict__
     const R dpy = qEy - qBe * vx + qBx * vw;
     const R dPe = t * (qEe - qBx * vy + qBy * vx);
     const R deta = dt_over_t * vw;
-    R xn = p.x + dt * vx, yn = p.y + dt * vy;
+    const R xn = p.x + dt * vx, yn = p.y + dt * vy;
     p.eta += deta;
     p.px += dt * dpx;
     p.py += dt * dpy;
     p.Pe += dt * dPe;
     const int jxu = (int)floor_r<R>(xn + R(0.5)), jyu = (int)floor_r<R>(yn + R(0.5));
-    xn = fmod_r<R>(xn, (R)N);
-    if (xn < R(0)) xn += (R)N;
-    yn = fmod_r<R>(yn, (R)N);
-    if (yn < R(0)) yn += (R)N;
-    p.x = xn;
-    p.y = yn;
+    p.x = wrap_position(xn, (R)N);
+    p.y = wrap_position(yn, (R)N);
     // CPIC: rotate with the crossed links at t_{n+1}, x first, then y.  A step
     // up takes U^+ Q U with the link of the old cell, a step down U Q U^+ =
     // (U^+)^+ Q U^+ with the link of the new cell.  Each lane has up to two
@@ -132,7 +164,7 @@ __device__ __forceinline__ void push_one(const typename Prec<R>::V* __restrict__
     // rapidity Wilson line at the new cell: Q <- e^{-i deta phi} Q e^{+i deta phi}
     if (deta != R(0)) {
         const A8<R> ph = load_alg(bn1.phi, (int64_t)jy * N + jx, Vn);
-        p.q = conj_up_t(exp_i_alg<R>(ph, -deta), p.q);
+        p.q = rapidity_rotation(ph, deta, p.q);
     }
     P.store_cs(i, p);
 }
