@@ -381,11 +381,12 @@ __device__ __forceinline__ M3<R> sq_herm(const M3<R>& X) {
             R sr = R(0), si = R(0);
 #pragma unroll
             for (int k = 0; k < 3; k++) {
+                // the diagonal entries are real
                 sr = fma(X.re[i][k], X.re[k][j], sr);
-                sr = fma(-X.im[i][k], X.im[k][j], sr);
+                if (k != i && k != j) sr = fma(-X.im[i][k], X.im[k][j], sr);
                 if (i != j) {
-                    si = fma(X.re[i][k], X.im[k][j], si);
-                    si = fma(X.im[i][k], X.re[k][j], si);
+                    if (k != j) si = fma(X.re[i][k], X.im[k][j], si);
+                    if (k != i) si = fma(X.im[i][k], X.re[k][j], si);
                 }
             }
             Z.re[i][j] = sr;
