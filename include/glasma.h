@@ -262,8 +262,8 @@ gl_status gl_step_coupled(gl_ctx* ctx, int32_t n_steps);
 /* Choose the launch shape of the field kernel and the push block size (64,
  * 128, 256) for this context from timed trial launches.  FP32 field shapes
  * (the strip kernel: a warp walks up a strip of 32 columns): 0 = 16 warps per
- * SM, 1 = 12, 2 = 8 (more registers per thread each).  FP64 tiles: 1 = 32x4,
- * 2 = 32x2.  Results do not depend on the shape.  Waits.  Needs the
+ * SM, 1 = 12, 2 = 8 (more registers per thread each).  FP64 tiles: 1 = 16x8
+ * sites, 2 = 32x2.  Results do not depend on the shape.  Waits.  Needs the
  * particles at the fields' time; the trials write only buffers that the next
  * coupled step rewrites.  Outputs may be NULL. */
 gl_status gl_autotune(gl_ctx* ctx, int32_t* tile_shape, int32_t* push_block);
@@ -335,7 +335,7 @@ gl_status gl_batch_init(gl_batch* batch);
 /* Choose the launch shapes and the step schedule from timed trial launches
  * that do not change the state (waits).  Chosen: the field launch shape (FP32
  * strips: 0 = 16 warps per SM, 1 = 12, 2 = 8, the rows of all events' strips
- * split evenly among the resident warps; FP64 batches use the 32x4 tile, 1),
+ * split evenly among the resident warps; FP64 batches use the 16x8 tile, 1),
  * by the whole step as for the push; the block size (128,
  * 256, 512) and chunk (particles per block: 128, 256, 512, 1024) of the
  * separate push kernel, by the time of the whole overlapped step, not of the
@@ -344,7 +344,7 @@ gl_status gl_batch_init(gl_batch* batch);
  *     chunk of particles or (push_grid 1, 2) that many resident 128-thread
  *     blocks per SM launched ahead of the field kernel (chunks of 1024), or
  *   - one persistent fused launch that interleaves field items (FP32: 24
- *     rows of a strip for each of a block's 8 warps; FP64: 32x4 tiles) and
+ *     rows of a strip for each of a block's 8 warps; FP64: 16x8 tiles) and
  *     push chunks of 512, 1024 or 2048 particles.
  * The push and whole-step trials run on copies of the particles in the spare
  * particle buffers that sorting provides; if an event with particles has
@@ -354,7 +354,7 @@ gl_status gl_batch_autotune(gl_batch* batch, int32_t* tile_shape, int32_t* push_
 /* Set the launch shapes and schedule directly (values as above: push_chunk
  * 128, 256, 512, 1024 or 2048; fused 0 or 1; push_grid 0, 1 or 2, ignored
  * when fused).  Results do not depend on them.
- * GL_ERR_ARG for other values or a tile other than 32x4 (1) in an FP64 batch. */
+ * GL_ERR_ARG for other values or a tile other than 1 in an FP64 batch. */
 gl_status gl_batch_set_launch(gl_batch* batch, int32_t tile_shape, int32_t push_block, int32_t push_chunk,
                               int32_t fused, int32_t push_grid);
 

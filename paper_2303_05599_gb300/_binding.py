@@ -107,7 +107,7 @@ SIGNATURES = {
 
 GL_NOALLOC_MAX_PARTICLES = 2097152
 GL_OBS_PARTICLES, GL_OBS_FIELDS, GL_OBS_ALL = 1, 2, 3
-BATCH_TILES = ("32x8", "32x4", "32x16")   # FP64 field tiles of a batch (32x4 is the one used)
+BATCH_TILES = ("32x8", "32x4", "32x16")   # FP64 field tiles of a batch ("32x4" names the one used, of 16x8 sites)
 # FP32 field launch shapes of the strip kernel: resident warps per SM
 STRIP_SHAPES = ("strip16", "strip12", "strip8")
 

@@ -191,12 +191,12 @@ __device__ __forceinline__ void push_item(const BatchArgs& b, int lag, int blk) 
 }
 
 template <typename R, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY, (Tile<R, TX, TY>::min_blocks)) batch_field_kernel(BatchArgs b) {
+__global__ void __launch_bounds__(TX * TY) batch_field_kernel(BatchArgs b) {
     field_item<R, TX, TY>(b, blockIdx.x);
 }
 
 __global__ void __launch_bounds__(SmallTile::NT) batch_small_kernel(BatchArgs b) {
-    field_item<double, 32, 4, true>(b, blockIdx.x);
+    field_item<double, TILE64_X, TILE64_Y, true>(b, blockIdx.x);
 }
 
 // FP32 field step of the whole batch: blocks of up to WPB warps take as many
@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(256, 1) batch_fused_strip_kernel(BatchArgs b, 
 }
 
 template <typename R, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY, (Tile<R, TX, TY>::min_blocks))
+__global__ void __launch_bounds__(TX * TY)
     batch_fused_kernel(BatchArgs b, int lag, int n_field, int n_small, int n_push) {
     const int64_t fields = (int64_t)n_field + n_small, total = fields + n_push;
     for (int64_t w = blockIdx.x; w < total; w += gridDim.x) {
@@ -342,9 +342,8 @@ __global__ void __launch_bounds__(OBS_FINAL_WARPS * 32) batch_obs_finish(const B
     }
 }
 
-// tile shapes the autotuner chooses from
+// launch shapes (FP64 takes the second only, whose tile of 128 sites is TILE64_X x TILE64_Y)
 enum { TILE_32x8 = 0, TILE_32x4 = 1, TILE_32x16 = 2, N_TILES = 3 };
-static const int TILE_DIMS[N_TILES][2] = {{32, 8}, {32, 4}, {32, 16}};
 static const int PUSH_BLOCKS[3] = {128, 256, 512};
 enum { N_CHUNKS = 3 };
 static const int PUSH_CHUNKS[N_CHUNKS] = {512, 1024, 2048};  // fused launch
@@ -404,11 +403,11 @@ static void strip_shape_geometry(int tile, int* wpb, int* warps_sm) {
 template <typename R>
 static void launch_batch_field(int tile, int blocks, int64_t nseg, const BatchArgs& b, cudaStream_t st) {
     if constexpr (sizeof(R) == 8) {
-        // FP64: the 32x4 tile only (shared memory), and the small lattices'
+        // FP64: the one tile, and the small lattices'
         // tiles (nseg of them) in a launch of their own, six blocks an SM
         (void)tile;
-        set_smem_attr<R, 32, 4>();
-        if (blocks > 0) batch_field_kernel<R, 32, 4><<<blocks, 128, Tile<R, 32, 4>::bytes, st>>>(b);
+        set_smem_attr<R, TILE64_X, TILE64_Y>();
+        if (blocks > 0) batch_field_kernel<R, TILE64_X, TILE64_Y><<<blocks, 128, Tile<R, TILE64_X, TILE64_Y>::bytes, st>>>(b);
         if (nseg > 0) batch_small_kernel<<<(unsigned)nseg, SmallTile::NT, sizeof(SmallTile), st>>>(b);
     } else if (tile == 1) {
         launch_strip_shape<12, 1>(nseg, b, st);
@@ -472,7 +471,7 @@ static void launch_batch_fused(int tile, const BatchArgs& b, int lag, int n_fiel
                                cudaStream_t st) {
     if constexpr (sizeof(R) == 8) {
         (void)tile;
-        launch_fused_t<R, 32, 4>(b, lag, n_field, (int)nseg, n_push, st);
+        launch_fused_t<R, TILE64_X, TILE64_Y>(b, lag, n_field, (int)nseg, n_push, st);
     } else {
         (void)tile;
         (void)n_field;
@@ -800,7 +799,7 @@ gl_status gl_batch_init(gl_batch* b) {
 static gl_status sync_desc(gl_batch* b) {
     int tb = 0, cb = 0;
     int64_t rb = 0;
-    const int TX = TILE_DIMS[b->tile][0], TY = TILE_DIMS[b->tile][1];
+    const int TX = TILE64_X, TY = TILE64_Y;
     int64_t step0 = -1, tiles_all = 0;
     const int sms = b->prec == GL_FP64 ? sm_count() : 0;
     for (int e = 0; e < b->ne && b->prec == GL_FP64; e++) {
@@ -1160,7 +1159,7 @@ gl_status gl_batch_step(gl_batch* b, int32_t n_steps) {
     if (n_steps == 0) return GL_OK;
     if (gl_status s = sync_desc(b)) return s;
     if (gl_status s = ensure_aux(b)) return s;
-    if (b->prec == GL_FP64) set_smem_attr<double, 32, 4>();
+    if (b->prec == GL_FP64) set_smem_attr<double, TILE64_X, TILE64_Y>();
     // (re)capture the overlapped step when the launch shapes changed
     if (!b->exec || b->graph_tile != b->tile || b->graph_push_block != b->push_block ||
         b->graph_push_chunk != b->push_chunk || b->graph_fused != b->fused || b->graph_push_grid != b->push_grid ||

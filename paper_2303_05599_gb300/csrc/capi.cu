@@ -676,7 +676,7 @@ gl_status gl_autotune(gl_ctx* c, int32_t* tile_out, int32_t* push_block_out) {
     };
     // field kernel: writes only the spare time slice and the site fields at
     // the current time, both of which the next coupled step rewrites
-    // FP64: tiles 32x4 (1) and 32x2 (2); FP32: strip shapes 0, 1, 2, each with
+    // FP64: tiles 16x8 (1) and 32x2 (2); FP32: strip shapes 0, 1, 2, each with
     // the cost model's segment length, its half and double, and 16 rows
     const int tiles[4] = {0, 1, 2, 3};
     float best = 1e30f;

@@ -1,7 +1,7 @@
 // Fused Glasma leapfrog step and site E/B interpolation (Sec. 2.1 and 3.2 of
 // arXiv:2303.05599) on shared-memory tiles.
 //
-// One CTA owns a TX x TY tile of sites (TX = 32: one warp per tile row).  Per
+// One CTA owns a TX x TY tile of sites (FP64; FP32 has strip_body.cuh).  Per
 // step it computes, from U(n), phi(n), e(n-1/2), pi(n-1/2):
 //   the momenta e(n+1/2), pi(n+1/2), the links U(n+1) and the scalar phi(n+1),
 //   and the site fields E, B at t_n that the particle push gathers.
@@ -16,16 +16,21 @@
 // one halo row (y0 - 1); nothing else of the halo is needed.
 //
 // The tile's inputs are copied to shared memory with cp.async in the storage
-// layout of global memory (16-byte vectors; FP32 links as two rows, the third
-// rebuilt when a link is read).  Regions, in tile coordinates:
+// layout of global memory (16-byte vectors).  Regions, in tile coordinates:
 //   links, phi:                   x in [-1, TX],   y in [-1, TY]    (LW x LH)
 //   plaquettes A, momenta, Lf:    x in [-1, TX-1], y in [-1, TY-1]  (EW x EH)
 // pi(n-1/2) is read by each site's thread straight from global memory.
 //
-// Every site does each computation at the same point of the code (own and
-// halo momenta share one loop body), so the results do not depend on the tile
-// shape.  The links arrive in their own group of copies, so the plaquettes
-// start while phi and e(n-1/2) are still in flight.
+// Bound by the FP64 pipe, which a warp instruction keeps for 64 cycles however
+// many of its lanes work, so the halo's work is packed: its plaquettes are
+// spread a matrix row a thread, its two kinds of transports over two warps.  A
+// 16x8 tile has 25 plaquettes and 24 momenta beyond its own 128 sites (32x4: 37
+// and 36, which took two and a half warps' passes of their own, a momentum's
+// both directions one after the other): nine events of 64/128/256 1283 -> 1164
+// us, a 256^2 event 379 -> 336 us; 32x4 tiles with the packed halo 1322 and 375.
+// Every operation whose fusion would depend on what surrounds it is explicit, so
+// the results do not depend on the tile shape.  The links arrive in their own
+// group of copies, so the plaquettes start while phi and e(n-1/2) are in flight.
 #pragma once
 #include "internal.h"
 #include "layout.cuh"
@@ -40,17 +45,11 @@ struct Tile {
     static constexpr int EW = TX + 1, EH = TY + 1, EN = EW * EH;
     static constexpr int NT = TX * TY;
     static constexpr int NH = TX + TY;  // halo momenta: left column (e_x), bottom row (e_y, Lf)
-    static_assert(NH <= NT, "halo momenta are one per thread");
-    // vectors: links 2 LP LN, phi AP LN, A AP EN, e sums 2 AP EN, Lf AP EN
-    static constexpr size_t vecs = (size_t)2 * LP * LN + (size_t)AP * LN + (size_t)4 * AP * EN;
-    // FP32 two-row links: the third rows, rebuilt once per staged link,
-    // [2][3][LN] float2 after the vectors
-    static constexpr size_t row2_bytes = sizeof(R) == 4 ? (size_t)2 * 3 * LN * 8 : 0;
-    static constexpr size_t bytes = vecs * sizeof(V) + row2_bytes;
-    // CTAs per SM the launch bounds ask for: FP32 kernels are capped at 128
-    // registers a thread so that 16 warps fit an SM (the shared memory of
-    // 32x4: 4 CTAs, 32x8: 2, 32x16: 1); FP64 tiles take one CTA
-    static constexpr int min_blocks = sizeof(R) == 8 ? 1 : (NT >= 512 ? 1 : 512 / NT);
+    static constexpr int REST = EN - NT;  // plaquettes beyond one a thread
+    static_assert(9 * REST <= AP * EN, "their matrices wait in the place of Lf");
+    // vectors: links 2 LP LN, phi AP LN, A AP EN, e sums 2 AP EN, Lf AP EN, halo items AP (NH + TY)
+    static constexpr size_t vecs = (size_t)2 * LP * LN + (size_t)AP * LN + (size_t)4 * AP * EN + (size_t)AP * (NH + TY);
+    static constexpr size_t bytes = vecs * sizeof(V);
 };
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
@@ -76,19 +75,8 @@ __device__ __forceinline__ M3<double> s_link(const double2* sU, int d, int li, i
     }
     return m;
 }
-__device__ __forceinline__ M3<float> s_link(const float4* sU, int d, int li, int LN) {
-    const float4* b = sU + (size_t)d * 3 * LN + li;
-    const float4 a = b[0], c = b[LN], e = b[2 * LN];
-    M3<float> m;
-    m.re[0][0] = a.x; m.im[0][0] = a.y; m.re[0][1] = a.z; m.im[0][1] = a.w;
-    m.re[0][2] = c.x; m.im[0][2] = c.y; m.re[1][0] = c.z; m.im[1][0] = c.w;
-    m.re[1][1] = e.x; m.im[1][1] = e.y; m.re[1][2] = e.z; m.im[1][2] = e.w;
-    rebuild_row2(m);
-    return m;
-}
 
-// links of the tile in shared memory; FP32 links come with their third rows
-// stored beside them (rebuilt once when staged)
+// links of the tile in shared memory
 template <typename R>
 struct SLinks;
 template <>
@@ -97,26 +85,6 @@ struct SLinks<double> {
     int LN;
     __device__ __forceinline__ M3<double> operator()(int d, int li) const { return s_link(u, d, li, LN); }
 };
-template <>
-struct SLinks<float> {
-    const float4* u;
-    const float2* r2;
-    int LN;
-    __device__ __forceinline__ M3<float> operator()(int d, int li) const {
-        const float4* b = u + (size_t)d * 3 * LN + li;
-        const float4 a = b[0], c = b[LN], e = b[2 * LN];
-        const float2* t = r2 + (size_t)d * 3 * LN + li;
-        const float2 f0 = t[0], f1 = t[LN], f2 = t[2 * LN];
-        M3<float> m;
-        m.re[0][0] = a.x; m.im[0][0] = a.y; m.re[0][1] = a.z; m.im[0][1] = a.w;
-        m.re[0][2] = c.x; m.im[0][2] = c.y; m.re[1][0] = c.z; m.im[1][0] = c.w;
-        m.re[1][1] = e.x; m.im[1][1] = e.y; m.re[1][2] = e.z; m.im[1][2] = e.w;
-        m.re[2][0] = f0.x; m.im[2][0] = f0.y; m.re[2][1] = f1.x; m.im[2][1] = f1.y;
-        m.re[2][2] = f2.x; m.im[2][2] = f2.y;
-        return m;
-    }
-};
-
 __device__ __forceinline__ A8<double> s_alg(const double2* s, int i, int n) {
     A8<double> x;
 #pragma unroll
@@ -127,58 +95,10 @@ __device__ __forceinline__ A8<double> s_alg(const double2* s, int i, int n) {
     }
     return x;
 }
-__device__ __forceinline__ A8<float> s_alg(const float4* s, int i, int n) {
-    const float4 a = s[i], b = s[n + i];
-    A8<float> x;
-    x.v[0] = a.x; x.v[1] = a.y; x.v[2] = a.z; x.v[3] = a.w;
-    x.v[4] = b.x; x.v[5] = b.y; x.v[6] = b.z; x.v[7] = b.w;
-    return x;
-}
 __device__ __forceinline__ void s_alg_put(double2* s, int i, int n, const A8<double>& x) {
 #pragma unroll
     for (int k = 0; k < 4; k++) s[k * n + i] = make_double2(x.v[2 * k], x.v[2 * k + 1]);
 }
-__device__ __forceinline__ void s_alg_put(float4* s, int i, int n, const A8<float>& x) {
-    s[i] = make_float4(x.v[0], x.v[1], x.v[2], x.v[3]);
-    s[n + i] = make_float4(x.v[4], x.v[5], x.v[6], x.v[7]);
-}
-
-// FP64 Gram-Schmidt of rows 0 and 1 (FP32 links are stored as two rows)
-__device__ __forceinline__ void reunit(M3<float>& u) {
-    double r0r[3], r0i[3], r1r[3], r1i[3];
-#pragma unroll
-    for (int j = 0; j < 3; j++) {
-        r0r[j] = u.re[0][j]; r0i[j] = u.im[0][j];
-        r1r[j] = u.re[1][j]; r1i[j] = u.im[1][j];
-    }
-    double n0 = 0;
-#pragma unroll
-    for (int j = 0; j < 3; j++) n0 += r0r[j] * r0r[j] + r0i[j] * r0i[j];
-    n0 = 1.0 / sqrt(n0);
-#pragma unroll
-    for (int j = 0; j < 3; j++) { r0r[j] *= n0; r0i[j] *= n0; }
-    double cr = 0, ci = 0;
-#pragma unroll
-    for (int j = 0; j < 3; j++) {
-        cr += r0r[j] * r1r[j] + r0i[j] * r1i[j];
-        ci += r0r[j] * r1i[j] - r0i[j] * r1r[j];
-    }
-#pragma unroll
-    for (int j = 0; j < 3; j++) {
-        r1r[j] -= cr * r0r[j] - ci * r0i[j];
-        r1i[j] -= cr * r0i[j] + ci * r0r[j];
-    }
-    double n1 = 0;
-#pragma unroll
-    for (int j = 0; j < 3; j++) n1 += r1r[j] * r1r[j] + r1i[j] * r1i[j];
-    n1 = 1.0 / sqrt(n1);
-#pragma unroll
-    for (int j = 0; j < 3; j++) {
-        u.re[0][j] = (float)r0r[j]; u.im[0][j] = (float)r0i[j];
-        u.re[1][j] = (float)(r1r[j] * n1); u.im[1][j] = (float)(r1i[j] * n1);
-    }
-}
-__device__ __forceinline__ void reunit(M3<double>&) {}
 
 struct StepArgs {
     int N;
@@ -215,6 +135,40 @@ __device__ __forceinline__ R next_e(R e, R F, R c, R t, R dt, R inv_t) {
     return fma(dt, fma(t, F, mul_rn(inv_t, c)), e);
 }
 
+// a row of a matrix product, q = p m and q = p m^+, in the order of mul and mul_nd
+template <typename R>
+__device__ __forceinline__ void row_mul(const R* pr, const R* pi, const M3<R>& m, R* qr, R* qi) {
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        R sr = 0, si = 0;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            sr = fma(pr[k], m.re[k][j], sr);
+            sr = fma(-pi[k], m.im[k][j], sr);
+            si = fma(pr[k], m.im[k][j], si);
+            si = fma(pi[k], m.re[k][j], si);
+        }
+        qr[j] = sr;
+        qi[j] = si;
+    }
+}
+template <typename R>
+__device__ __forceinline__ void row_mul_dag(const R* pr, const R* pi, const M3<R>& m, R* qr, R* qi) {
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+        R sr = 0, si = 0;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            sr = fma(pr[k], m.re[j][k], sr);
+            sr = fma(pi[k], m.im[j][k], sr);
+            si = fma(pi[k], m.re[j][k], si);
+            si = fma(-pr[k], m.im[j][k], si);
+        }
+        qr[j] = sr;
+        qi[j] = si;
+    }
+}
+
 // one tile (index `tile` of a lattice with tiles_x tiles per row); the caller
 // provides the dynamic shared memory of Tile<R, TX, TY>::bytes
 template <typename R, int TX, int TY>
@@ -223,17 +177,15 @@ __device__ __forceinline__ void fused_tile(const Fields<R>& in, const Fields<R>&
     using T = Tile<R, TX, TY>;
     using Vec = typename Prec<R>::V;
     constexpr int LP = T::LP, AP = T::AP;
-    constexpr int LW = T::LW, LN = T::LN, EW = T::EW, EN = T::EN, NT = T::NT, NH = T::NH;
+    constexpr int LW = T::LW, LN = T::LN, EW = T::EW, EN = T::EN, NT = T::NT, NH = T::NH, REST = T::REST;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Vec* sU = (Vec*)smem_raw;          // [2][LP][LN]
     Vec* sPhi = sU + 2 * LP * LN;      // [AP][LN]
     Vec* sA = sPhi + AP * LN;          // [AP][EN]
     Vec* sEs = sA + AP * EN;           // [2][AP][EN]: e(n-1/2), then e(n-1/2) + e(n+1/2)
     Vec* sLf = sEs + 2 * AP * EN;      // [AP][EN]
-    float2* sU2 = (float2*)(smem_raw + T::vecs * sizeof(Vec));  // FP32: [2][3][LN] third rows
-    SLinks<R> lk;
-    if constexpr (sizeof(R) == 4) lk = SLinks<R>{(const float4*)sU, sU2, LN};
-    else lk = SLinks<R>{(const double2*)sU, LN};
+    Vec* sHalo = sLf + AP * EN;        // [AP][NH] scalar currents, [AP][TY] transported plaquettes of the left column
+    const SLinks<R> lk{sU, LN};
 
     const int N = a.N;
     const int64_t Vn = (int64_t)N * N;
@@ -267,96 +219,114 @@ __device__ __forceinline__ void fused_tile(const Fields<R>& in, const Fields<R>&
     }
     cp_async_commit();
     cp_async_wait_group<1>();
-    if constexpr (sizeof(R) == 4) {
-        // third rows of the links this thread copied (its own copies are
-        // complete after the wait), once per staged link
-        for (int i = tid; i < LN; i += NT)
-#pragma unroll
-            for (int d = 0; d < 2; d++) {
-                const M3<float> m = s_link((const float4*)sU, d, i, LN);
-#pragma unroll
-                for (int k = 0; k < 3; k++)
-                    sU2[(size_t)(d * 3 + k) * LN + i] = make_float2(m.re[2][k], m.im[2][k]);
-            }
-    }
     __syncthreads();
 
-    // ---- phase 2: plaquettes of the cells x in [-1, TX-1], y in [-1, TY-1]
-    for (int i = tid; i < EN; i += NT) {
-        const int l = (i / EW) * LW + (i % EW);  // cell (i % EW - 1, i / EW - 1)
+    // ---- phase 2: plaquettes of the cells x in [-1, TX-1], y in [-1, TY-1]:
+    // one a thread, and of the REST that are left a row of the matrix a thread
+    // (in the place of Lf), so that they fill warps
+    for (int i = tid; i < 3 * REST; i += NT) {
+        const int r = i / REST, j = i - r * REST, c = NT + j, l = (c / EW) * LW + (c % EW);
+        R pr[3], pi[3], qr[3], qi[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const Vec v = sU[(size_t)(r * 3 + k) * LN + l];
+            pr[k] = v.x;
+            pi[k] = v.y;
+        }
+        row_mul(pr, pi, lk(1, l + 1), qr, qi);
+        row_mul_dag(qr, qi, lk(0, l + LW), pr, pi);
+        row_mul_dag(pr, pi, lk(1, l), qr, qi);
+#pragma unroll
+        for (int k = 0; k < 3; k++) sLf[(size_t)(r * 3 + k) * REST + j] = Vec{qr[k], qi[k]};
+    }
+    {
+        const int l = (tid / EW) * LW + (tid % EW);  // cell (tid % EW - 1, tid / EW - 1)
         const M3<R> C = mul(lk(0, l), lk(1, l + 1));
-        s_alg_put(sA, i, EN, iah_of_mul_nd(mul_nd(C, lk(0, l + LW)), lk(1, l)));
+        s_alg_put(sA, tid, EN, iah_of_mul_nd(mul_nd(C, lk(0, l + LW)), lk(1, l)));
     }
     cp_async_wait_group<0>();
     __syncthreads();
+    for (int j = tid; j < REST; j += NT) {
+        M3<R> P;
+#pragma unroll
+        for (int k = 0; k < 9; k++) {
+            const Vec v = sLf[(size_t)k * REST + j];
+            P.re[k / 3][k % 3] = v.x;
+            P.im[k / 3][k % 3] = v.y;
+        }
+        s_alg_put(sA, NT + j, EN, iah_to_alg(P));
+    }
+    __syncthreads();
 
     // ---- phase 3: momenta at n+1/2 of the tile site (kept in registers for
-    // phase 4) and of the halo.  Item 0 is the thread's own site (both components); item 1, for the first
-    // NH threads, a halo site: left column (-1, h) needs e_x only, bottom row
-    // (h, -1) e_y and Lf only.  One loop body (not unrolled) computes both, so
-    // a momentum is computed by the same code whether the site is a tile's
-    // own or another tile's halo.
+    // phase 4) and of the halo: bottom row (h, -1), e_y and Lf only, and left
+    // column (-1, h), e_x only.  A halo item's transport of the plaquette and its
+    // scalar current go to two warps, its update follows the barrier.  Each
+    // operation rounds alike wherever it stands (explicit fused operations), so a
+    // momentum is the same bits whether the site is a tile's own or another's halo.
     A8<R> my_ex, my_ey, my_tx, my_ty, my_b;
     const int gx = x0 + ix, gy = y0 + iy;
     const bool valid = gx < N && gy < N;
     const int64_t g = (int64_t)gy * N + gx;
-    const int n_items = tid < NH ? 2 : 1;
-#pragma unroll 1
-    for (int it = 0; it < n_items; it++) {
-        int e = es, l = ls;
-        bool wx = true, wy = true;
-        if (it == 1) {
-            if (tid < TY) {
-                e = (tid + 1) * EW;
-                l = (tid + 1) * LW;
-                wy = false;
-            } else {
-                e = tid - TY + 1;
-                l = tid - TY + 1;
-                wx = false;
-            }
-        }
-        const A8<R> A0 = s_alg(sA, e, EN);
-        const A8<R> ph = s_alg(sPhi, l, LN);
-        if (wx) {
-            const A8<R> Dn = conj_dn_t(lk(1, l - LW), s_alg(sA, e - EW, EN));
-            const A8<R> tx = conj_up_t(lk(0, l), s_alg(sPhi, l + 1, LN));
-            const A8<R> cx = icomm(tx, ph);
-            const A8<R> eox = s_alg(sEs, e, EN);
-            A8<R> ex_n, sx;
+    {
+        const A8<R> A0 = s_alg(sA, es, EN);
+        const A8<R> ph = s_alg(sPhi, ls, LN);
+        A8<R> sum;
+        const A8<R> Dn = conj_dn_t(lk(1, ls - LW), s_alg(sA, es - EW, EN));
+        my_tx = conj_up_t(lk(0, ls), s_alg(sPhi, ls + 1, LN));
+        const A8<R> cx = icomm(my_tx, ph);
+        const A8<R> eox = s_alg(sEs, es, EN);
 #pragma unroll
-            for (int c = 0; c < 8; c++) {
-                ex_n.v[c] = next_e(eox.v[c], A0.v[c] - Dn.v[c], cx.v[c], t, dt, inv_t);
-                sx.v[c] = eox.v[c] + ex_n.v[c];
-            }
-            // only this thread reads site e of sEs before the barrier
-            s_alg_put(sEs, e, EN, sx);
-            if (it == 0) {
-                my_ex = ex_n;
-                my_tx = tx;
-                my_b = Dn;
-            }
+        for (int c = 0; c < 8; c++) {
+            my_ex.v[c] = next_e(eox.v[c], A0.v[c] - Dn.v[c], cx.v[c], t, dt, inv_t);
+            sum.v[c] = eox.v[c] + my_ex.v[c];
         }
-        if (wy) {
-            const A8<R> Lf = conj_dn_t(lk(0, l - 1), s_alg(sA, e - 1, EN));
-            const A8<R> ty = conj_up_t(lk(1, l), s_alg(sPhi, l + LW, LN));
-            const A8<R> cy = icomm(ty, ph);
-            const A8<R> eoy = s_alg(sEs + AP * EN, e, EN);
-            A8<R> ey_n, sy;
+        // only this thread reads site es of sEs before the barrier
+        s_alg_put(sEs, es, EN, sum);
+        const A8<R> Lf = conj_dn_t(lk(0, ls - 1), s_alg(sA, es - 1, EN));
+        my_ty = conj_up_t(lk(1, ls), s_alg(sPhi, ls + LW, LN));
+        const A8<R> cy = icomm(my_ty, ph);
+        const A8<R> eoy = s_alg(sEs + AP * EN, es, EN);
 #pragma unroll
-            for (int c = 0; c < 8; c++) {
-                ey_n.v[c] = next_e(eoy.v[c], Lf.v[c] - A0.v[c], cy.v[c], t, dt, inv_t);
-                sy.v[c] = eoy.v[c] + ey_n.v[c];
-            }
-            s_alg_put(sEs + AP * EN, e, EN, sy);
-            s_alg_put(sLf, e, EN, Lf);
-            if (it == 0) {
-                my_ey = ey_n;
-                my_ty = ty;
-#pragma unroll
-                for (int c = 0; c < 8; c++) my_b.v[c] = A0.v[c] + Lf.v[c] + my_b.v[c];
-            }
+        for (int c = 0; c < 8; c++) {
+            my_ey.v[c] = next_e(eoy.v[c], Lf.v[c] - A0.v[c], cy.v[c], t, dt, inv_t);
+            sum.v[c] = eoy.v[c] + my_ey.v[c];
+            my_b.v[c] = A0.v[c] + Lf.v[c] + Dn.v[c];
         }
+        s_alg_put(sEs + AP * EN, es, EN, sum);
+        s_alg_put(sLf, es, EN, Lf);
+    }
+    constexpr int CH = (NH + 31) / 32;
+    for (int u = tid >> 5; u < 2 * CH; u += NT / 32) {
+        const int j = (u % CH) * 32 + (tid & 31);
+        if (j >= NH) continue;
+        const bool row = j < TX;  // bottom row, else left column
+        const int l = row ? j + 1 : (j - TX + 1) * LW, e = row ? j + 1 : (j - TX + 1) * EW;
+        if (u < CH) {
+            const A8<R> b = conj_dn_t(row ? lk(0, l - 1) : lk(1, l - LW), s_alg(sA, row ? e - 1 : e - EW, EN));
+            if (row) s_alg_put(sLf, e, EN, b);
+            else s_alg_put(sHalo + AP * NH, j - TX, TY, b);
+        } else {
+            const A8<R> f = conj_up_t(lk(row ? 1 : 0, l), s_alg(sPhi, row ? l + LW : l + 1, LN));
+            s_alg_put(sHalo, j, NH, icomm(f, s_alg(sPhi, l, LN)));
+        }
+    }
+    __syncthreads();
+    // by the warps that had no item
+    for (int j = NT - 1 - tid; j < NH; j += NT) {
+        const bool row = j < TX;
+        const int e = row ? j + 1 : (j - TX + 1) * EW;
+        const A8<R> A0 = s_alg(sA, e, EN), b = row ? s_alg(sLf, e, EN) : s_alg(sHalo + AP * NH, j - TX, TY);
+        const A8<R> cur = s_alg(sHalo, j, NH);
+        Vec* es_h = sEs + (row ? AP * EN : 0);
+        const A8<R> eo = s_alg(es_h, e, EN);
+        A8<R> sum;
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            const R F = row ? b.v[c] - A0.v[c] : A0.v[c] - b.v[c];
+            sum.v[c] = eo.v[c] + next_e(eo.v[c], F, cur.v[c], t, dt, inv_t);
+        }
+        s_alg_put(es_h, e, EN, sum);
     }
     __syncthreads();
 
@@ -407,10 +377,8 @@ __device__ __forceinline__ void fused_tile(const Fields<R>& in, const Fields<R>&
         store_alg_cs(out.pi, g, Vn, p_new);
         store_alg_cs(out.phi, g, Vn, ph_new);
         M3<R> nx = mul(exp_i_alg<R>(my_ex, a.dt_over_th), lk(0, ls));
-        if (a.reunit) reunit(nx);
         store_link_cs(out.U, 0, g, Vn, nx);
         M3<R> ny = mul(exp_i_alg<R>(my_ey, a.dt_over_th), lk(1, ls));
-        if (a.reunit) reunit(ny);
         store_link_cs(out.U, 1, g, Vn, ny);
     }
 }

@@ -34,7 +34,7 @@ struct SpeciesParams {
 // same kernel also writes the site E, B at t_n into site (not null).
 // FP32: the strip kernel, tile = launch shape 0 (16 warps per SM), 1 (12) or
 // 2 (8); its links of row y are re-unitarised in FP64 in the steps n with
-// (n + 1 + y) % reunit_every == 0 (0: never).  FP64: tile 2 = 32x2, else 32x4.
+// (n + 1 + y) % reunit_every == 0 (0: never).  FP64: tile 2 = 32x2, else 16x8.
 // seg: FP32 rows per strip segment (0: the cost model's choice for the shape)
 void launch_fused_step(int prec, void* in, void* out, void* site, int N, int64_t n, double dt, int reunit_every,
                        int tile, int seg, cudaStream_t st);

@@ -3,7 +3,7 @@
 //
 // Same quantities as fused_body.cuh.  What bounds a small FP64 lattice is the
 // rate of one scheduler: an FP64 warp instruction takes 64 cycles of it however
-// many lanes are active, and a thread of the 32x4 tile runs about 4,000 of them
+// many lanes are active, and a thread of the large tile runs about 4,000 of them
 // one after the other (127 us on a 32^2 lattice, 8 blocks on 152 SMs).  Here a
 // thread runs about 650: the three rows of a plaquette product go to three
 // warps, the transports and commutators of the two directions to four, the
@@ -11,19 +11,22 @@
 // arithmetic of a site is the same but for the halo (25 plaquettes and 40
 // momenta for 16 sites), so lattices that fill the chip anyway keep the larger
 // tiles.
-// Measured: 32^2 127 -> 29 us, 64^2 127 -> 39 us, 128^2 129 -> 119 us; nine events of 64/128/256,
-// which fill the chip, 1294 us in 32x4 tiles and 1482 us with the two smaller
-// sizes in these.  Both kernels give the same bits (su3.cuh, mul_rn).
+// Measured: 32^2 127 -> 29 us, 64^2 127 -> 39 us, 128^2 129 -> 119 us.  Both kernels
+// give the same bits (su3.cuh, mul_rn).
 #pragma once
 #include "fused_body.cuh"
 
 namespace gl {
 
-// The 32x4 tiles of an N x N lattice, and whether a launch of `tiles` of them in
-// all takes the small tiles instead: a 32x4 tile takes an SM to itself, so up to
-// one tile an SM the time is that of one tile, whatever the lattice.
-inline int64_t tiles64(int N) { return (int64_t)((N + 31) / 32) * ((N + 3) / 4); }
-inline bool small64(int64_t tiles, int sms) { return tiles <= sms; }
+// The large tiles of an N x N lattice, and whether a launch of `tiles` of them in
+// all takes the small tiles instead.  A large tile keeps an SM's FP64 pipe to
+// itself, so the time goes in steps of one tile an SM, and the small tiles' with
+// the sites: 140^2 (162 tiles) 146 us against 170, 152^2 (190) 163 against 170,
+// 156^2 (200) 177 against 170; batches of 5 and 6 events of 64^2 (160 and 192
+// tiles) 153 against 173 and 182 against 174 us.
+constexpr int TILE64_X = 16, TILE64_Y = 8;
+inline int64_t tiles64(int N) { return (int64_t)((N + TILE64_X - 1) / TILE64_X) * ((N + TILE64_Y - 1) / TILE64_Y); }
+inline bool small64(int64_t tiles, int sms) { return 4 * tiles <= 5 * sms; }
 
 struct SmallTile {
     static constexpr int T = 4, SITES = 16, LW = 6, LN = 36, EW = 5, EN = 25, ITEMS = 20, NT = 128;
@@ -78,44 +81,9 @@ __device__ __forceinline__ void small_tile(const Fields<double>& in, const Field
             pr[k] = v.x;
             pi[k] = v.y;
         }
-        {
-            const M3<double> m = link(1, l + 1);
-#pragma unroll
-            for (int j = 0; j < 3; j++) {
-                double sr = 0, si = 0;
-#pragma unroll
-                for (int k = 0; k < 3; k++) {
-                    sr = fma(pr[k], m.re[k][j], sr);
-                    sr = fma(-pi[k], m.im[k][j], sr);
-                    si = fma(pr[k], m.im[k][j], si);
-                    si = fma(pi[k], m.re[k][j], si);
-                }
-                qr[j] = sr;
-                qi[j] = si;
-            }
-        }
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const M3<double> m = h == 0 ? link(0, l + S_::LW) : link(1, l);
-#pragma unroll
-            for (int j = 0; j < 3; j++) {
-                double sr = 0, si = 0;
-#pragma unroll
-                for (int k = 0; k < 3; k++) {
-                    sr = fma(qr[k], m.re[j][k], sr);
-                    sr = fma(qi[k], m.im[j][k], sr);
-                    si = fma(qi[k], m.re[j][k], si);
-                    si = fma(-qr[k], m.im[j][k], si);
-                }
-                pr[j] = sr;
-                pi[j] = si;
-            }
-#pragma unroll
-            for (int j = 0; j < 3; j++) {
-                qr[j] = pr[j];
-                qi[j] = pi[j];
-            }
-        }
+        row_mul(pr, pi, link(1, l + 1), qr, qi);
+        row_mul_dag(qr, qi, link(0, l + S_::LW), pr, pi);
+        row_mul_dag(pr, pi, link(1, l), qr, qi);
 #pragma unroll
         for (int j = 0; j < 3; j++) S.P[warp * 3 + j][lane] = make_double2(qr[j], qi[j]);
     }

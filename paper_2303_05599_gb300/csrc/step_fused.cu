@@ -7,7 +7,7 @@
 namespace gl {
 
 template <typename R, int TX, int TY>
-__global__ void __launch_bounds__(TX * TY, (Tile<R, TX, TY>::min_blocks)) fused_step_kernel(Fields<R> in, Fields<R> out,
+__global__ void __launch_bounds__(TX * TY) fused_step_kernel(Fields<R> in, Fields<R> out,
                                                              typename Prec<R>::V* site, StepR<R> a) {
     fused_tile<R, TX, TY>(in, out, site, a, blockIdx.x);
 }
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(SmallTile::NT) small_step_kernel(Fields<double
 void launch_fused_step(int prec, void* in, void* out, void* site, int N, int64_t n, double dt, int reunit_every,
                        int tile, int seg, cudaStream_t st) {
     if (prec == 0) {
-        // FP64: 4x4 tiles of four warps for small lattices, else 32x4 (139 KB of
+        // FP64: 4x4 tiles of four warps for small lattices, else 16x8 (103 KB of
         // shared memory) or 32x2
         if (small64(tiles64(N), sm_count())) {
             const int64_t Vn = (int64_t)N * N;
@@ -101,7 +101,7 @@ void launch_fused_step(int prec, void* in, void* out, void* site, int N, int64_t
                 carve_fields<double>(in, Vn), carve_fields<double>(out, Vn), (double2*)site,
                 step_r<double>(step_args(N, nt, n, dt, 0)));
         } else if (tile == 2) launch_t<double, 32, 2>(in, out, site, N, n, dt, st);
-        else launch_t<double, 32, 4>(in, out, site, N, n, dt, st);
+        else launch_t<double, TILE64_X, TILE64_Y>(in, out, site, N, n, dt, st);
     } else if (tile == 1) {
         launch_strip<12, 1>(in, out, site, N, n, dt, reunit_every, seg, st);
     } else if (tile == 2) {

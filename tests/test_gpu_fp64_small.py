@@ -1,5 +1,5 @@
-"""The FP64 field step on both sides of the size that takes the small tiles (as
-many 32x4 tiles as SMs): against the oracle, with ragged and wrapping tiles;
+"""The FP64 field step on both sides of the size that takes the small tiles (a
+quarter more large tiles than SMs): against the oracle, with ragged and wrapping tiles;
 and batches that take the large tiles, bitwise as their events alone in the
 small ones, and the reverse, on two streams and as one fused launch."""
 import numpy as np
@@ -25,7 +25,7 @@ def rel(a, b):
     return np.abs(np.asarray(a).ravel() - np.asarray(b).ravel()).max() / max(1e-300, np.abs(b).max())
 
 
-@pytest.mark.parametrize("N", [4, 5, 7, 33, 128, 140])
+@pytest.mark.parametrize("N", [4, 5, 7, 33, 128, 140, 160, 165])
 def test_fields_against_the_oracle(N):
     w = wl(N)
     st, bad = O.mv_init(w.N, w.Ns, w.g2mu_a, w.m_a, w.Lambda_a, w.seed)
