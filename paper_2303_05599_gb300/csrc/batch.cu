@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(OBS_THREADS) batch_obs_kernel(const BObs* ev, 
     __syncthreads();
     const BObs& d = ev[s_e];
     const int b = blockIdx.x - d.block_begin;
-    const int64_t chunk = obs_chunk(d.np);
+    const int64_t chunk = obs_chunk(obs_prec<R>(), d.np);
     const int64_t c0 = (int64_t)b * chunk;
     const int64_t c1 = c0 + chunk < d.np ? c0 + chunk : d.np;
     particle_obs_block<R>(carve_parts<R>((void*)d.parts, d.np), d.t, d.mask, d.oa, c0, c1,
@@ -1366,7 +1366,7 @@ static gl_status obs_enqueue(gl_batch* b, uint32_t what, int k) {
             d.t = o.t;
             d.mask = o.mask;
             d.block_begin = blocks;
-            d.nblocks = obs_blocks(o.np);
+            d.nblocks = obs_blocks(b->prec == GL_FP64 ? 0 : 1, o.np);
             d.partials = o.partials;
             d.out = o.out;
             d.oa.sp = o.sp;

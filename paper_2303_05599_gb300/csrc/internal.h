@@ -91,7 +91,7 @@ size_t init_scratch_bytes(int prec, int N, int Ns);
 void launch_convert(int prec, int which, int to_device, void* dev, double* staging, int N, int64_t np,
                     cudaStream_t st);
 // observables: per-species particle sums and field checks, FP64, fixed-order reductions
-// (partials: obs_blocks(np) <= 1024 rows of GL_MAX_SPECIES * PO_N; out: GL_MAX_SPECIES * PO_N)
+// (partials: obs_blocks(prec, np) <= 1024 rows of GL_MAX_SPECIES * PO_N; out: GL_MAX_SPECIES * PO_N)
 void launch_particle_obs(int prec, const void* parts, int64_t np, double t, uint32_t active_mask,
                          const SpeciesParams& sp, const double q2ref[GL_MAX_SPECIES],
                          const double q3ref[GL_MAX_SPECIES], double* partials, double* out, cudaStream_t st);

@@ -2,11 +2,11 @@
 // <p_L^2>, <p_T^2(tau) - p_T^2(tau_form)>; Casimir drifts of the colour
 // charges) as one block's partial sums over a fixed chunk of particles.
 //
-// The particles of an event are cut into chunks of obs_chunk(np) particles,
+// The particles of an event are cut into chunks of obs_chunk(prec, np) particles,
 // one block each, and every block writes GL_MAX_SPECIES x PO_N partial values
 // (sums, or maxima for the Casimir drifts).  A second pass reduces the partials
 // of an event in a fixed order.  The chunking depends only on the event's
-// particle count, so an event gives bitwise the same observables whether it is
+// precision and particle count, so an event gives bitwise the same observables whether it is
 // reduced on its own or inside a batch.
 //
 // Per-particle quantities are evaluated in the state's precision.  Within a
@@ -30,21 +30,27 @@ namespace gl {
 static constexpr int OBS_THREADS = 256;
 static constexpr int OBS_MAX_BLOCKS = 1024;
 
-// particles per observables block: an eighth of the event's particles, kept
-// within [1024, 4096] (at least 4 a thread, so that the block's reductions of
-// its columns stay a small share of its work; small events still spread over
-// 8 blocks, large ones take 16 a thread), and at most OBS_MAX_BLOCKS blocks;
-// a multiple of OBS_THREADS.  A function of the event's particle count only.
-__host__ __device__ inline int64_t obs_chunk(int64_t np) {
-    int64_t t = (np + 7) / 8;
-    t = t < 1024 ? 1024 : t > 4096 ? 4096 : t;
+// particles per observables block, a multiple of OBS_THREADS, of at most
+// OBS_MAX_BLOCKS blocks.  FP32: an eighth of the event's particles, kept within
+// [256, 4096] (small events spread over 8 blocks, large ones take 16 a thread,
+// so that the block's reductions of its columns stay a small share of its
+// work).  FP64: a particle takes a thread 9 us of FP64 instructions, so they
+// spread over 64 blocks of at most 4 a thread (a request of one event of 1000
+// particles 62 -> 40 us, of 1e5 149 -> 62 us against the FP32 rule from 1024 on).
+// A function of the event's precision and particle count only.
+__host__ __device__ inline int64_t obs_chunk(int prec, int64_t np) {
+    int64_t t = prec == 0 ? (np + 63) / 64 : (np + 7) / 8;
+    const int64_t most = prec == 0 ? 1024 : 4096;
+    t = t < OBS_THREADS ? OBS_THREADS : t > most ? most : t;
     int64_t c = (np + OBS_MAX_BLOCKS - 1) / OBS_MAX_BLOCKS;
     if (c < t) c = t;
     return (c + OBS_THREADS - 1) / OBS_THREADS * OBS_THREADS;
 }
-__host__ __device__ inline int obs_blocks(int64_t np) {
-    return np > 0 ? (int)((np + obs_chunk(np) - 1) / obs_chunk(np)) : 0;
+__host__ __device__ inline int obs_blocks(int prec, int64_t np) {
+    return np > 0 ? (int)((np + obs_chunk(prec, np) - 1) / obs_chunk(prec, np)) : 0;
 }
+template <typename R>
+__host__ __device__ constexpr int obs_prec() { return sizeof(R) == 8 ? 0 : 1; }
 
 struct ObsArgs {
     SpeciesParams sp;

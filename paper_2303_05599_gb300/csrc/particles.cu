@@ -367,11 +367,11 @@ void launch_parts_convert(int prec, void* parts, int64_t np, double* stg, int to
 }
 
 // ------------------------------------------------------------ particle observables
-// one block per chunk of obs_chunk(np) particles, then one warp per value for the final reduction
+// one block per chunk of obs_chunk(prec, np) particles, then one warp per value for the final reduction
 template <typename R>
 __global__ void __launch_bounds__(OBS_THREADS) particle_obs_kernel(Parts<R> P, double t, uint32_t active, ObsArgs oa,
                                                                    double* partials) {
-    const int64_t chunk = obs_chunk(P.np);
+    const int64_t chunk = obs_chunk(obs_prec<R>(), P.np);
     const int64_t c0 = (int64_t)blockIdx.x * chunk;
     const int64_t c1 = c0 + chunk < P.np ? c0 + chunk : P.np;
     particle_obs_block<R>(P, t, active, oa, c0, c1, partials + (size_t)blockIdx.x * GL_MAX_SPECIES * PO_N);
@@ -389,7 +389,7 @@ void launch_particle_obs(int prec, const void* parts, int64_t np, double t, uint
     ObsArgs oa;
     oa.sp = sp;
     for (int k = 0; k < GL_MAX_SPECIES; k++) { oa.q2ref[k] = q2ref[k]; oa.q3ref[k] = q3ref[k]; }
-    const int blocks = obs_blocks(np);
+    const int blocks = obs_blocks(prec, np);
     if (blocks < 1) {
         cudaMemsetAsync(out, 0, GL_MAX_SPECIES * PO_N * sizeof(double), st);
         return;
