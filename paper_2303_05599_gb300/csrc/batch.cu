@@ -34,7 +34,7 @@
 namespace gl {
 
 static constexpr int MAX_EVENTS = 1024;
-static constexpr int PUSH_CHUNK = 1024;  // default particles per push block
+static constexpr int PUSH_CHUNK = 1024;  // particles per push block of the trials with resident blocks
 
 struct EvDesc {
     void* field[2];
@@ -604,6 +604,24 @@ static float time_trial(gl_batch* b, cudaEvent_t e0, cudaEvent_t e1, int reps, F
     return total / (reps - 1);
 }
 
+// Particles per push block of a batch that was not tuned, in blocks of 128.  A
+// particle takes a thread about 25 us in FP64 and 8 us in FP32, one after the
+// other, so threads take more than one only where the particles fill the chip
+// many times over (30 events of 2e5: 4 a thread is the tuned choice, 64 of 1e4:
+// one).  Two steps, against 8 a thread for every batch: FP64, 5 events of 64^2 with
+// 5000 particles 630 -> 386 us, 9 of 64/128/256 with 1e4 2767 -> 2499 us; FP32, 16 of
+// 64/128/256 with 1e4 316 -> 284 us, 30 of 256^2 with 2e5 1514 -> 1342 us.
+static int default_push_chunk(const gl_batch* b) {
+    int64_t np = 0;
+    for (int e = 0; e < b->ne; e++) {
+        CtxView v;
+        ctx_view(b->ev[e], &v);
+        np += v.np;
+    }
+    const int64_t rounds = np / ((int64_t)sm_count() * 1024);
+    return b->prec == GL_FP64 || rounds < 16 ? 128 : rounds < 32 ? 256 : 512;
+}
+
 extern "C" {
 
 size_t gl_batch_obs_row_bytes(void) { return sizeof(double) * OBS_W; }
@@ -701,7 +719,7 @@ gl_status gl_batch_create(const gl_config* cfgs, const gl_species* species, int3
     b->strip_wpb = 8;
     b->plan_tile = -1;
     b->push_block = 128;
-    b->push_chunk = PUSH_CHUNK;
+    b->push_chunk = default_push_chunk(b);
     b->fused = 0;
     b->push_grid = 0;
     b->graph_tile = -1;
