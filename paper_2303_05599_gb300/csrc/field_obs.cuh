@@ -135,10 +135,12 @@ __device__ __forceinline__ double gram_deviation(const M3<float>& u) {
 // FP32 sums, which are more exact.  The sums of squares of the six site fields,
 // whose halves are tr X^2 = X^a X^a / 2, go into SquareSum<R> slots: an FP32
 // state's squares are exact as float pairs, so its sums cost no FP64 issue
-// (field_obs_finish turns the slots into FP64 values).
+// (field_obs_block_reduce turns the slots into FP64 values).
 // Bound by the FP64 pipe (87 % of its cycles): 18 events of 64/128/256, FP32,
 // 540 FP64 warp instructions a site, 559 us under ncu; with FP64 Gram matrices,
-// converted inputs and one block reduction a site the call took 786 us, now 612.
+// converted inputs and one block reduction a site the call took 786 us, now 601.
+// (The commutator and the first product of the transport in three-part sums,
+// 107 FP64 operations fewer and 4,400 FP32 ones more: 663 us.)
 template <typename R>
 __device__ __forceinline__ void field_obs_site(const Fields<R>& f, const typename Prec<R>::V* __restrict__ site,
                                                int N, int64_t Vn, int64_t s, double* v) {
@@ -176,33 +178,30 @@ __device__ __forceinline__ void field_obs_init(double* v) {
     for (int k = FO_ET2; k <= FO_BL2; k++) v[k] = SquareSum<R>::init();
 }
 
-// after its last site: the sums of squares as FP64 halves (tr X^2)
+// the block's accumulators (maxima and sums, fixed order) into row[FO_N]; every
+// thread of the block calls it.  Eight threads a value: each combines an eighth
+// of the threads' accumulators in order, then three shuffles; the sums of
+// squares stay SquareSum<R> slots until the last, whose halves are tr X^2.  (Five
+// shuffle levels of all seven values took each warp 60 FP64 instructions.)
 template <typename R>
-__device__ __forceinline__ void field_obs_finish(double* v) {
+__device__ __forceinline__ void field_obs_block_reduce(const double* v, double* row) {
+    __shared__ double acc[FO_N][FIELD_OBS_THREADS + 1];
+    static_assert(FIELD_OBS_THREADS == 64 && FO_N <= 8, "eight threads a value");
 #pragma unroll
-    for (int k = FO_ET2; k <= FO_BL2; k++) v[k] = 0.5 * SquareSum<R>::finish(v[k]);
-}
-
-// the block's accumulators (maxima and sums, fixed order) into row[FO_N];
-// every thread of the block calls it
-__device__ __forceinline__ void field_obs_block_reduce(double* v, double* row) {
-    __shared__ double wacc[32][FO_N];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int o = 16; o > 0; o >>= 1)
-        for (int k = 0; k < FO_N; k++) {
-            const double oth = __shfl_down_sync(0xffffffffu, v[k], o);
-            v[k] = (k == FO_GMAX || k == FO_UMAX) ? nanmax(v[k], oth) : v[k] + oth;
-        }
-    if (lane == 0)
-        for (int k = 0; k < FO_N; k++) wacc[warp][k] = v[k];
+    for (int k = 0; k < FO_N; k++) acc[k][threadIdx.x] = v[k];
     __syncthreads();
-    if (threadIdx.x < FO_N) {
-        const int k = threadIdx.x;
-        double a = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); w++)
-            a = (k == FO_GMAX || k == FO_UMAX) ? nanmax(a, wacc[w][k]) : a + wacc[w][k];
-        row[k] = a;
+    const int k = threadIdx.x >> 3, part = threadIdx.x & 7;
+    auto combine = [&](double a, double b) {
+        if (k == FO_GMAX || k == FO_UMAX) return nanmax(a, b);
+        return k == FO_GSUM ? a + b : SquareSum<R>::combine(a, b);
+    };
+    double a = 0.0;
+    if (k < FO_N) {
+        a = acc[k][part * 8];
+        for (int j = 1; j < 8; j++) a = combine(a, acc[k][part * 8 + j]);
     }
+    for (int o = 4; o > 0; o >>= 1) a = combine(a, __shfl_down_sync(0xffffffffu, a, o, 8));
+    if (k < FO_N && part == 0) row[k] = k >= FO_ET2 ? 0.5 * SquareSum<R>::finish(a) : a;
 }
 
 }  // namespace gl

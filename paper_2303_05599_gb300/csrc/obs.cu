@@ -35,8 +35,7 @@ __global__ void __launch_bounds__(FIELD_OBS_THREADS) field_obs_kernel(FieldObsEv
     field_obs_init<R>(v);
     for (int64_t s = (int64_t)blk * blockDim.x + threadIdx.x; s < Vn; s += (int64_t)d.nblocks * blockDim.x)
         field_obs_site<R>(f, site, d.N, Vn, s, v);
-    field_obs_finish<R>(v);
-    field_obs_block_reduce(v, d.partials + (size_t)blk * FO_N);
+    field_obs_block_reduce<R>(v, d.partials + (size_t)blk * FO_N);
 }
 
 // the FO_N values of event e in block e, a warp each
