@@ -58,7 +58,15 @@ static constexpr int INIT_T = 256;                  // threads of the line kerne
 static constexpr int INIT_MAX_N = 3072;             // longest line
 static constexpr int INIT_GEN_OUT = 12;             // outputs a thread of a prime pass: 256 x 12 = 3072 points
 static_assert(sizeof(FFTables) % 16 == 0, "alignment of the tables behind it");
-static constexpr size_t INIT_ROUND_BYTES = (size_t)32 << 20;  // scratch small events may use for more sheets a round
+
+// Scratch for the sheets of a round.  What the other uses of the scratch need
+// (`base`) holds two sheets, 1.7 waves of blocks on a 256^2 lattice; events
+// take 32 MB more, up to 96 MB in all (six sheets: 4.75 -> 4.45 ms; larger
+// lattices fill the chip with two).
+static size_t init_room(size_t base) {
+    const size_t more = base + ((size_t)32 << 20), most = (size_t)96 << 20;
+    return base > most ? base : more < most ? more : most;
+}
 
 struct InitPlan {
     int S, groups, per_group;  // sheets a round, groups of sheets, sheets a group
@@ -72,8 +80,7 @@ static InitPlan init_plan(int prec, int N, int Ns) {
         // per site: 288 B a sheet (both nuclei), 288 B lines, 8 B Green
         // function; the commutators, 128 B, later in the place of the sheets
         const size_t lines = 288 * V, tables = ((size_t)2 * N * 16 + 255) & ~(size_t)255;
-        size_t room = lines + tables + 296 * V;
-        if (room < INIT_ROUND_BYTES) room = INIT_ROUND_BYTES;
+        const size_t room = init_room(lines + tables + 296 * V);
         const size_t most = (room - lines - tables - 8 * V) / (288 * V);
         p.groups = 1;
         p.per_group = Ns;
@@ -95,7 +102,7 @@ static InitPlan init_plan(int prec, int N, int Ns) {
     p.groups = (Ns + p.per_group - 1) / p.per_group;
     p.S = Ns;
     const size_t base = 576 * V;
-    const size_t room = base > INIT_ROUND_BYTES ? base : INIT_ROUND_BYTES;
+    const size_t room = init_room(base);
     if ((size_t)Ns * 128 * V + 8 * V + (size_t)p.groups * 192 * V + tw > room) {
         p.groups = 1;
         p.per_group = Ns;
