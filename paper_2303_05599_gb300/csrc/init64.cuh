@@ -21,8 +21,8 @@
 // Twiddles come from a table of each sign, and the Jacobian of a Newton step
 // from the entries of K that K T^b is made of (the other products are with 0).
 // Measured: a 32^2 event of 50 sheets 10474 us with seven launches a sheet, a
-// sincospi a butterfly and eight matrix products a Newton step, 816 us so (normal
-// variates 60, transforms 170, exponentials 71, products 128, links 280); with
+// sincospi a butterfly and eight matrix products a Newton step, 829 us so (normal
+// variates 60, transforms 170, exponentials 68, products 89, links 270); with
 // init.cu's transforms and series in FP64 it was 550 us, in other roundings.
 #pragma once
 #include "internal.h"
@@ -248,9 +248,14 @@ __global__ void __launch_bounds__(96) init64_products_kernel(const InitEv* evs, 
 #pragma unroll
         for (int j = 0; j < 3; j++) v[j] = V[(size_t)j * Vn];
     }
-#pragma unroll 2
+    // the next sheet's exponential on its way while one is multiplied
+    const size_t step = (size_t)INIT64_PLANES * Vn;
+    M3<double> next = m_zero<double>();
+    if (first < n) next = load_link(w + first * step, 0, s, Vn);
+#pragma unroll 1
     for (int k = first; k < n; k++) {
-        const M3<double> m = load_link(w + (size_t)k * INIT64_PLANES * Vn, 0, s, Vn);
+        const M3<double> m = next;
+        if (k + 1 < n) next = load_link(w + (k + 1) * step, 0, s, Vn);
         double2 o[3];
 #pragma unroll
         for (int j = 0; j < 3; j++) {
@@ -285,7 +290,7 @@ __device__ __forceinline__ double residual64(const M3<double>& W, const M3<doubl
 // column b of the Jacobian, -Re tr(T^a K T^b).  Columns p and q of K T^b are columns q and p of K times
 // +-1/2 or +-i/2; those of T^3 and T^8, which are diagonal, times its entries.
 template <int b>
-__device__ __forceinline__ void jacobian_column(const M3<double>& K, double J[8][8]) {
+__device__ __forceinline__ void jacobian_column(const M3<double>& K, double (&J)[8][8]) {
     M3<double> T = m_zero<double>();
     if (b == 2 || b == 7) {
         const double c = 0.5 * inv_sqrt3<double>();
@@ -316,40 +321,41 @@ __device__ __forceinline__ void jacobian_column(const M3<double>& K, double J[8]
     for (int a = 0; a < 8; a++) J[a][b] = -re[a];
 }
 
-// J x = b in place of b, rows exchanged for the largest pivot; 1 if J is singular
-__device__ __forceinline__ int solve8(double J[8][8], double* b) {
+// J x = b in place of b, rows exchanged for the largest pivot (by selects, so
+// that J stays in registers); 1 if J is singular
+template <int c>
+__device__ __forceinline__ int eliminate8(double (&J)[8][8], double (&b)[8]) {
+    int p = c;
+    double most = fabs(J[c][c]);
 #pragma unroll
-    for (int c = 0; c < 8; c++) {
-        int p = c;
-        double most = fabs(J[c][c]);
+    for (int r = c + 1; r < 8; r++)
+        if (fabs(J[r][c]) > most) { most = fabs(J[r][c]); p = r; }
+    int singular = most < 1e-300;
 #pragma unroll
-        for (int r = c + 1; r < 8; r++)
-            if (fabs(J[r][c]) > most) { most = fabs(J[r][c]); p = r; }
-        if (most < 1e-300) return 1;
-        if (p != c) {
+    for (int r = c + 1; r < 8; r++) {
+        const bool swap = r == p;
 #pragma unroll
-            for (int r = c + 1; r < 8; r++)
-                if (r == p) {
-#pragma unroll
-                    for (int k = c; k < 8; k++) { const double t = J[c][k]; J[c][k] = J[r][k]; J[r][k] = t; }
-                    const double t = b[c]; b[c] = b[r]; b[r] = t;
-                }
+        for (int k = c; k < 8; k++) {
+            const double u = J[c][k], w = J[r][k];
+            J[c][k] = swap ? w : u;
+            J[r][k] = swap ? u : w;
         }
-#pragma unroll
-        for (int r = c + 1; r < 8; r++) {
-            const double f = J[r][c] / J[c][c];
-#pragma unroll
-            for (int k = c + 1; k < 8; k++) J[r][k] = fma(-f, J[c][k], J[r][k]);
-            b[r] = fma(-f, b[c], b[r]);
-        }
+        const double u = b[c], w = b[r];
+        b[c] = swap ? w : u;
+        b[r] = swap ? u : w;
     }
 #pragma unroll
-    for (int c = 7; c >= 0; c--) {
+    for (int r = c + 1; r < 8; r++) {
+        const double f = J[r][c] / J[c][c];
 #pragma unroll
-        for (int k = c + 1; k < 8; k++) b[c] = fma(-J[c][k], b[k], b[c]);
-        b[c] /= J[c][c];
+        for (int k = c + 1; k < 8; k++) J[r][k] = fma(-f, J[c][k], J[r][k]);
+        b[r] = fma(-f, b[c], b[r]);
     }
-    return 0;
+    if constexpr (c < 7) singular |= eliminate8<c + 1>(J, b);
+#pragma unroll
+    for (int k = c + 1; k < 8; k++) b[c] = fma(-J[c][k], b[k], b[c]);
+    b[c] /= J[c][c];
+    return singular;
 }
 
 // Newton solve for the Glasma link from the pure-gauge links of both nuclei
@@ -368,7 +374,7 @@ __device__ __forceinline__ int solve_link64(const M3<double>& UA, const M3<doubl
             jacobian_column<4>(K, J); jacobian_column<5>(K, J); jacobian_column<6>(K, J); jacobian_column<7>(K, J);
 #pragma unroll
             for (int a = 0; a < 8; a++) dx.v[a] = -F[a];
-            if (solve8(J, dx.v)) break;
+            if (eliminate8<0>(J, dx.v)) break;
         }
         double lam = 1.0;
 #pragma unroll 1
