@@ -80,8 +80,8 @@ TRAFFIC = {
 # of the push, which depends on the species mix (all Wong charm quarks in the
 # 64-event batch; half Wong, half static in 30 x 256^2).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-FP64_FLOP_PER_SITE = 4815
-FP64_FLOP_PER_PARTICLE = {"batched64": 958, "n256_charm_static": 498}
+FP64_FLOP_PER_SITE = 4261
+FP64_FLOP_PER_PARTICLE = {"batched64": 681, "n256_charm_static": 360}
 
 
 def sort_launches(ws):
