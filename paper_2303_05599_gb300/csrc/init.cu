@@ -693,41 +693,15 @@ __device__ __forceinline__ void match_jacobian(const M3<R>& K, R J[8][8]) {
 #undef GL_F
 }
 
-// the step in FP64 with row exchanges, 1 if J is singular
-__device__ __noinline__ int match_step_pivot(const M3<double>& K, const double* F, double* b) {
-    double J[8][8];
-    match_jacobian(K, J);
-    for (int c = 0; c < 8; c++) b[c] = -F[c];
-    for (int c = 0; c < 8; c++) {
-        int p = c;
-        for (int r = c + 1; r < 8; r++) if (fabs(J[r][c]) > fabs(J[p][c])) p = r;
-        if (fabs(J[p][c]) < 1e-300) return 1;
-        if (p != c) {
-            for (int k = 0; k < 8; k++) { double t = J[c][k]; J[c][k] = J[p][k]; J[p][k] = t; }
-            double t = b[c]; b[c] = b[p]; b[p] = t;
-        }
-        for (int r = c + 1; r < 8; r++) {
-            const double f = J[r][c] / J[c][c];
-            for (int k = c; k < 8; k++) J[r][k] -= f * J[c][k];
-            b[r] -= f * b[c];
-        }
-    }
-    for (int c = 7; c >= 0; c--) {
-        for (int k = c + 1; k < 8; k++) b[c] -= J[c][k] * b[k];
-        b[c] /= J[c][c];
-    }
-    return 0;
-}
-
-// The Newton step dx = -J^-1 F at K.  Its direction needs no more than FP32: an
+// The Newton step dx = -J^-1 F at K, false where it is not to be trusted.  Its
+// direction needs no more than FP32 as long as the full step contracts: an
 // error of 1e-6 in it leaves 1e-6 of the residual, where the iteration's own
 // square would leave less only in its last step, so the Jacobian and its
 // elimination (half of the operations of an iteration) run on the FP32 pipe
 // and the residual, the step's exponential and the link in FP64.  J is close
 // to -1 for links near the unit matrix, so the elimination runs in its own
-// order, in registers; where a pivot falls below 1/16 of the diagonal's scale
-// it is done again in FP64 with row exchanges.
-__device__ __forceinline__ int match_step(const M3<double>& K, const double* F, double* x) {
+// order, in registers; not where a pivot falls below 1/16 of the diagonal's scale.
+__device__ __forceinline__ bool match_step(const M3<double>& K, const double* F, double* x) {
     float J[8][8], y[8], inv[8];
     M3<float> Kf;
 #pragma unroll
@@ -757,7 +731,7 @@ __device__ __forceinline__ int match_step(const M3<double>& K, const double* F, 
         y[c] *= inv[c];
         x[c] = (double)y[c];
     }
-    return small ? match_step_pivot(K, F, x) : 0;
+    return !small;
 }
 
 // F^a = Im tr T^a (W + K), K = W U^+, and its largest entry
@@ -772,7 +746,17 @@ __device__ __forceinline__ double match_residual(const M3<double>& K, const doub
     return r;
 }
 
-// Newton solve for the Glasma link from the pure-gauge links of both nuclei
+// the plain FP64 method of init64.cuh, which few links of few events need
+__device__ __noinline__ int solve_link_plain(const M3<double>& UA, const M3<double>& UB, M3<double>& U) {
+    return solve_link64(UA, UB, U);
+}
+
+// Newton solve for the Glasma link from the pure-gauge links of both nuclei, by
+// full steps of FP32 directions while each leaves at most a quarter of the
+// residual.  Iterations that do not contract (strong fields on coarse lattices,
+// g^2 mu a of order 1) wander before they converge, or do not: there an error of
+// 1e-6 in a direction ends at another solution of the matching condition, or
+// at none, so such a link starts again with the plain method.
 __device__ int solve_link(const M3<double>& UA, const M3<double>& UB, M3<double>& U) {
     const M3<double> W = add(UA, UB);
     double fw[8], F[8];
@@ -780,31 +764,19 @@ __device__ int solve_link(const M3<double>& UA, const M3<double>& UB, M3<double>
     U = mul(UA, UB);
     M3<double> K = mul_nd(W, U);
     double r = match_residual(K, fw, F);
-    for (int it = 0; it < 100 && r > 1e-14; it++) {
-        double dx[8];
-        if (match_step(K, F, dx)) break;
-        double lam = 1.0;
-        for (int k = 0; k < 30; k++) {
-            A8<double> st;
-#pragma unroll
-            for (int a = 0; a < 8; a++) st.v[a] = lam * dx[a];
-            M3<double> Un = mul_rows(exp_i_alg<double>(st, 1.0), U);
-            rebuild_row2(Un);
-            const M3<double> Kn = mul_nd(W, Un);
-            double Fn[8];
-            const double rn = match_residual(Kn, fw, Fn);
-            if (rn < r || k == 29) {
-                U = Un;
-                K = Kn;
-                r = rn;
-#pragma unroll
-                for (int a = 0; a < 8; a++) F[a] = Fn[a];
-                break;
-            }
-            lam *= 0.5;
-        }
+    bool contracts = r == r;
+    while (contracts && r > 1e-14) {
+        A8<double> dx;
+        contracts = match_step(K, F, dx.v);
+        if (!contracts) break;
+        U = mul_rows(exp_i_alg<double>(dx, 1.0), U);
+        rebuild_row2(U);
+        K = mul_nd(W, U);
+        const double rn = match_residual(K, fw, F);
+        contracts = rn <= 0.25 * r;  // not for a NaN
+        r = rn;
     }
-    return r > 1e-12;
+    return contracts ? 0 : solve_link_plain(UA, UB, U);
 }
 
 // The Glasma link (d, s), as two rows, and i[-i[U^A]_ah, -i[U^B]_ah] of the
