@@ -49,27 +49,31 @@ __device__ __forceinline__ A8<double> rapidity_rotation(const A8<double>& ph, do
     return conj_up_t(exp_i_alg<double>(ph, -s), q);
 }
 // FP32: the rotation is that of Q's eight components by exp(s ad), whose series
-// Q - s i[phi, Q] + ... needs K terms where |s phi|^(K+1) / (K+1)! <= 2^-25 (ad's
-// largest eigenvalue is at most |phi|, the length of SU(3)'s roots being 1).  A
-// step turns Q by dt / t v_w phi, 1e-4 .. 1e-2 for most particles, and a term
-// takes 80 operations, the exponential and the transport about 320, so angles
-// to 0.08 (four terms) take the series.  The push is bound by memory where the
-// particles are few a cell (30 x 256^2: 0.216 ms with either), and by issue as
-// well on 1024^2 with 4 a cell: 0.212 -> 0.203 ms.
+// Q - s i[phi, Q] + ... needs K terms where x^(K+1) / (K+1)! <= 2^-25 for x =
+// |s phi| (ad's largest eigenvalue is at most |phi|, the length of SU(3)'s roots
+// being 1).  Two things would move |Q|^2 always to one side, which a charge that
+// turns by nearly the same angle every step adds up.  The truncated series is not
+// orthogonal: K = 1, 2, 3, 4 multiply the part of |Q|^2 of that eigenvalue by 1 +
+// x^2, 1 + x^4/4, 1 - x^4/12, 1 - x^6/72; the limits keep that below 2^-30 as
+// well.  And terms added to Q one by one are lost below half a unit in its last
+// place, the first one not; so by Horner's rule they are summed inside, and Q
+// is rounded once.  (Terms one by one, with limits for the value alone: the mean
+// |Q|^2 of 4 off by 2.1e-5 after 300 turns by 2.3e-4 and by -1.3e-5 by 2.8e-2.)
+// A step turns Q by dt / t v_w phi, 1e-4 .. 1e-2 for most particles, and a term
+// takes 80 operations, the exponential and the transport about 320.  The push is
+// bound by memory where the particles are few a cell (30 x 256^2: 0.216 ms with
+// either), and by issue as well on 1024^2 with 4 a cell: 0.212 -> 0.203 ms.
 __device__ __forceinline__ A8<float> rapidity_rotation(const A8<float>& ph, float s, const A8<float>& q) {
     const float x2 = s * s * a_dot(ph, ph);
-    if (!(x2 <= 6.6e-3f)) return conj_up_t(exp_i_alg<float>(ph, -s), q);
-    const float terms = x2 <= 5.9e-8f ? 1.f : x2 <= 3.1e-5f ? 2.f : x2 <= 8.4e-4f ? 3.f : 4.f;
-    A8<float> o = q, t = q;
+    if (!(x2 <= 4e-3f)) return conj_up_t(exp_i_alg<float>(ph, -s), q);
+    const float terms = x2 <= 9e-10f ? 1.f : x2 <= 3.1e-5f ? 2.f : x2 <= 1e-4f ? 3.f : 4.f;
+    A8<float> o = q;
 #pragma unroll 1
-    for (float k = 1.f; k <= terms; k += 1.f) {
+    for (float k = terms; k >= 1.f; k -= 1.f) {
         const float f = k == 1.f ? -s : k == 2.f ? -0.5f * s : k == 3.f ? s * (-1.f / 3) : -0.25f * s;
-        t = icomm(ph, t);
+        const A8<float> t = icomm(ph, o);
 #pragma unroll
-        for (int a = 0; a < 8; a++) {
-            t.v[a] *= f;
-            o.v[a] += t.v[a];
-        }
+        for (int a = 0; a < 8; a++) o.v[a] = fmaf(f, t.v[a], q.v[a]);
     }
     return o;
 }
