@@ -133,12 +133,15 @@ __device__ __forceinline__ double gram_deviation(const M3<float>& u) {
 // as squared norms (the root, monotonic, is taken once of the maximum).  The
 // Gauss residual is FP64 throughout; an FP32 link's unitarity takes three-part
 // FP32 sums, which are more exact.  The sums of squares of the six site fields,
-// whose halves are tr X^2 = X^a X^a / 2, go into SquareSum<R> slots: an FP32
-// state's squares are exact as float pairs, so its sums cost no FP64 issue
-// (field_obs_block_reduce turns the slots into FP64 values).
+// whose halves are tr X^2 = X^a X^a / 2, are FP64 sums of site values; an FP32
+// state's squares are exact as float pairs, and a site's 8 or 16 of them are
+// summed as a pair (SquareSum) before they cost FP64 issue, two additions a
+// value.  (As pairs over all sites of a thread and of a block they lost up to
+// 2.5e-14 on 1024^2, against 1.5e-15, and overflowed at FP32's range: the
+// additions cost 1 % of the call on 18 events of 64/128/256, 3 % on 1024^2.)
 // Bound by the FP64 pipe (87 % of its cycles): 18 events of 64/128/256, FP32,
 // 540 FP64 warp instructions a site, 559 us under ncu; with FP64 Gram matrices,
-// converted inputs and one block reduction a site the call took 786 us, now 601.
+// converted inputs and one block reduction a site the call took 786 us, now 602.
 // (The commutator and the first product of the transport in three-part sums,
 // 107 FP64 operations fewer and 4,400 FP32 ones more: 663 us.)
 template <typename R>
@@ -161,29 +164,29 @@ __device__ __forceinline__ void field_obs_site(const Fields<R>& f, const typenam
     const double g2 = a_dot(G, G);
     v[FO_GMAX] = nanmax(v[FO_GMAX], g2);
     v[FO_GSUM] += g2;
+    double sum = SquareSum<R>::init();
 #pragma unroll
     for (int k = 0; k < 6; k++) {
         const A8<R> X = load_alg(site + (size_t)k * AP * Vn, s, Vn);
         const int slot = k < 2 ? FO_ET2 : k == 2 ? FO_EL2 : k < 5 ? FO_BT2 : FO_BL2;
+        if constexpr (sizeof(R) == 8) {
 #pragma unroll
-        for (int a = 0; a < 8; a++) v[slot] = SquareSum<R>::add(v[slot], X.v[a]);
+            for (int a = 0; a < 8; a++) v[slot] = SquareSum<R>::add(v[slot], X.v[a]);
+        } else {
+#pragma unroll
+            for (int a = 0; a < 8; a++) sum = SquareSum<R>::add(sum, X.v[a]);
+            if (k == 0 || k == 3) continue;  // the second component of the same value follows
+            v[slot] += widen(f2_lo(sum)) + widen(f2_hi(sum));
+            sum = SquareSum<R>::init();
+        }
     }
-}
-
-// the thread's accumulators before its first site
-template <typename R>
-__device__ __forceinline__ void field_obs_init(double* v) {
-    v[FO_GMAX] = v[FO_GSUM] = v[FO_UMAX] = 0.0;
-#pragma unroll
-    for (int k = FO_ET2; k <= FO_BL2; k++) v[k] = SquareSum<R>::init();
 }
 
 // the block's accumulators (maxima and sums, fixed order) into row[FO_N]; every
 // thread of the block calls it.  Eight threads a value: each combines an eighth
-// of the threads' accumulators in order, then three shuffles; the sums of
-// squares stay SquareSum<R> slots until the last, whose halves are tr X^2.  (Five
-// shuffle levels of all seven values took each warp 60 FP64 instructions.)
-template <typename R>
+// of the threads' accumulators in order, then three shuffles; the halves of the
+// sums of squares are tr X^2.  (Five shuffle levels of all seven values took each
+// warp 60 FP64 instructions.)
 __device__ __forceinline__ void field_obs_block_reduce(const double* v, double* row) {
     __shared__ double acc[FO_N][FIELD_OBS_THREADS + 1];
     static_assert(FIELD_OBS_THREADS == 64 && FO_N <= 8, "eight threads a value");
@@ -191,17 +194,14 @@ __device__ __forceinline__ void field_obs_block_reduce(const double* v, double* 
     for (int k = 0; k < FO_N; k++) acc[k][threadIdx.x] = v[k];
     __syncthreads();
     const int k = threadIdx.x >> 3, part = threadIdx.x & 7;
-    auto combine = [&](double a, double b) {
-        if (k == FO_GMAX || k == FO_UMAX) return nanmax(a, b);
-        return k == FO_GSUM ? a + b : SquareSum<R>::combine(a, b);
-    };
+    auto combine = [&](double a, double b) { return k == FO_GMAX || k == FO_UMAX ? nanmax(a, b) : a + b; };
     double a = 0.0;
     if (k < FO_N) {
         a = acc[k][part * 8];
         for (int j = 1; j < 8; j++) a = combine(a, acc[k][part * 8 + j]);
     }
     for (int o = 4; o > 0; o >>= 1) a = combine(a, __shfl_down_sync(0xffffffffu, a, o, 8));
-    if (k < FO_N && part == 0) row[k] = k >= FO_ET2 ? 0.5 * SquareSum<R>::finish(a) : a;
+    if (k < FO_N && part == 0) row[k] = k >= FO_ET2 ? 0.5 * a : a;
 }
 
 }  // namespace gl

@@ -31,11 +31,10 @@ __global__ void __launch_bounds__(FIELD_OBS_THREADS) field_obs_kernel(FieldObsEv
     const int64_t Vn = (int64_t)d.N * d.N;
     const Fields<R> f = carve_fields<R>((void*)d.fields, Vn);
     const typename Prec<R>::V* site = (const typename Prec<R>::V*)d.site;
-    double v[FO_N];
-    field_obs_init<R>(v);
+    double v[FO_N] = {};
     for (int64_t s = (int64_t)blk * blockDim.x + threadIdx.x; s < Vn; s += (int64_t)d.nblocks * blockDim.x)
         field_obs_site<R>(f, site, d.N, Vn, s, v);
-    field_obs_block_reduce<R>(v, d.partials + (size_t)blk * FO_N);
+    field_obs_block_reduce(v, d.partials + (size_t)blk * FO_N);
 }
 
 // the FO_N values of event e in block e, a warp each
