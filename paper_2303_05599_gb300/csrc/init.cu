@@ -889,10 +889,14 @@ void init_block_table(InitEv* evs, int ne) {
     }
 }
 
-// what the launches of one kind need beyond the default is a per-device function attribute, set on every call
+// The shared memory a launch may ask for is an attribute of the kernel on its
+// device, which calls on other contexts and host threads set too: every call
+// sets the most that any lattice needs (a row's four planes of the longest line).
+static constexpr int INIT_MAX_SMEM = 4 * INIT_MAX_N * 16;
+static_assert(INIT_MAX_SMEM <= 227 * 1024, "beyond a block's shared memory");
 template <typename K>
 static void line_smem(K* kernel, size_t bytes) {
-    if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, INIT_MAX_SMEM);
 }
 
 void launch_mv_init(const InitEv* h, const InitEv* d_ev, int ne, cudaStream_t st) {
