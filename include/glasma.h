@@ -171,7 +171,9 @@ typedef struct {
 typedef struct gl_ctx gl_ctx;
 
 /* Bytes of device workspace a context with this configuration needs.
- * Returns 0 for an invalid configuration. */
+ * Returns 0 for an invalid configuration.  The initial conditions take at
+ * most 576 bytes a site of it (4 MB below 86 x 86 sites) for themselves and
+ * otherwise use buffers that are idle until the first step. */
 size_t gl_workspace_bytes(const gl_config* cfg, const gl_species* species, int32_t n_species);
 
 /* Create a context on the current CUDA device.  d_workspace: caller-owned

@@ -249,8 +249,8 @@ PartsCheckEv ctx_parts_check_event(const gl_ctx* c) {
     return e;
 }
 InitEv ctx_init_event(const gl_ctx* c, int* bad) {
-    return init_event(c->prec, c->field[c->cur], c->scratch, c->N, c->cfg.Ns, c->g2mu_a, c->m_a, c->Lambda_a,
-                      c->cfg.seed, bad);
+    return init_event(c->prec, c->field[c->cur], c->scratch, c->field[1 - c->cur], c->site_buf[0], c->N, c->cfg.Ns,
+                      c->g2mu_a, c->m_a, c->Lambda_a, c->cfg.seed, bad);
 }
 void ctx_init_done(gl_ctx* c) {
     for (int k = 0; k < 2; k++) cudaMemsetAsync(c->site_buf[k], 0, site_bytes(c->prec, c->Vn), c->stream);

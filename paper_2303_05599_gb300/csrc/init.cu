@@ -47,76 +47,67 @@ namespace gl {
 // about 48 bits) and only the links' matching in FP64.  FP64 events have
 // kernels of their own, in one fixed order of roundings (init64.cuh).
 //
-// A sheet's planes wait in `work`, as many sheets a round as the scratch holds.
-// Small lattices (all sheets in one round) split each nucleus's product over
-// groups of consecutive sheets, whose partial products are multiplied at the
-// end: 1024 sites alone would leave most of the chip idle.  Rounds and groups
-// depend on N and Ns only, so an event's fields are bitwise the same alone and
-// in a batch.
+// A sheet's planes wait in a slot of the workspace, as many sheets a round as
+// there are slots.  Small lattices split each nucleus's product over groups of
+// consecutive sheets (a round takes some of every group), whose partial products
+// are multiplied at the end: 1024 sites alone would leave most of the chip idle.
+// Groups depend on N and Ns only, and rounds do not change the order of a
+// product, so an event's fields are bitwise the same alone and in a batch.
 
 static constexpr int INIT_T = 256;                  // threads of the line kernels
 static constexpr int INIT_MAX_N = 3072;             // longest line
 static constexpr int INIT_GEN_OUT = 12;             // outputs a thread of a prime pass: 256 x 12 = 3072 points
 static_assert(sizeof(FFTables) % 16 == 0, "alignment of the tables behind it");
 
-// Scratch for the sheets of a round.  What the other uses of the scratch need
-// (`base`) holds two sheets, 1.7 waves of blocks on a 256^2 lattice; events
-// take 32 MB more, up to 96 MB in all (six sheets: 4.75 -> 4.45 ms; larger
-// lattices fill the chip with two).
-static size_t init_room(size_t base) {
-    const size_t more = base + ((size_t)32 << 20), most = (size_t)96 << 20;
-    return base > most ? base : more < most ? more : most;
-}
+// Where the slots are.  The scratch holds the Wilson lines, the tables and as many
+// slots as fit 576 B a site (nine FP64 matrices of both nuclei and their lines) or, on
+// lattices below 86 sites a side, INIT_SMALL_ROOM.  The others lie in buffers of
+// the event that are idle until its first step: the slice of the fields that is
+// not current and the two site-field buffers, which are cleared afterwards.  An
+// FP32 event of 256^2 has 14 slots, 7 sheets a round, and takes 4.46 ms (2 sheets
+// a round: 4.75 ms).  The scratch is each event's own for good and serves the start
+// alone, so it stays small: with 32 MB more an event, nine events of 64/128/256
+// take 15.21 ms in 595 MB, with this 15.33 ms in 343 MB; a single small event,
+// which needs many sheets a round to fill the chip, pays more: FP64 32^2 0.65 ms in
+// 17 MB, here 0.72 ms in 7 MB and within 576 B a site 1.39 ms in 3 MB; FP32 64^2 0.37
+// ms in 32 MB and 0.59 ms in 7 MB.
+static constexpr size_t INIT_SMALL_ROOM = (size_t)4 << 20;
 
 struct InitPlan {
-    int S, groups, per_group;  // sheets a round, groups of sheets, sheets a group
-    size_t v, tw, work, green, total; // byte offsets
+    int groups, per_group, K;        // groups of sheets, sheets a group, sheets of each group a round
+    int n0, n1;                      // slots up to n0 in the scratch, up to n1 in the fields, the rest in the site fields
+    size_t unit, tw, work, green, total;  // bytes of a slot; byte offsets in the scratch (the lines are first)
 };
 
 static InitPlan init_plan(int prec, int N, int Ns) {
     const size_t V = (size_t)N * N;
+    // per site: a slot, a group's lines of both nuclei, the slots that fit the idle buffers (FP64 544 and 768 B, FP32 224 and 384 B)
+    const size_t unit = (prec == 0 ? 144 : 64) * V, lines = (prec == 0 ? 288 : 192) * V;
+    const int in_fields = 3, in_site = prec == 0 ? 5 : 6;
+    const size_t line_tw = ((size_t)N * 16 * (prec == 0 ? 2 : 1) + 255) & ~(size_t)255;
+    const size_t tables = line_tw + (prec == 0 ? 0 : sizeof(FFTables));
+    const size_t base = 576 * V, room = base > INIT_SMALL_ROOM ? base : INIT_SMALL_ROOM;
+    auto slots = [&](int groups) {
+        const size_t head = groups * lines + tables + 8 * V;
+        return (int)((room > head ? (room - head) / unit : 0) + in_fields + in_site);
+    };
     InitPlan p;
-    if (prec == 0) {
-        // per site: 288 B a sheet (both nuclei), 288 B lines, 8 B Green
-        // function; the commutators, 128 B, later in the place of the sheets
-        const size_t lines = 288 * V, tables = ((size_t)2 * N * 16 + 255) & ~(size_t)255;
-        const size_t room = init_room(lines + tables + 296 * V);
-        const size_t most = (room - lines - tables - 8 * V) / (288 * V);
-        p.groups = 1;
-        p.per_group = Ns;
-        p.S = most < (size_t)Ns ? (int)most : Ns;
-        p.v = 0;
-        p.tw = lines;
-        p.work = p.tw + tables;
-        p.green = p.work + (size_t)p.S * 288 * V;
-        p.total = p.green + 8 * V;
-        return p;
-    }
-    const size_t tw = (((size_t)N * 16 + 255) & ~(size_t)255) + sizeof(FFTables);
-    // per site: 128 B a sheet (both nuclei), 8 B Green function, 192 B a group
-    // (two nuclei's lines as two rows); later 192 B links and 128 B commutators
-    // in the place of work and Green function
-    int g = (int)(16384 / V);
-    g = g < 1 ? 1 : (g > Ns ? Ns : g);
+    int g = prec == 0 ? 1 : (int)(16384 / V);
+    g = g < 1 ? 1 : g > Ns ? Ns : g;
+    // at least two sheets a round of each group (64^2: 0.63 -> 0.59 ms, 48^2: 1.20 -> 0.96 ms)
+    while (g > 1 && slots(g) < 4 * g) g--;
     p.per_group = (Ns + g - 1) / g;
     p.groups = (Ns + p.per_group - 1) / p.per_group;
-    p.S = Ns;
-    const size_t base = 576 * V;
-    const size_t room = init_room(base);
-    if ((size_t)Ns * 128 * V + 8 * V + (size_t)p.groups * 192 * V + tw > room) {
-        p.groups = 1;
-        p.per_group = Ns;
-        p.S = (int)((room - 200 * V - tw) / (128 * V));
-        if (p.S < 2) p.S = 2;
-        if (p.S > Ns) p.S = Ns;
-    }
-    size_t w = (size_t)p.S * 128 * V + 8 * V;
-    if (w < 320 * V) w = 320 * V;
-    p.v = 0;
-    p.tw = (size_t)p.groups * 192 * V;
-    p.work = p.tw + tw;
-    p.green = p.work + (size_t)p.S * 128 * V;
-    p.total = p.work + w;
+    const int fit = slots(p.groups) / (2 * p.groups);
+    p.K = fit < p.per_group ? fit : p.per_group;
+    const int need = 2 * p.groups * p.K;
+    p.n0 = need > in_fields + in_site ? need - in_fields - in_site : 0;
+    p.n1 = p.n0 + (need - p.n0 < in_fields ? need - p.n0 : in_fields);
+    p.unit = unit;
+    p.tw = p.groups * lines;
+    p.work = p.tw + tables;
+    p.green = p.work + p.n0 * unit;
+    p.total = p.green + 8 * V;
     return p;
 }
 
@@ -137,7 +128,7 @@ static inline int cols64(int N) {
     return c > N ? N : c;
 }
 
-InitEv init_event(int prec, void* fields, void* scratch, int N, int Ns, double g2mu_a, double m_a, double Lambda_a,
+InitEv init_event(int prec, void* fields, void* scratch, void* idle_fields, void* idle_site, int N, int Ns, double g2mu_a, double m_a, double Lambda_a,
                   uint64_t seed, int* bad) {
     InitEv e;
     memset(&e, 0, sizeof e);
@@ -145,9 +136,10 @@ InitEv init_event(int prec, void* fields, void* scratch, int N, int Ns, double g
     const int64_t V = (int64_t)N * N;
     e.N = N;
     e.Ns = Ns;
-    e.S = p.S;
     e.groups = p.groups;
     e.per_group = p.per_group;
+    e.K = p.K;
+    e.S = p.groups * p.K;
     e.pow2 = (N & (N - 1)) == 0;
     if (e.pow2) {
         int l = 0;
@@ -173,13 +165,18 @@ InitEv init_event(int prec, void* fields, void* scratch, int N, int Ns, double g
     e.k0 = (uint32_t)seed;
     e.k1 = (uint32_t)(seed >> 32);
     char* s = (char*)scratch;
-    e.V = (double2*)(s + p.v);
+    e.V = (double2*)s;
     e.normal = (FFTables*)(s + p.tw);
     e.tw = (double2*)(s + p.tw + (prec == 0 ? 0 : sizeof(FFTables)));
-    e.work = (double2*)(s + p.work);
     e.green = (double*)(s + p.green);
-    e.U64 = (double2*)(s + p.work);
-    e.comm = prec == 0 ? e.work : e.U64 + (size_t)12 * V;
+    e.work[0] = (double2*)(s + p.work);
+    e.work[1] = (double2*)idle_fields;
+    e.work[2] = (double2*)idle_site;
+    e.end0 = p.n0 * p.unit / sizeof(double2);
+    e.end1 = p.n1 * p.unit / sizeof(double2);
+    // after the last sheet, in the site fields: FP32 192 B a site of links, 128 B of commutators
+    e.U64 = e.work[2];
+    e.comm = prec == 0 ? e.work[2] : e.U64 + (size_t)12 * V;
     e.fields = fields;
     e.prec = prec;
     e.bad = bad;
@@ -197,6 +194,15 @@ __device__ __forceinline__ const InitEv& init_find(const InitEv* evs, int ne, co
     const InitEv& d = evs ? evs[lo] : one;
     *blk = blockIdx.x - (evs ? d.begin[k] : 0);
     return d;
+}
+// element o of the slots, one after another
+__device__ __forceinline__ double2* slot_at(const InitEv& d, size_t o) {
+    return o < d.end0 ? d.work[0] + o : o < d.end1 ? d.work[1] + (o - d.end0) : d.work[2] + (o - d.end1);
+}
+// the sheet that slot j of a nucleus has in a round, -1 for none
+__device__ __forceinline__ int slot_sheet(const InitEv& d, int j, int round) {
+    const int g = j / d.K, l = round * d.K + j - g * d.K, sheet = g * d.per_group + l;
+    return l < d.per_group && sheet < d.Ns ? sheet : -1;
 }
 enum { IK_TABLES = 0, IK_ROWS, IK_COLS, IK_SHEETS, IK_SITES, IK_LINKS, IK_PRODUCTS, IK_N };
 static_assert(IK_N <= InitEv::KINDS, "block table");
@@ -427,14 +433,14 @@ __device__ __forceinline__ void init_rows(const InitEv& d, int blk, int round, f
     const int nl = (int)(all - line0 < d.lines ? all - line0 : d.lines);
     // nothing to do beyond the last sheet (the other events of a batch may go on)
     const int slot0 = (int)(line0 / (4 * (int64_t)N)), slot1 = (int)((line0 + nl - 1) / (4 * (int64_t)N));
-    if (round * S + slot0 % S >= d.Ns && round * S + slot1 % S >= d.Ns && slot1 - slot0 < 2) return;
+    if (slot1 - slot0 < 2 && slot_sheet(d, slot0 % S, round) < 0 && slot_sheet(d, slot1 % S, round) < 0) return;
     for (int idx = threadIdx.x; idx < nl * N; idx += INIT_T) {
         const int l = idx / N, x = idx - l * N;
         const int64_t line = line0 + l;
         const int row = (int)(line % N), plane = (int)(line / N) & 3, slot = (int)(line / (4 * (int64_t)N));
-        const int nucleus = slot / S, sheet = round * S + slot - nucleus * S;
+        const int nucleus = slot / S, sheet = slot_sheet(d, slot - nucleus * S, round);
         ff2 z = {};
-        if (sheet < d.Ns) {
+        if (sheet >= 0) {
             const U4 w = philox4x32_10(U4{(uint32_t)(row * N + x), (uint32_t)((nucleus * d.Ns + sheet) * 2 + (plane >> 1)),
                                           1u, 0u}, d.k0, d.k1);
             z = normal_pair(d, (plane & 1) ? w.z : w.x, (plane & 1) ? w.w : w.y);
@@ -443,8 +449,8 @@ __device__ __forceinline__ void init_rows(const InitEv& d, int blk, int round, f
     }
     __syncthreads();
     lines_forward(sh, nl, N, d);
-    ff2* out = (ff2*)d.work + (size_t)line0 * N;  // work[slot][plane][row][position]
-    for (int idx = threadIdx.x; idx < nl * N; idx += INIT_T) out[idx] = sh[idx];
+    // [slot][plane][row][position]
+    for (int idx = threadIdx.x; idx < nl * N; idx += INIT_T) *(ff2*)slot_at(d, (size_t)line0 * N + idx) = sh[idx];
 }
 __global__ void __launch_bounds__(INIT_T, 4) init_rows_kernel(const InitEv* evs, int ne, InitEv one, int round) {
     extern __shared__ __align__(16) unsigned char init_smem[];
@@ -462,9 +468,9 @@ __global__ void __launch_bounds__(INIT_T, 4) init_cols_kernel(const InitEv* evs,
     const int N = d.N, S = d.S, ls = N + 1;  // a point of padding: neighbouring columns in other banks
     const int nt = (N + d.cols - 1) / d.cols;
     const int c0 = (blk % nt) * d.cols, sp = blk / nt, slot = sp >> 2;
-    if (round * S + slot % S >= d.Ns) return;
+    if (slot_sheet(d, slot % S, round) < 0) return;
     const int nc = N - c0 < d.cols ? N - c0 : d.cols;
-    ff2* w = (ff2*)d.work + (size_t)sp * N * N + c0;
+    ff2* w = (ff2*)slot_at(d, (size_t)sp * N * N) + c0;
     for (int idx = threadIdx.x; idx < nc * N; idx += INIT_T) {
         const int r = idx / nc, c = idx - r * nc;
         sh[c * ls + r] = w[(size_t)r * N + c];
@@ -558,12 +564,12 @@ __global__ void __launch_bounds__(INIT_T, 2) init_sheets_kernel(const InitEv* ev
     const int r0 = (blk % nrb) * d.rows, g = (blk / nrb) % d.groups, nucleus = blk / (nrb * d.groups);
     const int nr = N - r0 < d.rows ? N - r0 : d.rows, np = nr * N;
     const int first = g * d.per_group;
-    int s0 = round * S, s1 = s0 + S < d.Ns ? s0 + S : d.Ns;
-    if (s0 < first) s0 = first;
-    if (s1 > first + d.per_group) s1 = first + d.per_group;
+    const int s0 = first + round * d.K;
+    int s1 = s0 + d.K < first + d.per_group ? s0 + d.K : first + d.per_group;
+    if (s1 > d.Ns) s1 = d.Ns;
     ff2* V = (ff2*)d.V + (size_t)(nucleus * d.groups + g) * 6 * Vn + (int64_t)r0 * N;
     for (int s = s0; s < s1; s++) {
-        const ff2* w = (const ff2*)d.work + (size_t)(nucleus * S + s - round * S) * 4 * Vn + (int64_t)r0 * N;
+        const ff2* w = (const ff2*)slot_at(d, (size_t)(nucleus * S + g * d.K + s - s0) * 4 * Vn) + (int64_t)r0 * N;
         for (int idx = threadIdx.x; idx < 4 * np; idx += INIT_T) {
             const int p = idx / np;
             sh[idx] = w[(size_t)p * Vn + idx - p * np];
@@ -914,7 +920,7 @@ void launch_mv_init(const InitEv* h, const InitEv* d_ev, int ne, cudaStream_t st
         rows = r > rows ? r : rows;
         cols = c > cols ? c : cols;
         sheets = s > sheets ? s : sheets;
-        const int n = (h[e].Ns + h[e].S - 1) / h[e].S;
+        const int n = (h[e].per_group + h[e].K - 1) / h[e].K;
         rounds = n > rounds ? n : rounds;
         grouped = grouped || h[e].groups > 1;
     }

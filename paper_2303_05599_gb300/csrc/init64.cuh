@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(256) init64_rows_kernel(const InitEv* evs, int
     if (sheet >= d.Ns) return;
     const int nl = N - row0 < d.lines ? N - row0 : d.lines, np = nl * N;
     const int64_t Vn = (int64_t)N * N;
-    double2* w = d.work + ((size_t)slot * INIT64_PLANES + 2 * pair) * Vn + (size_t)row0 * N;
+    double2* w = slot_at(d, (size_t)slot * INIT64_PLANES * Vn) + 2 * pair * Vn + (size_t)row0 * N;
     for (int idx = threadIdx.x; idx < np; idx += blockDim.x) {
         const int l = idx / N, at = l * N + line_place(d, idx - l * N);
         if (FIRST) {
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(256) init64_cols_kernel(const InitEv* evs, int
     const int c0 = (blk % nt) * d.cols, plane = (blk / nt) & 7, slot = blk / (8 * nt);
     if (round * S + slot % S >= d.Ns) return;
     const int nc = N - c0 < d.cols ? N - c0 : d.cols;
-    double2* w = d.work + ((size_t)slot * INIT64_PLANES + plane) * N * N + c0;
+    double2* w = slot_at(d, (size_t)slot * INIT64_PLANES * N * N) + (size_t)plane * N * N + c0;
     for (int idx = threadIdx.x; idx < nc * N; idx += blockDim.x) {
         const int r = idx / nc, c = idx - r * nc;
         sh[c * ls + line_place(d, r)] = w[(size_t)r * N + c];
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(128) init64_exp_kernel(const InitEv* evs, int 
     if (slot >= 2 * d.S || round * d.S + slot % d.S >= d.Ns) return;
     const int64_t s = t - slot * Vn;
     // only this thread reads and writes the site's slot
-    double2* w = d.work + (size_t)slot * INIT64_PLANES * Vn;
+    double2* w = slot_at(d, (size_t)slot * INIT64_PLANES * Vn);
     A8<double> al;
 #pragma unroll
     for (int a = 0; a < 8; a++) al.v[a] = -w[(size_t)a * Vn + s].x;
@@ -235,13 +235,15 @@ __global__ void __launch_bounds__(96) init64_products_kernel(const InitEv* evs, 
     int n = d.Ns - round * d.S;
     if (n > d.S) n = d.S;
     double2* V = d.V + ((size_t)nucleus * 9 + 3 * r) * Vn + s;
-    const double2* w = d.work + (size_t)nucleus * d.S * INIT64_PLANES * Vn;
+    // this round's sheet k
+    const size_t step = (size_t)INIT64_PLANES * Vn;
+    auto sheet = [&](int k) { return slot_at(d, (size_t)(nucleus * d.S + k) * step); };
     double2 v[3];
     int first = 0;
     if (round == 0) {
         // the unit matrix times the first sheet
 #pragma unroll
-        for (int j = 0; j < 3; j++) v[j] = w[(size_t)(3 * r + j) * Vn + s];
+        for (int j = 0; j < 3; j++) v[j] = sheet(0)[(size_t)(3 * r + j) * Vn + s];
         first = 1;
     } else {
         if (n <= 0) return;
@@ -249,13 +251,12 @@ __global__ void __launch_bounds__(96) init64_products_kernel(const InitEv* evs, 
         for (int j = 0; j < 3; j++) v[j] = V[(size_t)j * Vn];
     }
     // the next sheet's exponential on its way while one is multiplied
-    const size_t step = (size_t)INIT64_PLANES * Vn;
     M3<double> next = m_zero<double>();
-    if (first < n) next = load_link(w + first * step, 0, s, Vn);
+    if (first < n) next = load_link(sheet(first), 0, s, Vn);
 #pragma unroll 1
     for (int k = first; k < n; k++) {
         const M3<double> m = next;
-        if (k + 1 < n) next = load_link(w + (k + 1) * step, 0, s, Vn);
+        if (k + 1 < n) next = load_link(sheet(k + 1), 0, s, Vn);
         double2 o[3];
 #pragma unroll
         for (int j = 0; j < 3; j++) {

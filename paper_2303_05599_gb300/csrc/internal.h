@@ -59,21 +59,26 @@ struct InitEv {
     static constexpr int KINDS = 7;
     int N, Ns, prec;
     int pow2, log2N, nrad, rad[12];
-    int S, groups, per_group;  // sheets a round; groups of sheets multiplied apart
+    // groups of sheets multiplied apart, sheets a group, sheets of each group a
+    // round, sheets of a nucleus a round (groups K): their slots
+    int groups, per_group, K, S;
     int lines, cols, rows;     // lines, columns and rows a block of the three launches takes
     int begin[KINDS];
     double sigma, m2, lam2;
     float sigma_h, sigma_l;
     uint32_t k0, k1;
     // FP32 events keep V, tw, work and green as pairs of FP32 values in the place of each double
-    double2 *V, *tw, *work, *U64, *comm;
+    double2 *V, *tw, *work[3], *U64, *comm;
+    size_t end0, end1;  // elements of the slots up to which they lie in work[0], work[1]
     double* green;
     FFTables* normal;   // FP32 events: tables of the normal variates
     void* fields;
     int* bad;                  // links whose matching did not converge
 };
-InitEv init_event(int prec, void* fields, void* scratch, int N, int Ns, double g2mu_a, double m_a, double Lambda_a,
-                  uint64_t seed, int* bad);
+// idle_fields, idle_site: the slice of the fields that is not current and the two
+// site-field buffers, which are free until the first step and hold sheets meanwhile
+InitEv init_event(int prec, void* fields, void* scratch, void* idle_fields, void* idle_site, int N, int Ns,
+                  double g2mu_a, double m_a, double Lambda_a, uint64_t seed, int* bad);
 // lattices whose lines fit the transforms
 bool init_supported(int N);
 // begin[] of every event, in order
