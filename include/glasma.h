@@ -281,9 +281,11 @@ gl_status observables(gl_ctx* ctx, gl_obs* out);
 /* Parts of gl_obs to compute.  GL_OBS_PARTICLES: the per-species sums and
  * Casimir drifts (a pass over the particles; per-particle values in the
  * context's precision, accumulated in FP64).  GL_OBS_FIELDS: Gauss residual,
- * link unitarity and the site-field means (an FP64 pass over the lattice,
- * which on GPUs with slow FP64 costs more than a coupled step: meant for
- * report intervals). */
+ * link unitarity and the site-field means (a pass over the lattice with the
+ * residual and the sums over sites in FP64, the unitarity of an FP32 link and
+ * the squares of one site's fields in exact products of FP32 parts; on GPUs
+ * with slow FP64 it costs more than a coupled step: meant for report
+ * intervals). */
 #define GL_OBS_PARTICLES 1u
 #define GL_OBS_FIELDS 2u
 #define GL_OBS_ALL 3u

@@ -342,8 +342,8 @@ __global__ void __launch_bounds__(OBS_FINAL_WARPS * 32) batch_obs_finish(const B
     }
 }
 
-// launch shapes (FP64 takes the second only, whose tile of 128 sites is TILE64_X x TILE64_Y)
-enum { TILE_32x8 = 0, TILE_32x4 = 1, TILE_32x16 = 2, N_TILES = 3 };
+// launch shapes of the field kernel: 0, 1, 2; FP64 takes 1 only (tiles of TILE64_X x TILE64_Y sites)
+enum { SHAPE_FP64 = 1, N_TILES = 3 };
 static const int PUSH_BLOCKS[3] = {128, 256, 512};
 enum { N_CHUNKS = 3 };
 static const int PUSH_CHUNKS[N_CHUNKS] = {512, 1024, 2048};  // fused launch
@@ -714,7 +714,7 @@ gl_status gl_batch_create(const gl_config* cfgs, const gl_species* species, int3
         }
         o += a256b(w);
     }
-    b->tile = b->prec == GL_FP64 ? TILE_32x4 : 0;
+    b->tile = b->prec == GL_FP64 ? SHAPE_FP64 : 0;
     b->seg_rows = 16;  // replaced by the first descriptor sync
     b->strip_wpb = 8;
     b->plan_tile = -1;
@@ -958,7 +958,7 @@ gl_status gl_batch_autotune(gl_batch* b, int32_t* tile_out, int32_t* push_block_
     float best_f = 1e30f;
     int bt = b->tile;
     for (int tile = 0; tile < N_TILES; tile++) {
-        if (b->prec == GL_FP64 && tile != TILE_32x4) continue;  // FP64 tile must fit shared memory
+        if (b->prec == GL_FP64 && tile != SHAPE_FP64) continue;
         b->tile = tile;
         // FP32: the segment lengths tried beside the cost model's choice (its
         // half and double, and 16 rows); the fastest is kept for the shape
@@ -1043,12 +1043,9 @@ gl_status gl_batch_autotune(gl_batch* b, int32_t* tile_out, int32_t* push_block_
         const int tile0 = b->tile;
         for (int g = 0; g <= 2; g++)
             for (int tile = 0; tile < N_TILES; tile++) {
-                if (b->prec == GL_FP64 && tile != TILE_32x4) continue;
-                // resident push blocks (g > 0) leave no room beside the
-                // 512-thread tiles; the plain two-stream step tries every
-                // tile shape, since the fastest field kernel alone is not
-                // always the fastest beside the push
-                if (g > 0 && b->prec == GL_FP64 && tile == TILE_32x16) continue;
+                // every shape: the fastest field kernel alone is not always
+                // the fastest beside the push
+                if (b->prec == GL_FP64 && tile != SHAPE_FP64) continue;
                 b->tile = tile;
                 float best_g = 1e30f;
                 const bool per_chunk = g == 0;  // separate push blocks, one per chunk
@@ -1079,7 +1076,7 @@ gl_status gl_batch_autotune(gl_batch* b, int32_t* tile_out, int32_t* push_block_
                         }
                     }
                 }
-                float& slot = b->tune_step_ms[g == 0 ? 0 : 1 + N_CHUNKS + 2 * (g - 1) + (tile == TILE_32x4)];
+                float& slot = b->tune_step_ms[g == 0 ? 0 : 1 + N_CHUNKS + 2 * (g - 1) + (tile == 1)];
                 if (slot == 0 || best_g < slot) slot = best_g;
             }
         b->tile = tile0;
@@ -1475,7 +1472,7 @@ gl_status gl_batch_set_launch(gl_batch* b, int32_t tile, int32_t push_block, int
                               int32_t push_grid) {
     if (!b || tile < 0 || tile >= N_TILES || (fused != 0 && fused != 1) || push_grid < 0 || push_grid > 2)
         return GL_ERR_ARG;
-    if (b->prec == GL_FP64 && tile != TILE_32x4) return GL_ERR_ARG;
+    if (b->prec == GL_FP64 && tile != SHAPE_FP64) return GL_ERR_ARG;
     bool ok_b = false, ok_c = false;
     for (int k = 0; k < 3; k++) ok_b = ok_b || PUSH_BLOCKS[k] == push_block;
     for (int k = 0; k < N_CHUNKS; k++) ok_c = ok_c || PUSH_CHUNKS[k] == push_chunk;

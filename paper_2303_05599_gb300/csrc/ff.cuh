@@ -17,7 +17,6 @@ struct ff {
 
 __host__ __device__ constexpr ff ff_of(double d) { return ff{(float)d, (float)(d - (double)(float)d)}; }
 __device__ __forceinline__ double to_double(ff a) { return (double)a.h + (double)a.l; }
-__device__ __forceinline__ double to_double(double a) { return a; }
 __device__ __forceinline__ ff ff_quick(float a, float b) {  // |a| >= |b| or a = 0
     const float s = __fadd_rn(a, b);
     return ff{s, __fsub_rn(b, __fsub_rn(s, a))};

@@ -70,7 +70,7 @@ static_assert(sizeof(FFTables) % 16 == 0, "alignment of the tables behind it");
 // take 15.21 ms in 595 MB, with this 15.33 ms in 343 MB; a single small event,
 // which needs many sheets a round to fill the chip, pays more: FP64 32^2 0.65 ms in
 // 17 MB, here 0.72 ms in 7 MB and within 576 B a site 1.39 ms in 3 MB; FP32 64^2 0.37
-// ms in 32 MB and 0.59 ms in 7 MB.
+// ms in 32 MB and 0.59 ms in 7 MB (0.47 ms in 11 MB, twice the room).
 static constexpr size_t INIT_SMALL_ROOM = (size_t)4 << 20;
 
 struct InitPlan {

@@ -119,8 +119,9 @@ int strip_model_seg(int N, int tile) {
 
 // Launch shape of an event that has not been tuned.  Lattices that leave the
 // SMs with one or two warps a scheduler take the 8-warp shape (203 registers a
-// thread), larger ones the 12-warp shape, which needs three to pay: 256^2 21
-// against 22 us, 1024^2 164 against 158 us.
+// thread), larger ones the 12-warp shape, which needs three to pay: 256^2 19.6
+// against 20.3 us, 300^2 24.7 against 24.5 us, 1024^2 153 against 139 us (trial
+// launches, the best segment length of each shape).
 int strip_default_tile(int N) { return (int64_t)N * N <= (int64_t)sm_count() * 8 * 32 * 4 ? 2 : 1; }
 
 }  // namespace gl
