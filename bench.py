@@ -65,10 +65,10 @@ BATCHED = "batched64"
 # shapes), keyed by (workload, events per GPU, kernel, precision).  Absent:
 # not captured for the current kernels.
 TRAFFIC = {
-    ("batched64", 64, "field_step", 1): 514717696 + 694459904,
-    ("batched64", 64, "wong_push", 1): 376806400 + 28170496,
-    ("n1024_mixed", 1, "field_step", 1): 301978624 + 377472000,
-    ("n1024_mixed", 1, "wong_push", 1): 589935360 + 197241088,
+    ("batched64", 64, "field_step", 1): 514889216 + 693578496,
+    ("batched64", 64, "wong_push", 1): 376802560 + 28008960,
+    ("n1024_mixed", 1, "field_step", 1): 302055168 + 377191936,
+    ("n1024_mixed", 1, "wong_push", 1): 594009600 + 196966144,
 }
 
 
