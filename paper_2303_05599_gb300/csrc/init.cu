@@ -770,7 +770,8 @@ __device__ int solve_link(const M3<double>& UA, const M3<double>& UB, M3<double>
     U = mul(UA, UB);
     M3<double> K = mul_nd(W, U);
     double r = match_residual(K, fw, F);
-    bool contracts = r == r;
+    // a finite residual: quartered by every pass, so at most 522 passes follow
+    bool contracts = r <= 1e300;
     while (contracts && r > 1e-14) {
         A8<double> dx;
         contracts = match_step(K, F, dx.v);
@@ -779,7 +780,7 @@ __device__ int solve_link(const M3<double>& UA, const M3<double>& UB, M3<double>
         rebuild_row2(U);
         K = mul_nd(W, U);
         const double rn = match_residual(K, fw, F);
-        contracts = rn <= 0.25 * r;  // not for a NaN
+        contracts = rn <= 0.25 * r;
         r = rn;
     }
     return contracts ? 0 : solve_link_plain(UA, UB, U);

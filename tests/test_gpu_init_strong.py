@@ -24,3 +24,17 @@ def test_fp32_links_of_a_strong_field(N, Ns, a, g2mu, seed):
     U = ev.download(B.GL_BUF_LINKS)[:, :, :12]
     # the rounding of the stored entries, and 48-bit lines through as many steps
     assert np.abs(U - st.U.reshape(2, w.N * w.N, 18)[:, :, :12]).max() < 2.0 ** -25 + 1e-8
+
+
+@pytest.mark.parametrize("precision", [W.FP64, W.FP32_2ROW])
+@pytest.mark.parametrize("g2mu", [1e6, 1e20, 1e37, 1e160, 1e300])
+def test_charges_beyond_any_range_end(g2mu, precision):
+    """Infinite and undefined residuals end the matching, with an error or with
+    fields that are not finite; the context is usable afterwards."""
+    w = W.Workload("huge", N=8, L_fm=0.4, Ns=2, precision=precision, seed=1, g2mu_GeV=g2mu, species=[])
+    ev = B.Event(w)
+    try:
+        ev.glasma_init()
+    except B.GlasmaError as err:
+        assert err.status == B.GL_ERR_NUMERIC
+    assert ev.download(B.GL_BUF_LINKS).shape == (2, 64, 18)
