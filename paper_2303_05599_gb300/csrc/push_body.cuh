@@ -53,24 +53,26 @@ __device__ __forceinline__ A8<double> rapidity_rotation(const A8<double>& ph, do
 // |s phi| (ad's largest eigenvalue is at most |phi|, the length of SU(3)'s roots
 // being 1).  Two things would move |Q|^2 always to one side, which a charge that
 // turns by nearly the same angle every step adds up.  The truncated series is not
-// orthogonal: K = 1, 2, 3, 4 multiply the part of |Q|^2 of that eigenvalue by 1 +
-// x^2, 1 + x^4/4, 1 - x^4/12, 1 - x^6/72; the limits keep that below 2^-30 as
-// well.  And terms added to Q one by one are lost below half a unit in its last
+// orthogonal: K = 1 .. 5 multiply the part of |Q|^2 of that eigenvalue by 1 + x^2,
+// 1 + x^4/4, 1 - x^4/12, 1 - x^6/72, 1 + x^6/360; the limits keep that below 2^-30
+// as well.  And terms added to Q one by one are lost below half a unit in its last
 // place, the first one not; so by Horner's rule they are summed inside, and Q
 // is rounded once.  (Terms one by one, with limits for the value alone: the mean
 // |Q|^2 of 4 off by 2.1e-5 after 300 turns by 2.3e-4 and by -1.3e-5 by 2.8e-2.)
+// One rotation is off by 1.8e-8 rms at any angle to 0.08, the rounding of the
+// result alone; terms one by one 1.9e-8 .. 3.7e-8, the exponential's route 5.2e-8.
 // A step turns Q by dt / t v_w phi, 1e-4 .. 1e-2 for most particles, and a term
 // takes 80 operations, the exponential and the transport about 320.  The push is
 // bound by memory where the particles are few a cell (30 x 256^2: 0.216 ms with
 // either), and by issue as well on 1024^2 with 4 a cell: 0.212 -> 0.203 ms.
 __device__ __forceinline__ A8<float> rapidity_rotation(const A8<float>& ph, float s, const A8<float>& q) {
     const float x2 = s * s * a_dot(ph, ph);
-    if (!(x2 <= 4e-3f)) return conj_up_t(exp_i_alg<float>(ph, -s), q);
-    const float terms = x2 <= 9e-10f ? 1.f : x2 <= 3.1e-5f ? 2.f : x2 <= 1e-4f ? 3.f : 4.f;
+    if (!(x2 <= 6.6e-3f)) return conj_up_t(exp_i_alg<float>(ph, -s), q);
+    const float terms = x2 <= 9e-10f ? 1.f : x2 <= 3.1e-5f ? 2.f : x2 <= 1e-4f ? 3.f : x2 <= 4e-3f ? 4.f : 5.f;
     A8<float> o = q;
 #pragma unroll 1
     for (float k = terms; k >= 1.f; k -= 1.f) {
-        const float f = k == 1.f ? -s : k == 2.f ? -0.5f * s : k == 3.f ? s * (-1.f / 3) : -0.25f * s;
+        const float f = k == 1.f ? -s : k == 2.f ? -0.5f * s : k == 3.f ? s * (-1.f / 3) : k == 4.f ? -0.25f * s : -0.2f * s;
         const A8<float> t = icomm(ph, o);
 #pragma unroll
         for (int a = 0; a < 8; a++) o.v[a] = fmaf(f, t.v[a], q.v[a]);

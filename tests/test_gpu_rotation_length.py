@@ -13,8 +13,8 @@ torch = pytest.importorskip("torch")
 STEPS = 300
 
 
-# below the limits of one, two, three and four terms, and between them
-@pytest.mark.parametrize("angle", [3.0e-5, 2.3e-4, 5.5e-3, 1.0e-2, 2.8e-2, 6.2e-2])
+# below the limits of one to five terms, and between them
+@pytest.mark.parametrize("angle", [3.0e-5, 2.3e-4, 5.5e-3, 1.0e-2, 2.8e-2, 6.2e-2, 7.9e-2])
 def test_mean_length_is_kept(angle):
     N, n = 32, 8
     w = W.Workload("length", N=N, L_fm=1.5, precision=W.FP32_2ROW, reunit_every=0, sort_every=0,
