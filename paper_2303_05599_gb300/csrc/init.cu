@@ -26,7 +26,7 @@ namespace gl {
 // of rho (the Green function is real and even, so the two parts of a plane
 // stay apart through both transforms), and three launches over all events:
 //   rows      rho of a few lattice rows into shared memory, their forward
-//             transforms, out to `work`
+//             transforms, out to the sheet's slot
 //   columns   a tile of columns in: forward transform, Green function, inverse
 //             transform, out
 //   sheets    rows in: inverse transform, then per site exp(-i alpha) and the

@@ -21,9 +21,10 @@
 // Twiddles come from a table of each sign, and the Jacobian of a Newton step
 // from the entries of K that K T^b is made of (the other products are with 0).
 // Measured: a 32^2 event of 50 sheets 10474 us with seven launches a sheet, a
-// sincospi a butterfly and eight matrix products a Newton step, 829 us so (normal
-// variates 60, transforms 170, exponentials 68, products 89, links 270); with
-// init.cu's transforms and series in FP64 it was 550 us, in other roundings.
+// sincospi a butterfly and eight matrix products a Newton step, 900 us so, in three
+// rounds of 17 sheets; all in one round 829 us (normal variates 60, transforms 170,
+// exponentials 68, products 89, links 270); with init.cu's transforms and series in
+// FP64 it was 550 us, in other roundings.
 #pragma once
 #include "internal.h"
 #include "layout.cuh"
